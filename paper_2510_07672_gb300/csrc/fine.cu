@@ -31,6 +31,7 @@
 // once when it is stored.
 #include "common.cuh"
 #include "fft_reg.cuh"
+#include "fine.cuh"
 #include "tc_ptx.cuh"
 
 namespace cg = cooperative_groups;
@@ -68,34 +69,6 @@ __device__ __forceinline__ void bulk_s2peer(uint32_t dst_cluster, uint32_t src_c
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-
-struct FineArgs {
-    const void* in;
-    void* out;
-    int num_fields;
-    int steps;
-    // Field f = g * per_group + i reads field (map[g] * in_gs + in_off + i) of
-    // `in` and writes field (map[g] * out_gs + out_off + i) of `out` (map NULL:
-    // identity).  Plain batched calls use per_group = num_fields.
-    int per_group;
-    long long in_gs, in_off, out_gs, out_off;
-    const int* map;
-    // Work list (overrides the mapping above and `steps`): field f reads field
-    // work[f].x of `in`, writes field work[f].y of `out`, runs work[f].z steps.
-    const int4* work;
-    int mass;        // 1: hold the (0,0) mode at the entry mean
-    // adjoint = 1 runs the transposed steps: lambda_n = a mu + dt f'(u_n) * (mu -
-    // [mass] mean mu), mu = A^{-1} lambda_{n+1}, with u_n read from
-    // states[n][field] (n = steps-1 .. 0, plain field index).
-    int adjoint;
-    const void* states;
-    // traj != NULL stores the state before the first step and after every
-    // step: traj[s][field] for s = 0..steps (plain field index).
-    void* traj;
-    double a;        // 1 + S dt
-    double dt;
-    double lam_scale;  // dt eps^2 (4 / h^2)
-};
 
 // Smallest value >= len that is congruent to B modulo 16 (B < 16); B = 16
 // (one line per half-warp) takes len + 1.
@@ -554,11 +527,14 @@ static int launch_fine(const FineArgs& args, cudaStream_t stream) {
 // all on the caller's problem and keeps the fastest.
 struct FineVariant {
     const char* name;
-    int (*launch)(const FineArgs&, cudaStream_t);
+    int (*launch)(const FineArgs&, cudaStream_t);  // NULL: the polynomial solve
     bool async;  // asynchronous exchange: no adjoint mode
     int P;       // CTAs per field (the split that fixes the rounding)
 };
 
+// The polynomial solve (fine_stencil.cu) where the step allows it, else the
+// next entry.
+#define ACPR_POLY {"stencil", nullptr, false, 0}
 #define ACPR_FV(T, N, P, A, B, M) {"P" #P "_A" #A "_B" #B "_occ" #M, &launch_fine<T, N, P, A, B, M>, false, P}
 #define ACPR_FVA(T, N, P, A, B, M) \
     {"P" #P "_A" #A "_B" #B "_occ" #M "_async", &launch_fine<T, N, P, A, B, M, true>, true, P}
@@ -569,10 +545,10 @@ template <typename T>
 static const FineVariant* fine_variants(int n, int* count) {
     static const FineVariant v8[] = {ACPR_FV(T, 8, 1, 4, 2, 1)};
     static const FineVariant v16[] = {ACPR_FV(T, 16, 1, 4, 4, 1)};
-    static const FineVariant v32[] = {ACPR_FV(T, 32, 1, 8, 4, 1)};
-    static const FineVariant v64[] = {ACPR_FV(T, 64, 1, 8, 8, 2), ACPR_FV(T, 64, 2, 8, 8, 3)};
+    static const FineVariant v32[] = {ACPR_POLY, ACPR_FV(T, 32, 1, 8, 4, 1)};
+    static const FineVariant v64[] = {ACPR_POLY, ACPR_FV(T, 64, 1, 8, 8, 2), ACPR_FV(T, 64, 2, 8, 8, 3)};
     if constexpr (sizeof(T) == 4) {
-        static const FineVariant v128[] = {ACPR_FV(T, 128, 2, 16, 8, 2), ACPR_FV(T, 128, 4, 16, 8, 3),
+        static const FineVariant v128[] = {ACPR_POLY, ACPR_FV(T, 128, 2, 16, 8, 2), ACPR_FV(T, 128, 4, 16, 8, 3),
                                            ACPR_FV(T, 128, 1, 16, 8, 1), ACPR_FVA(T, 128, 4, 16, 8, 3),
                                            ACPR_FVA(T, 128, 2, 16, 8, 2)};
         // entry 0 (clusters of 8, asynchronous exchange, no separate exchange
@@ -582,37 +558,38 @@ static const FineVariant* fine_variants(int n, int* count) {
         // shape change alters the rounding, and F must stay one function within
         // a solve and between a Parareal solve and its sequential reference
         // (exactness at k = s): the default does not depend on the batch size.
-        static const FineVariant v256[] = {ACPR_FVN(T, 256, 8, 16, 16, 3), ACPR_FVA(T, 256, 8, 16, 16, 2),
+        static const FineVariant v256[] = {ACPR_POLY, ACPR_FVN(T, 256, 8, 16, 16, 3), ACPR_FVA(T, 256, 8, 16, 16, 2),
                                            ACPR_FVA(T, 256, 16, 16, 16, 3), ACPR_FVA(T, 256, 4, 16, 16, 1),
                                            ACPR_FV(T, 256, 8, 16, 16, 2), ACPR_FV(T, 256, 4, 16, 16, 1),
                                            ACPR_FV(T, 256, 16, 16, 16, 3), ACPR_FV(T, 256, 8, 16, 16, 1),
                                            ACPR_FVN(T, 256, 8, 16, 16, 2)};
-        static const FineVariant v512[] = {ACPR_FV(T, 512, 16, 32, 16, 1), ACPR_FVA(T, 512, 16, 32, 16, 1)};
+        static const FineVariant v512[] = {ACPR_POLY, ACPR_FV(T, 512, 16, 32, 16, 1), ACPR_FVA(T, 512, 16, 32, 16, 1)};
         switch (n) {
-            case 128: *count = 5; return v128;
-            case 256: *count = 9; return v256;
-            case 512: *count = 2; return v512;
+            case 128: *count = 6; return v128;
+            case 256: *count = 10; return v256;
+            case 512: *count = 3; return v512;
             default: break;
         }
     } else {
-        static const FineVariant v128[] = {ACPR_FV(T, 128, 4, 16, 8, 1), ACPR_FV(T, 128, 2, 16, 8, 1),
+        static const FineVariant v128[] = {ACPR_POLY, ACPR_FV(T, 128, 4, 16, 8, 1), ACPR_FV(T, 128, 2, 16, 8, 1),
                                            ACPR_FVA(T, 128, 4, 16, 8, 1)};
-        static const FineVariant v256[] = {ACPR_FV(T, 256, 8, 16, 16, 1), ACPR_FV(T, 256, 16, 16, 16, 2),
+        static const FineVariant v256[] = {ACPR_POLY, ACPR_FV(T, 256, 8, 16, 16, 1), ACPR_FV(T, 256, 16, 16, 16, 2),
                                            ACPR_FVA(T, 256, 8, 16, 16, 1)};
         switch (n) {
-            case 128: *count = 3; return v128;
-            case 256: *count = 3; return v256;
+            case 128: *count = 4; return v128;
+            case 256: *count = 4; return v256;
             default: break;
         }
     }
     switch (n) {
         case 8: *count = 1; return v8;
         case 16: *count = 1; return v16;
-        case 32: *count = 1; return v32;
-        case 64: *count = 2; return v64;
+        case 32: *count = 2; return v32;
+        case 64: *count = 3; return v64;
         default: *count = 0; return nullptr;
     }
 }
+#undef ACPR_POLY
 #undef ACPR_FV
 #undef ACPR_FVA
 #undef ACPR_FVN
@@ -637,15 +614,21 @@ static int dispatch_fine(int n, const FineArgs& args, cudaStream_t stream) {
     const int pr = sizeof(T) == 8 ? AC_F64 : AC_F32;
     int idx = g_variant[pr][ilog2(n)];
     if (idx < 0 || idx >= count) idx = 0;
+    if (!v[idx].launch) {
+        bool taken = false;
+        const int rc = launch_stencil<T>(n, args, stream, &taken);
+        if (rc || taken) return rc;
+        ++idx;  // too stiff for the polynomial: the Fourier solve
+    }
     // the adjoint's mean broadcast is ordered by cluster barriers: take the
     // barrier-exchange shape of the same split (same rounding), else the first
     if (args.adjoint && v[idx].async) {
         const int want = v[idx].P;
         int alt = -1;
         for (int i = 0; i < count && alt < 0; ++i)
-            if (!v[i].async && v[i].P == want) alt = i;
+            if (v[i].launch && !v[i].async && v[i].P == want) alt = i;
         for (int i = 0; i < count && alt < 0; ++i)
-            if (!v[i].async) alt = i;
+            if (v[i].launch && !v[i].async) alt = i;
         idx = alt < 0 ? count : alt;
         if (idx == count) {
             set_error("ac_fine: no barrier-exchange shape for the adjoint at n=%d", n);

@@ -1,0 +1,815 @@
+// fine_stencil.cu -- the fine propagator by a polynomial solve: the same
+// stabilised step as fine.cu (Sec. 3.1),
+//   (a - dt eps^2 Lap_h) u' = r,  r = u + u (kappa - dt u^2),  a = 1 + S dt,
+//   kappa = S dt + dt,
+// with A^{-1} applied as a polynomial of the 5-point stencil instead of a pair
+// of Fourier transforms.  With lambda = dt eps^2 4 / h^2 the spectrum of
+// -dt eps^2 Lap_h is [0, 2 lambda]; an interface resolved by a few cells and a
+// step that resolves the dynamics make lambda about 25 dt (1e-3 at the paper's
+// steps), A is within 1e-3 of a multiple of the identity, and the Chebyshev
+// series of 1 / (a + s) on the spectrum converges by a factor rho = lambda / 4
+// per degree: degree 2 is exact to 1e-9 and degree 4 to 4e-16.  A cell then
+// costs 4 M + 4 operations (12 at degree 2) and M rows of neighbours where the
+// Fourier solve costs about 75 instructions and two transposes over the
+// cluster.  Steps too stiff for a built degree take the Fourier kernel.
+//
+// p(Lap) = sum_j b_j T^j (T: sum of the four neighbours), evaluated as
+//   w_M = r,  w_j = r + (b_{j+1} / b_j) T w_{j+1},  u' = r + (b_0 - 1) r + b_1 T w_1,
+// so every rounded coefficient multiplies a term of size lambda: a rounding of
+// b_0 itself would be a gain error repeated in every step.  A cell's value is
+// the same sequence of operations whatever the split into warps, CTAs and
+// clusters, so the split follows the batch size and F stays one function.
+//
+// Mass-conserving model: beta shifts every cell alike, so u' = p(Lap) r + shift
+// with the shift that puts the mean at the field's entry mean: mean(p(Lap) r) =
+// mean(r) / a.  The sum of r over the field is formed in integers (fixed point,
+// 2^-24 for float32 and two words for float64), which makes it independent of
+// the order and of the split.
+//
+// Bound: FP32 (float64: FP64) issue.  Measured, Fourier kernel -> this one:
+//   512 fields of 256^2, mass, 100 steps        11.40 -> 2.22 ms
+//   21 fields of 512^2, 50 to 90 steps           3.01 -> 0.37 ms
+//   float64 256^2, 300 steps, their recomputation and adjoint  138 -> 26 ms
+//   one step of one 128^2 field (call included)  16.4 -> 11.8 us
+// Error against 64 bits after 100 float32 steps at 256^2: 1.5e-5 -> 2e-6.
+#include <algorithm>
+#include <cmath>
+
+#include "fine.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace acpr {
+
+SolvePoly solve_poly(double a, double lam_scale, int dims, int precision, int min_degree, int max_degree) {
+    SolvePoly out;
+    // 1 / (C - x) on [-h, h], x = (lambda / 4) T, in Chebyshev polynomials of
+    // z = x / h = T / (2 dims): c_0 = 1 / R, c_k = 2 rho^k / R
+    const double h = 0.5 * dims * lam_scale, C = a + h;
+    const double R = std::sqrt((C - h) * (C + h)), rho = h / (C + R);
+    // The error is largest for the checkerboard mode, 4 rho^(M+1): at most a
+    // quarter of a rounding in float32, two in float64.  Against a long double
+    // solve, 300 steps at 128^2 (lambda = 1.25e-3): degree 4 6e-14, degree 5
+    // 2.6e-14, a float64 Fourier solve 5e-14; at 64^2 (1e-3), 400 steps:
+    // degree 4 2.8e-14, Fourier 6e-14.
+    const double tol = precision == AC_F64 ? 0x1p-52 : 0x1p-26;
+    int M = std::max(1, min_degree);
+    while (M <= max_degree && 4.0 * std::pow(rho, M + 1) > tol) ++M;
+    if (M > max_degree || M > kMaxDegree || !(a > 0.0) || !std::isfinite(rho)) return out;
+    double c[kMaxDegree + 1];
+    double sum = 0.0;
+    for (int k = 0; k <= M; ++k) {
+        c[k] = (k ? 2.0 : 1.0) * std::pow(rho, k) / R;
+        sum += c[k];
+    }
+    c[M] += 1.0 / a - sum;  // exact for the mean mode (z = 1)
+    // Chebyshev to monomials
+    double t0[kMaxDegree + 1] = {1.0}, t1[kMaxDegree + 1] = {0.0, 1.0}, z[kMaxDegree + 1] = {};
+    for (int k = 0; k <= M; ++k) {
+        for (int j = 0; j <= k; ++j) z[j] += c[k] * t0[j];
+        double t2[kMaxDegree + 1] = {};
+        for (int j = 0; j <= M; ++j) t2[j] = (j ? 2.0 * t1[j - 1] : 0.0) - t0[j];
+        std::copy(t1, t1 + kMaxDegree + 1, t0);
+        std::copy(t2, t2 + kMaxDegree + 1, t1);
+    }
+    out.degree = M;
+    for (int j = 0; j <= M; ++j) out.b[j] = z[j] / std::pow(2.0 * dims, j);
+    return out;
+}
+
+namespace {
+
+// Coefficients of one call in the fields' precision.
+template <typename T, int M>
+struct Coef {
+    T kappa, mdt;   // r = u + u (kappa + mdt u^2)
+    T be0, b1;      // u' = r + be0 r + b1 T w_1
+    T g[M];         // g[k], k = 0 .. M - 2: stage k, w = r + g[k] T (input)
+    T a, dt;        // adjoint: lambda' = a mu + dt f'(u) (mu - mean)
+};
+
+template <typename T, int M>
+Coef<T, M> make_coef(const FineArgs& args, const SolvePoly& p) {
+    Coef<T, M> c{};
+    c.kappa = T((args.a - 1.0) + args.dt);
+    c.mdt = T(-args.dt);
+    c.be0 = T(p.b[0] - 1.0);
+    c.b1 = T(p.b[1]);
+    // stage k applies the ratio of the coefficients M - k and M - k - 1
+    for (int k = 0; k + 1 < M; ++k) {
+        const double hi = p.b[M - k], lo = p.b[M - k - 1];
+        c.g[k] = std::fabs(lo) > 1e-200 ? T(hi / lo) : T(0);
+    }
+    c.a = T(args.a);
+    c.dt = T(args.dt);
+    return c;
+}
+
+template <int P>
+__device__ __forceinline__ void cl_arrive() {
+    if constexpr (P > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+template <int P>
+__device__ __forceinline__ void cl_wait() {
+    if constexpr (P > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    else __syncthreads();
+}
+
+template <int P, typename V>
+__device__ __forceinline__ V* peer(V* local, int rank) {
+    if constexpr (P > 1) return cg::this_cluster().map_shared_rank(local, rank);
+    else return local;
+}
+
+// Field and step count of this block's work item.
+struct Item {
+    long long fin, fout;
+    int steps;
+};
+__device__ __forceinline__ Item item_of(const FineArgs& args, int field) {
+    Item it;
+    it.steps = args.steps;
+    if (args.work) {
+        const int4 w = args.work[field];
+        it.fin = w.x;
+        it.fout = w.y;
+        it.steps = w.z;
+    } else {
+        const int g = field / args.per_group, i = field % args.per_group;
+        const long long pg = args.map ? args.map[g] : g;
+        it.fin = pg * args.in_gs + args.in_off + i;
+        it.fout = pg * args.out_gs + args.out_off + i;
+    }
+    return it;
+}
+
+// ------------------------------------------------ float32, in registers --
+// A warp owns H full rows; lane l holds the W = N / 32 adjacent columns l W ..
+// of each, so the horizontal neighbours at the run's ends come by one shuffle
+// each way (the ring of lanes is the periodic row).  The rows of the warps
+// above and below come through shared memory (`halo`), those of the
+// neighbouring CTAs of the cluster through their shared memory: M rows each
+// way per step, double-buffered, one cluster barrier per step.
+
+template <int W>
+__device__ __forceinline__ void row_store(float* dst, const float (&x)[W], int lane) {
+    // chunks of VW floats, chunk-major: lanes store consecutive vectors
+    constexpr int VW = W >= 4 ? 4 : W;
+#pragma unroll
+    for (int v = 0; v < W / VW; ++v) {
+        float* p = dst + v * 32 * VW + lane * VW;
+        if constexpr (VW == 4) *reinterpret_cast<float4*>(p) = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+        else if constexpr (VW == 2) *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+        else *p = x[0];
+    }
+}
+template <int W>
+__device__ __forceinline__ void row_load(const float* src, float (&x)[W], int lane) {
+    constexpr int VW = W >= 4 ? 4 : W;
+#pragma unroll
+    for (int v = 0; v < W / VW; ++v) {
+        const float* p = src + v * 32 * VW + lane * VW;
+        if constexpr (VW == 4) {
+            const float4 q = *reinterpret_cast<const float4*>(p);
+            x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w;
+        } else if constexpr (VW == 2) {
+            const float2 q = *reinterpret_cast<const float2*>(p);
+            x[0] = q.x; x[1] = q.y;
+        } else {
+            x[0] = *p;
+        }
+    }
+}
+// The lane's W columns of a row in global memory (row base, 16-byte aligned).
+template <int W>
+__device__ __forceinline__ void grow_load(const float* row, float (&x)[W], int lane) {
+    const float* p = row + lane * W;
+    if constexpr (W >= 4) {
+#pragma unroll
+        for (int v = 0; v < W / 4; ++v) {
+            const float4 q = reinterpret_cast<const float4*>(p)[v];
+            x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int c = 0; c < W; ++c) x[c] = p[c];
+    }
+}
+template <int W>
+__device__ __forceinline__ void grow_store(float* row, const float (&x)[W], int lane) {
+    float* p = row + lane * W;
+    if constexpr (W >= 4) {
+#pragma unroll
+        for (int v = 0; v < W / 4; ++v)
+            reinterpret_cast<float4*>(p)[v] = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+    } else {
+#pragma unroll
+        for (int c = 0; c < W; ++c) p[c] = x[c];
+    }
+}
+
+// Left plus right neighbour of every column of a row.
+template <int W>
+__device__ __forceinline__ void hsum(const float (&x)[W], float (&h)[W], int lane) {
+    const float l = __shfl_sync(0xffffffffu, x[W - 1], (lane + 31) & 31);
+    const float r = __shfl_sync(0xffffffffu, x[0], (lane + 1) & 31);
+#pragma unroll
+    for (int c = 0; c < W; ++c) h[c] = (c ? x[c - 1] : l) + (c + 1 < W ? x[c + 1] : r);
+}
+
+// r <- p(Lap) r for the warp's H rows; halo(y, x) gives row y of r outside
+// them (-M <= y < 0 or H <= y < H + M).  Rows stream through the M stages; a
+// stage keeps its last row (p) and the three known neighbours of that row's
+// cells (s), so T = ((left + right) + above) + below for every cell.
+// SHIFT: plus `shift`, added to the small term: r + be0 r lies on the coarse
+// grid of its binade, where a shift below half a unit would be rounded away in
+// all of its cells alike.
+template <int W, int H, int M, bool SHIFT, class Halo>
+__device__ __forceinline__ void apply_poly(float (&r)[H][W], const Coef<float, M>& cf, int lane, float shift,
+                                           Halo halo) {
+    float s[M][W], p[M][W];
+#pragma unroll
+    for (int y = -M; y < H + M; ++y) {
+        float x[W];
+        if (y >= 0 && y < H) {
+#pragma unroll
+            for (int c = 0; c < W; ++c) x[c] = r[y][c];
+        } else {
+            halo(y, x);
+        }
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+            const int yk = y - k, first = k - M;  // x is row yk of the stage's input, whose first row is `first`
+            if (yk < first) break;
+            float nx[W];
+            const bool emit = yk >= first + 2;
+            if (emit) {
+                if (k < M - 1) {
+                    float rr[W];
+                    const int yr = yk - 1;
+                    if (k == 0) {
+#pragma unroll
+                        for (int c = 0; c < W; ++c) rr[c] = p[0][c];
+                    } else if (yr >= 0 && yr < H) {
+#pragma unroll
+                        for (int c = 0; c < W; ++c) rr[c] = r[yr][c];
+                    } else {
+                        halo(yr, rr);
+                    }
+#pragma unroll
+                    for (int c = 0; c < W; ++c) nx[c] = fmaf(cf.g[k], s[k][c] + x[c], rr[c]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < W; ++c) {
+                        const float t0 = fmaf(cf.be0, r[yk - 1][c], r[yk - 1][c]);
+                        r[yk - 1][c] = SHIFT ? t0 + fmaf(cf.b1, s[k][c] + x[c], shift) : fmaf(cf.b1, s[k][c] + x[c], t0);
+                    }
+                }
+            }
+            if (yk > first && yk < H + M - k - 1) {
+                float h[W];
+                hsum<W>(x, h, lane);
+#pragma unroll
+                for (int c = 0; c < W; ++c) s[k][c] = h[c] + p[k][c];
+            }
+#pragma unroll
+            for (int c = 0; c < W; ++c) p[k][c] = x[c];
+            if (!emit || k == M - 1) break;
+#pragma unroll
+            for (int c = 0; c < W; ++c) x[c] = nx[c];
+        }
+    }
+}
+
+constexpr float kFix = 16777216.f;  // 2^24: fixed point of the sums of r
+constexpr long long kBadSum = (long long)(1ULL << 63);
+
+// Sum over the warp's lanes of a 62-bit integer, on every lane.
+__device__ __forceinline__ long long warp_sum_s64(long long v) {
+    const int a0 = int(v & 0xfffff), a1 = int((v >> 20) & 0xfffff), a2 = int(v >> 40);
+    return (long long)__reduce_add_sync(0xffffffffu, a0) + ((long long)__reduce_add_sync(0xffffffffu, a1) << 20) +
+           ((long long)__reduce_add_sync(0xffffffffu, a2) << 40);
+}
+
+// Sum of the two rows' cells of a lane (the same order under every split).
+template <int W>
+__device__ __forceinline__ float pair_sum(const float (&x)[W], const float (&y)[W]) {
+    float t[W];
+#pragma unroll
+    for (int c = 0; c < W; ++c) t[c] = x[c] + y[c];
+#pragma unroll
+    for (int o = W / 2; o > 0; o /= 2)
+#pragma unroll
+        for (int c = 0; c < o; ++c) t[c] += t[c + o];
+    return t[0];
+}
+
+template <int N, int H, int NW, int P, int M>
+struct RegShape {
+    static constexpr int W = N / 32, R = NW * H;
+    static constexpr size_t HALO = size_t(2) * 2 * NW * M * N;  // floats
+    static constexpr size_t SMEM = HALO * sizeof(float) + size_t(2) * P * NW * sizeof(long long);
+    static_assert(R * P == N && H % 2 == 0 && H >= M && N % 32 == 0, "split");
+};
+
+template <int N, int H, int NW, int P, int M, int MINB, bool MASS, bool ADJ>
+__global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid_constant__ FineArgs args,
+                                                                    const __grid_constant__ Coef<float, M> cf) {
+    using Sh = RegShape<N, H, NW, P, M>;
+    constexpr int W = Sh::W, R = Sh::R;
+    constexpr long long NN = (long long)N * N;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* halo = reinterpret_cast<float*>(smem_raw);  // [buffer][0: above, 1: below][warp][M][N]
+    long long* tot = reinterpret_cast<long long*>(halo + Sh::HALO);  // [buffer][P NW] sums of the warps
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int rank = 0;
+    if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
+    const int field = blockIdx.x / P;
+    const Item it = item_of(args, field);
+    const int row0 = rank * R + warp * H;
+    const float* in = static_cast<const float*>(args.in) + it.fin * NN + (long long)row0 * N;
+    float* out = static_cast<float*>(args.out) + it.fout * NN + (long long)row0 * N;
+    float* traj = args.traj ? static_cast<float*>(args.traj) + field * NN + (long long)row0 * N : nullptr;
+    const long long traj_step = (long long)args.num_fields * NN;
+
+    float u[H][W];
+#pragma unroll
+    for (int y = 0; y < H; ++y) grow_load<W>(in + y * N, u[y], lane);
+    if (traj) {
+#pragma unroll
+        for (int y = 0; y < H; ++y) grow_store<W>(traj + y * N, u[y], lane);
+    }
+
+    // where this warp's first and last M rows go: `below` of the warp above,
+    // `above` of the warp below (in the neighbouring CTAs at the slab's ends)
+    constexpr int BUF = 2 * NW * M * N;
+    float* up = halo + (NW + (warp > 0 ? warp - 1 : NW - 1)) * M * N;
+    float* down = halo + (warp < NW - 1 ? warp + 1 : 0) * M * N;
+    if (P > 1 && warp == 0) up = peer<P>(up, (rank + P - 1) % P);
+    if (P > 1 && warp == NW - 1) down = peer<P>(down, (rank + 1) % P);
+    const float* above = halo + warp * M * N;
+    const float* below = halo + (NW + warp) * M * N;
+
+    long long target = 0;   // sum of r that keeps the entry mean, in 2^-24
+    double msum = 0.0;      // adjoint: this warp's part of the sum of lambda
+    auto publish_total = [&](long long v, int buf) {
+        for (int q = lane; q < P; q += 32) peer<P>(tot, q)[buf * P * NW + rank * NW + warp] = v;
+    };
+    cl_arrive<P>();
+    if constexpr (MASS && !ADJ) {
+        // entry sum, cell by cell
+        long long acc = 0;
+        bool bad = false;
+#pragma unroll
+        for (int y = 0; y < H; ++y)
+#pragma unroll
+            for (int c = 0; c < W; ++c) {
+                acc += __float2ll_rn(u[y][c] * kFix);
+                bad |= !(fabsf(u[y][c]) < 0x1p19f);
+            }
+        acc = warp_sum_s64(acc);
+        if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
+        cl_wait<P>();
+        publish_total(acc, 1);
+        cl_arrive<P>();
+        cl_wait<P>();
+        long long t = 0;
+        bool b2 = false;
+        for (int i = lane; i < P * NW; i += 32) {
+            t += tot[P * NW + i];
+            b2 |= tot[P * NW + i] == kBadSum;
+        }
+        t = warp_sum_s64(t);
+        b2 = __any_sync(0xffffffffu, b2);
+        target = b2 ? kBadSum : __double2ll_rn(args.a * double(t));
+    } else {
+        cl_wait<P>();
+    }
+    const float inv_fix = float(1.0 / (args.a * double(NN) * double(kFix)));
+
+    for (int step = 0; step < it.steps; ++step) {
+        const int buf = step & 1;
+        if constexpr (!ADJ) {
+#pragma unroll
+            for (int y = 0; y < H; ++y)
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    const float v = u[y][c];
+                    u[y][c] = fmaf(v, fmaf(cf.mdt, v * v, cf.kappa), v);
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            row_store<W>(up + buf * BUF + m * N, u[m], lane);
+            row_store<W>(down + buf * BUF + m * N, u[H - M + m], lane);
+        }
+        if constexpr (MASS) {
+            if constexpr (!ADJ) {
+                long long acc = 0;
+                bool bad = false;
+#pragma unroll
+                for (int y = 0; y < H; y += 2) {
+                    const float t = pair_sum<W>(u[y], u[y + 1]);
+                    acc += __float2ll_rn(t * kFix);
+                    bad |= !(fabsf(t) < 0x1p24f);  // 2^13 such sums stay below 2^62
+                }
+                acc = warp_sum_s64(acc);
+                if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
+                publish_total(acc, buf);
+            } else {
+                msum = 0.0;
+#pragma unroll
+                for (int y = 0; y < H; y += 2) msum += double(pair_sum<W>(u[y], u[y + 1]));
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
+                publish_total(__double_as_longlong(msum), buf);
+            }
+        }
+        cl_arrive<P>();
+        cl_wait<P>();
+        float shift = 0.f;
+        if constexpr (MASS) {
+            const long long* tb = tot + buf * P * NW;
+            if constexpr (!ADJ) {
+                long long t = 0;
+                bool bad = target == kBadSum;
+                for (int i = lane; i < P * NW; i += 32) {
+                    t += tb[i];
+                    bad |= tb[i] == kBadSum;
+                }
+                t = warp_sum_s64(t);
+                shift = float(target - t) * inv_fix;
+                if (__any_sync(0xffffffffu, bad)) shift = __int_as_float(0x7fffffff);
+            } else {
+                double t = 0.0;
+                for (int i = lane; i < P * NW; i += 32) t += __longlong_as_double(tb[i]);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                shift = float(t / (double(NN) * args.a));  // mean of mu
+            }
+        }
+        apply_poly<W, H, M, MASS && !ADJ>(u, cf, lane, shift, [&](int y, float(&x)[W]) {
+            row_load<W>((y < 0 ? above + (y + M) * N : below + (y - H) * N) + buf * BUF, x, lane);
+        });
+        if constexpr (ADJ) {
+            const float* un = static_cast<const float*>(args.states) +
+                              ((long long)(it.steps - 1 - step) * args.num_fields + field) * NN + (long long)row0 * N;
+#pragma unroll
+            for (int y = 0; y < H; ++y) {
+                float v[W];
+                grow_load<W>(un + y * N, v, lane);
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    const float f = 1.f - 3.f * v[c] * v[c];
+                    u[y][c] = fmaf(cf.a, u[y][c], cf.dt * f * (u[y][c] - shift));
+                }
+            }
+        }
+        if (traj) {
+            float* ts = traj + (step + 1) * traj_step;
+#pragma unroll
+            for (int y = 0; y < H; ++y) grow_store<W>(ts + y * N, u[y], lane);
+        }
+    }
+#pragma unroll
+    for (int y = 0; y < H; ++y) grow_store<W>(out + y * N, u[y], lane);
+}
+
+template <int N, int H, int NW, int P, int M, int MINB, bool MASS, bool ADJ>
+int launch_reg_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
+    using Sh = RegShape<N, H, NW, P, M>;
+    auto kern = stencil_reg_kernel<N, H, NW, P, M, MINB, MASS, ADJ>;
+    static bool configured = false;
+    if (!configured) {
+        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM)));
+        if (P > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        configured = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(args.num_fields) * P, 1, 1);
+    cfg.blockDim = dim3(NW * 32, 1, 1);
+    cfg.dynamicSmemBytes = Sh::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = P;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = P > 1 ? 1 : 0;
+    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<float, M>(args, poly)));
+    count_launch();
+    return AC_OK;
+}
+
+template <int N, int H, int NW, int P, int M, int MINB>
+int launch_reg(const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
+    if (args.adjoint)
+        return args.mass ? launch_reg_t<N, H, NW, P, M, MINB, true, true>(args, poly, st)
+                         : launch_reg_t<N, H, NW, P, M, MINB, false, true>(args, poly, st);
+    return args.mass ? launch_reg_t<N, H, NW, P, M, MINB, true, false>(args, poly, st)
+                     : launch_reg_t<N, H, NW, P, M, MINB, false, false>(args, poly, st);
+}
+
+// The split by size, degree and batch.
+template <int M>
+int dispatch_reg(int n, const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
+    const int F = args.num_fields;
+    switch (n) {
+        case 32: return launch_reg<32, 4, 8, 1, M, 1>(args, poly, st);
+        case 64:
+            if (F <= 38) return launch_reg<64, 4, 4, 4, M, 1>(args, poly, st);
+            return launch_reg<64, 8, 8, 1, M, 1>(args, poly, st);
+        case 128:
+            if (F <= 19) return launch_reg<128, 4, 4, 8, M, 1>(args, poly, st);
+            return launch_reg<128, 8, 8, 2, M, 2>(args, poly, st);
+        case 256:
+            if constexpr (M == 2)
+                if (F > 19) return launch_reg<256, 8, 8, 4, M, 2>(args, poly, st);
+            return launch_reg<256, 4, 8, 8, M, 2>(args, poly, st);
+        case 512:
+            if constexpr (M <= 3) return launch_reg<512, 4, 8, 16, M, 1>(args, poly, st);
+            return AC_ERR_UNSUPPORTED;
+        default: return AC_ERR_UNSUPPORTED;
+    }
+}
+
+// -------------------------------------------------- any type, shared memory --
+// The same solve with r and the stages in shared memory: cluster of P CTAs,
+// CTA q holds rows [q R, q R + R) plus M halo rows each way; a stage is
+// computed on the rows the later stages need (the halo shrinks by a row per
+// stage), a CTA barrier between stages, one cluster barrier per step.  Used in
+// float64, whose arithmetic (two lanes per SM and cycle) is the bound.
+constexpr int kShThreads = 256;
+
+template <typename T, int N, int P, int M>
+struct ShShape {
+    static constexpr int R = N / P, RH = R + 2 * M, RW = R + 2 * (M - 1);
+    static constexpr int K = R * N / kShThreads;  // cells per thread
+    static constexpr size_t SMEM =
+        sizeof(T) * N * (size_t(2) * RH + size_t(M > 2 ? 2 : 1) * RW) + size_t(2) * 2 * P * 8 * sizeof(long long);
+    static_assert(R >= M && R * N % kShThreads == 0, "split");
+};
+
+// Exact sum pieces of a float64: x = hi 2^-24 + lo 2^-68 to 2^-69, |x| < 2^26
+// (2^16 cells below 2^20 keep both words below 2^61).
+__device__ __forceinline__ void fix64(double x, long long& hi, long long& lo) {
+    constexpr double m1 = 0x1.8p28, m2 = 0x1.8p-16;
+    const double t = x + m1;
+    const double rem = x - (t - m1);
+    const double t2 = rem + m2;
+    hi += __double_as_longlong(t) - __double_as_longlong(m1);
+    lo += __double_as_longlong(t2) - __double_as_longlong(m2);
+}
+
+template <typename T, int N, int P, int M, bool MASS, bool ADJ>
+__global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_constant__ FineArgs args,
+                                                                  const __grid_constant__ Coef<T, M> cf) {
+    using Sh = ShShape<T, N, P, M>;
+    constexpr int R = Sh::R, RH = Sh::RH, RW = Sh::RW, K = Sh::K;
+    constexpr long long NN = (long long)N * N;
+    constexpr int WARPS = kShThreads / 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* rbuf = reinterpret_cast<T*>(smem_raw);       // [2][RH][N], row 0 is row -M
+    T* wbuf = rbuf + 2 * RH * N;                     // [1 or 2][RW][N], row 0 is row -(M-1)
+    long long* tot = reinterpret_cast<long long*>(wbuf + (M > 2 ? 2 : 1) * RW * N);  // [buffer][P WARPS][hi, lo]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int rank = 0;
+    if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
+    const int field = blockIdx.x / P;
+    const Item it = item_of(args, field);
+    const T* in = static_cast<const T*>(args.in) + it.fin * NN + (long long)rank * R * N;
+    T* out = static_cast<T*>(args.out) + it.fout * NN + (long long)rank * R * N;
+    T* traj = args.traj ? static_cast<T*>(args.traj) + field * NN + (long long)rank * R * N : nullptr;
+    const long long traj_step = (long long)args.num_fields * NN;
+    T* rup = peer<P>(rbuf, (rank + P - 1) % P);
+    T* rdown = peer<P>(rbuf, (rank + 1) % P);
+
+    T u[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        u[i] = in[tid + i * kShThreads];
+        if (traj) traj[tid + i * kShThreads] = u[i];
+    }
+    auto publish = [&](long long hi, long long lo, bool bad, int buf) {
+        // integer sums: any order gives the same bits
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            hi += __shfl_xor_sync(0xffffffffu, hi, o);
+            lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        }
+        if (__any_sync(0xffffffffu, bad)) lo = kBadSum;
+        for (int q = lane; q < P; q += 32) {
+            long long* p = peer<P>(tot, q) + ((buf * P + rank) * WARPS + warp) * 2;
+            p[0] = hi;
+            p[1] = lo;
+        }
+    };
+    // the field's sum; not a number when a cell was out of range
+    auto collect = [&](int buf) -> double {
+        long long hi = 0, lo = 0;
+        bool nan = false;
+        for (int i = lane; i < P * WARPS; i += 32) {
+            hi += tot[(buf * P * WARPS + i) * 2];
+            lo += tot[(buf * P * WARPS + i) * 2 + 1];
+            nan |= tot[(buf * P * WARPS + i) * 2 + 1] == kBadSum;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            hi += __shfl_xor_sync(0xffffffffu, hi, o);
+            lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        }
+        if (__any_sync(0xffffffffu, nan)) return __longlong_as_double(0x7ff8000000000000LL);
+        return double(hi) * 0x1p-24 + double(lo) * 0x1p-68;
+    };
+    cl_arrive<P>();
+    cl_wait<P>();
+    double mean = 0.0;
+    bool bad = false;
+    // sums of the cells in fixed point, scaled to [-1, 1]-like sizes for the
+    // adjoint, whose fields have no natural scale
+    double scale = 1.0;
+    if constexpr (MASS) {
+        if constexpr (ADJ) {
+            // power of two at the field's largest entry
+            T mx = T(0);
+#pragma unroll
+            for (int i = 0; i < K; ++i) mx = fmax(mx, fabs(u[i]));
+            long long e = __double_as_longlong(double(mx));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) e = max(e, (long long)__shfl_xor_sync(0xffffffffu, e, o));
+            for (int q = lane; q < P; q += 32) peer<P>(tot, q)[(P * WARPS + rank * WARPS + warp) * 2] = e;
+            cl_arrive<P>();
+            cl_wait<P>();
+            e = 0;
+            for (int i = lane; i < P * WARPS; i += 32) e = max(e, tot[(P * WARPS + i) * 2]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) e = max(e, (long long)__shfl_xor_sync(0xffffffffu, e, o));
+            // 2^-exponent, exact; a zero or subnormal field keeps 1
+            const int ex = int(e >> 52) - 1023;
+            if (ex > -1000 && ex < 1000) scale = __longlong_as_double((long long)(1023 - ex) << 52);
+        } else {
+            long long hi = 0, lo = 0;
+#pragma unroll
+            for (int i = 0; i < K; ++i) {
+                fix64(double(u[i]), hi, lo);
+                bad |= !(fabs(u[i]) < T(0x1p20));
+            }
+            publish(hi, lo, bad, 1);
+            cl_arrive<P>();
+            cl_wait<P>();
+            mean = collect(1) / double(NN);
+        }
+    }
+
+    for (int step = 0; step < it.steps; ++step) {
+        const int buf = step & 1;
+        T* r = rbuf + buf * RH * N;
+        long long hi = 0, lo = 0;
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const int e = tid + i * kShThreads, y = e / N;
+            T v = u[i];
+            if constexpr (!ADJ) v = fma(v, fma(cf.mdt, v * v, cf.kappa), v);
+            r[M * N + e] = v;
+            if (y < M) rup[buf * RH * N + (M + R) * N + e] = v;
+            if (y >= R - M) rdown[buf * RH * N + e - (R - M) * N] = v;
+            if constexpr (MASS) {
+                fix64(double(v) * scale, hi, lo);
+                bad |= !(fabs(double(v) * scale) < 0x1p20);
+            }
+        }
+        if constexpr (MASS) publish(hi, lo, bad, buf);
+        cl_arrive<P>();
+        cl_wait<P>();
+        T shift = T(0);
+        if constexpr (MASS) {
+            const double m = collect(buf) / (double(NN) * args.a * scale);
+            shift = T(ADJ ? m : mean - m);
+        }
+        // stages: w_k on rows -(M-1-k) .. R + (M-1-k)
+        const T* src = r;
+        int srow = -M;  // row index of src's first stored row
+#pragma unroll
+        for (int k = 0; k < M - 1; ++k) {
+            T* dst = wbuf + (k & 1) * RW * N;
+            const int ext = M - 1 - k;
+            const T g = cf.g[k];
+            for (int e = tid; e < (R + 2 * ext) * N; e += kShThreads) {
+                const int y = e / N - ext, x = e % N;
+                const T* p = src + (y - srow) * N + x;
+                const T* row = p - x;
+                const T t = ((row[(x + N - 1) % N] + row[(x + 1) % N]) + p[-N]) + p[N];
+                dst[(y + M - 1) * N + x] = fma(g, t, r[(y + M) * N + x]);
+            }
+            __syncthreads();
+            src = dst;
+            srow = -(M - 1);
+        }
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const int e = tid + i * kShThreads, y = e / N, x = e % N;
+            const T* p = src + (y - srow) * N + x;
+            const T* row = p - x;
+            const T t = ((row[(x + N - 1) % N] + row[(x + 1) % N]) + p[-N]) + p[N];
+            const T rv = r[(y + M) * N + x];
+            const T t0 = fma(cf.be0, rv, rv);
+            T v = MASS && !ADJ ? t0 + fma(cf.b1, t, shift) : fma(cf.b1, t, t0);
+            if constexpr (ADJ) {
+                const T w = static_cast<const T*>(args.states)[((long long)(it.steps - 1 - step) * args.num_fields + field) * NN +
+                                                               (long long)rank * R * N + e];
+                v = fma(cf.a, v, cf.dt * (T(1) - T(3) * w * w) * (v - shift));
+            }
+            u[i] = v;
+            if (traj) traj[(step + 1) * traj_step + e] = v;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < K; ++i) out[tid + i * kShThreads] = u[i];
+}
+
+template <typename T, int N, int P, int M, bool MASS, bool ADJ>
+int launch_smem_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
+    using Sh = ShShape<T, N, P, M>;
+    auto kern = stencil_smem_kernel<T, N, P, M, MASS, ADJ>;
+    static bool configured = false;
+    if (!configured) {
+        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM)));
+        if (P > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        configured = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(args.num_fields) * P, 1, 1);
+    cfg.blockDim = dim3(kShThreads, 1, 1);
+    cfg.dynamicSmemBytes = Sh::SMEM;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = P;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = P > 1 ? 1 : 0;
+    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<T, M>(args, poly)));
+    count_launch();
+    return AC_OK;
+}
+
+template <typename T, int N, int P, int M>
+int launch_smem(const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
+    if (args.adjoint)
+        return args.mass ? launch_smem_t<T, N, P, M, true, true>(args, poly, st)
+                         : launch_smem_t<T, N, P, M, false, true>(args, poly, st);
+    return args.mass ? launch_smem_t<T, N, P, M, true, false>(args, poly, st)
+                     : launch_smem_t<T, N, P, M, false, false>(args, poly, st);
+}
+
+template <int M>
+int dispatch_smem(int n, const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
+    switch (n) {
+        case 32: return launch_smem<double, 32, 4, M>(args, poly, st);
+        case 64:
+            if constexpr (M <= 4) {
+                if (args.num_fields <= 9) return launch_smem<double, 64, 16, M>(args, poly, st);
+            }
+            return launch_smem<double, 64, 8, M>(args, poly, st);
+        case 128: return launch_smem<double, 128, 16, M>(args, poly, st);
+        case 256: return launch_smem<double, 256, 16, M>(args, poly, st);
+        default: return AC_ERR_UNSUPPORTED;
+    }
+}
+
+}  // namespace
+
+template <>
+int launch_stencil<float>(int n, const FineArgs& args, cudaStream_t stream, bool* taken) {
+    *taken = false;
+    if (n < 32 || n > 512) return AC_OK;
+    // degree 4 rows of 512 columns would need 262 KB of halo buffers
+    const SolvePoly p = solve_poly(args.a, args.lam_scale, 2, AC_F32, 2, n == 512 ? 3 : 4);
+    if (!p.degree) return AC_OK;
+    *taken = true;
+    if (!args.num_fields) return AC_OK;
+    switch (p.degree) {
+        case 2: return dispatch_reg<2>(n, args, p, stream);
+        case 3: return dispatch_reg<3>(n, args, p, stream);
+        default: return dispatch_reg<4>(n, args, p, stream);  // n <= 256
+    }
+}
+
+template <>
+int launch_stencil<double>(int n, const FineArgs& args, cudaStream_t stream, bool* taken) {
+    *taken = false;
+    if (n < 32 || n > 256) return AC_OK;
+    const SolvePoly p = solve_poly(args.a, args.lam_scale, 2, AC_F64, 4, 6);
+    if (!p.degree) return AC_OK;
+    *taken = true;
+    if (!args.num_fields) return AC_OK;
+    switch (p.degree) {
+        case 4: return dispatch_smem<4>(n, args, p, stream);
+        case 5: return dispatch_smem<5>(n, args, p, stream);
+        default: return dispatch_smem<6>(n, args, p, stream);
+    }
+}
+
+}  // namespace acpr

@@ -1,0 +1,114 @@
+"""The polynomial solve of the fine step (fine_stencil.cu, the first launch
+shape) against the Fourier solve (the other shapes) over the forms it accepts:
+every size, degree, model, batch split, trajectories and adjoints."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import acpr_inputs as I
+import paper_2510_07672_gb300 as G
+
+pytestmark = pytest.mark.gpu
+
+F32, F64 = G.AC_F32, G.AC_F64
+
+
+def fields(n, count, prec, amp=0.9, shift=0.0):
+    u = np.stack([I.random_field(n, seed=300 + s, amp=amp) for s in range(count)]) + shift
+    return torch.tensor(u, dtype=torch.float64 if prec == F64 else torch.float32, device="cuda")
+
+
+def with_shape(n, prec, index, call):
+    G.ac_fine_set_variant(n, prec, index)
+    try:
+        return call()
+    finally:
+        G.ac_fine_set_variant(n, prec, 0)
+
+
+def params(n, prec, variant, lam, dt=1e-4):
+    """lam = dt eps^2 4 / h^2 fixes the degree of the polynomial."""
+    return G.FineParams(n, float(np.sqrt(lam / (4 * dt))) / n, 2.0, dt, variant=variant, precision=prec)
+
+
+# lam: float32 degrees 2, 3, 4 below 3.1e-3, 1.5e-2, 4e-2 (512: up to 3); float64 degrees 4, 5, 6 below 1.1e-3, 3.8e-3, 1e-2
+CASES = [(n, F32, lam) for n in (32, 64, 128, 256, 512) for lam in (1.25e-3, 1e-2, 3e-2)]
+CASES += [(n, F64, lam) for n in (32, 64, 128, 256) for lam in (8e-4, 3e-3, 8e-3)]
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n,prec,lam", CASES)
+def test_matches_the_fourier_solve(n, prec, lam, variant):
+    """5 steps.  Tolerance: the round-off of the float32 Fourier solve, about
+    eps log2(n^2) |u| = 2e-6 a step at most; float64 the same with its eps."""
+    fp = params(n, prec, variant, lam)
+    u = fields(n, 3, prec, shift=0.05)
+    a = with_shape(n, prec, 0, lambda: G.ac_fine_propagate_slices(fp, 5, u))
+    b = with_shape(n, prec, 1, lambda: G.ac_fine_propagate_slices(fp, 5, u))
+    assert (a - b).abs().max().item() < (1e-14 if prec == F64 else 1e-5)
+    if variant:
+        drift = (a.double().mean(dim=(1, 2)) - u.double().mean(dim=(1, 2))).abs().max().item()
+        assert drift < (1e-15 if prec == F64 else 1e-8)
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n,prec", [(32, F32), (64, F32), (128, F32), (256, F32), (512, F32), (64, F64), (128, F64)])
+def test_batch_size_does_not_change_the_bits(n, prec, variant):
+    """The split over warps and CTAs follows the batch size; a field's result
+    does not (Parareal's F and the sequential solve are one function)."""
+    count = 80 if n <= 256 else 24
+    fp = params(n, prec, variant, 8e-4)
+    u = fields(n, count, prec)
+    full = G.ac_fine_propagate_slices(fp, 6, u)
+    for f in (0, 1, count - 1):
+        assert torch.equal(G.ac_fine_propagate_slices(fp, 6, u[f:f + 1].clone())[0], full[f])
+    work = torch.tensor([[f, count - 1 - f, 6, 0] for f in range(count)], dtype=torch.int32, device="cuda")
+    out = torch.empty_like(u)
+    G.ac_fine_propagate_work(fp, work, u, out)
+    assert torch.equal(out.flip(0), full)
+    traj = G.ac_fine_trajectory(fp, 6, u[:3].clone())
+    assert torch.equal(traj[0], u[:3]) and torch.equal(traj[6], full[:3])
+    assert torch.equal(traj[2], G.ac_fine_propagate_slices(fp, 2, u[:3].clone()))
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n,prec", [(32, F32), (64, F32), (128, F32), (256, F32), (512, F32), (32, F64), (64, F64), (256, F64)])
+def test_adjoint_matches_the_fourier_solve(n, prec, variant):
+    """lambda of any scale (here 1e-6): relative to its largest value, the
+    tolerance of the forward comparison."""
+    fp = params(n, prec, variant, 1.25e-3)
+    u = fields(n, 2, prec)
+    states = G.ac_fine_trajectory(fp, 4, u)[:4].contiguous()
+    lam = fields(n, 2, prec, amp=0.5, shift=0.2) * 1e-6
+    a = with_shape(n, prec, 0, lambda: G.ac_fine_adjoint(fp, 4, states, lam))
+    b = with_shape(n, prec, 1, lambda: G.ac_fine_adjoint(fp, 4, states, lam))
+    assert (a - b).abs().max().item() < (1e-14 if prec == F64 else 1e-5) * lam.abs().max().item()
+
+
+def test_stiff_steps_take_the_fourier_solve():
+    n = 128
+    for prec in (F32, F64):
+        fp = params(n, prec, 0, 0.25, dt=1e-2)
+        u = fields(n, 2, prec)
+        a = with_shape(n, prec, 0, lambda: G.ac_fine_propagate_slices(fp, 3, u))
+        assert torch.equal(a, with_shape(n, prec, 1, lambda: G.ac_fine_propagate_slices(fp, 3, u)))
+
+
+def test_no_diffusion_and_not_a_number():
+    n = 64
+    for prec in (F32, F64):
+        fp = G.FineParams(n, 0.0, 2.0, 1e-4, precision=prec)  # eps = 0: A is a multiple of the identity
+        u = fields(n, 2, prec)
+        ref = u.double()
+        for _ in range(3):
+            ref = (1.0002 * ref + 1e-4 * (ref - ref ** 3)) / 1.0002
+        assert (G.ac_fine_propagate_slices(fp, 3, u).double() - ref).abs().max().item() < (1e-15 if prec == F64 else 3e-7)
+        for bad in (float("nan"), float("inf")):
+            v = u.clone()
+            v[1, 5, 7] = bad
+            for variant in (0, 1):
+                out = G.ac_fine_propagate_slices(params(n, prec, variant, 1e-3), 2, v)
+                assert torch.isfinite(out[0]).all() and not torch.isfinite(out[1]).all()
+                if variant:  # the mean is not a number
+                    assert torch.isnan(out[1]).all()
