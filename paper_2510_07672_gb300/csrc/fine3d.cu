@@ -2,6 +2,10 @@
 // (d = 3; the 3D experiments of Sec. 4): the 7-point Laplacian, solved by a
 // 3D FFT.
 //
+// Float32 steps whose solve is a polynomial of degree 2 in the 7-point stencil
+// stream the cube once per step (fine_tiles.cu); the passes below serve the
+// stiffer ones and float64.
+//
 // A 128^3 float32 field is 8 MB, beyond one thread-block cluster, so a step is
 // five passes over L2/HBM, each a batch of 1D transforms of length N, 16 lines
 // per CTA:
@@ -19,6 +23,7 @@
 // call (the scheme conserves it exactly; the same reading as the 2D kernel).
 #include "common.cuh"
 #include "fft_reg.cuh"
+#include "fine_tiles.cuh"
 
 #include <cmath>
 
@@ -212,6 +217,15 @@ int propagate3d(const ac_params* p, int steps, int fields, const T* u_in, T* u_o
     T* s2 = reinterpret_cast<T*>(work + s2_off);
     double* part = reinterpret_cast<double*>(work + part_off);
     const double h = p->length / N;
+    if constexpr (sizeof(T) == 4) {
+        const SolvePoly poly = solve_poly(1.0 + p->S * p->dt, 4.0 * p->dt * p->eps * p->eps / (h * h), 3, AC_F32, 2, 2);
+        // (the streaming kernel reads vectors)
+        const bool aligned = (reinterpret_cast<uintptr_t>(u_in) | reinterpret_cast<uintptr_t>(u_out) |
+                              reinterpret_cast<uintptr_t>(work)) % 16 == 0;
+        if (poly.degree && steps > 0 && aligned)
+            return cube_run(p, poly, steps, fields, u_in, u_out, reinterpret_cast<float*>(W),
+                            reinterpret_cast<long long*>(part), st);
+    }
     fine3d_tables<T, N><<<1, N, 0, st>>>(tw, s2, 4.0 * p->dt * p->eps * p->eps / (h * h));
     ACPR_LAUNCH_CHECK();
     if (p->variant == AC_MASS_CONSERVING) {

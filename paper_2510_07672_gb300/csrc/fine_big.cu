@@ -1,6 +1,7 @@
 // fine_big.cu -- the fine propagator for fields too large for one cluster's
-// shared memory (1024 x 1024 float32: 4 MB), in two passes per step through
-// L2/HBM.  Same step and same arithmetic layout as fine.cu (Sec. 3.1): rows
+// shared memory (1024 x 1024 float32: 4 MB).  Steps whose solve is a polynomial
+// of degree 2 run on tiles (fine_tiles.cu); the kernels here serve the stiffer
+// ones, in two passes per step through L2/HBM.  Same step and same arithmetic layout as fine.cu (Sec. 3.1): rows
 // 2p and 2p+1 of a field share a complex line, the row spectra Z_p[k] are
 // split into the two rows' half spectra by the column owner (DC and Nyquist
 // columns packed in column 0), and rebuilt before the inverse row FFT.
@@ -16,6 +17,7 @@
 
 #include "common.cuh"
 #include "fft_reg.cuh"
+#include "fine_tiles.cuh"
 
 namespace acpr {
 
@@ -387,6 +389,15 @@ int fine_big_run(const ac_params* p, int groups, int per_group, int steps, const
     a.dt = p->dt;
     const double h = p->length / p->n;
     a.lam_scale = p->dt * p->eps * p->eps * 4.0 / (h * h);
+    const SolvePoly poly = solve_poly(a.a, a.lam_scale, 2, AC_F32, 2, 2);
+    if (poly.degree && steps > 0) {
+        // the first half of the spectra's space holds the intermediate fields,
+        // the second the sums of the mass model
+        const FieldMap src{const_cast<float*>(static_cast<const float*>(in)), per_group, in_gs, in_off, map};
+        const FieldMap dst{static_cast<float*>(out), per_group, out_gs, out_off, map};
+        return big_tiles_run(poly, a.a, a.dt, a.mass, fields, steps, src, dst, reinterpret_cast<float*>(base),
+                             reinterpret_cast<long long*>(base + zbytes), st);
+    }
     big_tables_kernel<T, N><<<(N + 255) / 256, 256, 0, st>>>(tw_tab, lam_tab, a.lam_scale);
     ACPR_LAUNCH_CHECK();
     if (a.mass) {

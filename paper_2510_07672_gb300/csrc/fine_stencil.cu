@@ -35,7 +35,7 @@
 #include <algorithm>
 #include <cmath>
 
-#include "fine.cuh"
+#include "fine_stencil.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -47,12 +47,12 @@ SolvePoly solve_poly(double a, double lam_scale, int dims, int precision, int mi
     // z = x / h = T / (2 dims): c_0 = 1 / R, c_k = 2 rho^k / R
     const double h = 0.5 * dims * lam_scale, C = a + h;
     const double R = std::sqrt((C - h) * (C + h)), rho = h / (C + R);
-    // The error is largest for the checkerboard mode, 4 rho^(M+1): at most a
-    // quarter of a rounding in float32, two in float64.  Against a long double
+    // The error is largest for the checkerboard mode, 4 rho^(M+1): at most one
+    // rounding in float32, two in float64.  Against a long double
     // solve, 300 steps at 128^2 (lambda = 1.25e-3): degree 4 6e-14, degree 5
     // 2.6e-14, a float64 Fourier solve 5e-14; at 64^2 (1e-3), 400 steps:
     // degree 4 2.8e-14, Fourier 6e-14.
-    const double tol = precision == AC_F64 ? 0x1p-52 : 0x1p-26;
+    const double tol = precision == AC_F64 ? 0x1p-52 : 0x1p-24;
     int M = std::max(1, min_degree);
     while (M <= max_degree && 4.0 * std::pow(rho, M + 1) > tol) ++M;
     if (M > max_degree || M > kMaxDegree || !(a > 0.0) || !std::isfinite(rho)) return out;
@@ -78,32 +78,6 @@ SolvePoly solve_poly(double a, double lam_scale, int dims, int precision, int mi
 }
 
 namespace {
-
-// Coefficients of one call in the fields' precision.
-template <typename T, int M>
-struct Coef {
-    T kappa, mdt;   // r = u + u (kappa + mdt u^2)
-    T be0, b1;      // u' = r + be0 r + b1 T w_1
-    T g[M];         // g[k], k = 0 .. M - 2: stage k, w = r + g[k] T (input)
-    T a, dt;        // adjoint: lambda' = a mu + dt f'(u) (mu - mean)
-};
-
-template <typename T, int M>
-Coef<T, M> make_coef(const FineArgs& args, const SolvePoly& p) {
-    Coef<T, M> c{};
-    c.kappa = T((args.a - 1.0) + args.dt);
-    c.mdt = T(-args.dt);
-    c.be0 = T(p.b[0] - 1.0);
-    c.b1 = T(p.b[1]);
-    // stage k applies the ratio of the coefficients M - k and M - k - 1
-    for (int k = 0; k + 1 < M; ++k) {
-        const double hi = p.b[M - k], lo = p.b[M - k - 1];
-        c.g[k] = std::fabs(lo) > 1e-200 ? T(hi / lo) : T(0);
-    }
-    c.a = T(args.a);
-    c.dt = T(args.dt);
-    return c;
-}
 
 template <int P>
 __device__ __forceinline__ void cl_arrive() {
@@ -151,35 +125,6 @@ __device__ __forceinline__ Item item_of(const FineArgs& args, int field) {
 // neighbouring CTAs of the cluster through their shared memory: M rows each
 // way per step, double-buffered, one cluster barrier per step.
 
-template <int W>
-__device__ __forceinline__ void row_store(float* dst, const float (&x)[W], int lane) {
-    // chunks of VW floats, chunk-major: lanes store consecutive vectors
-    constexpr int VW = W >= 4 ? 4 : W;
-#pragma unroll
-    for (int v = 0; v < W / VW; ++v) {
-        float* p = dst + v * 32 * VW + lane * VW;
-        if constexpr (VW == 4) *reinterpret_cast<float4*>(p) = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
-        else if constexpr (VW == 2) *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
-        else *p = x[0];
-    }
-}
-template <int W>
-__device__ __forceinline__ void row_load(const float* src, float (&x)[W], int lane) {
-    constexpr int VW = W >= 4 ? 4 : W;
-#pragma unroll
-    for (int v = 0; v < W / VW; ++v) {
-        const float* p = src + v * 32 * VW + lane * VW;
-        if constexpr (VW == 4) {
-            const float4 q = *reinterpret_cast<const float4*>(p);
-            x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w;
-        } else if constexpr (VW == 2) {
-            const float2 q = *reinterpret_cast<const float2*>(p);
-            x[0] = q.x; x[1] = q.y;
-        } else {
-            x[0] = *p;
-        }
-    }
-}
 // The lane's W columns of a row in global memory (row base, 16-byte aligned).
 template <int W>
 __device__ __forceinline__ void grow_load(const float* row, float (&x)[W], int lane) {
@@ -206,102 +151,6 @@ __device__ __forceinline__ void grow_store(float* row, const float (&x)[W], int 
 #pragma unroll
         for (int c = 0; c < W; ++c) p[c] = x[c];
     }
-}
-
-// Left plus right neighbour of every column of a row.
-template <int W>
-__device__ __forceinline__ void hsum(const float (&x)[W], float (&h)[W], int lane) {
-    const float l = __shfl_sync(0xffffffffu, x[W - 1], (lane + 31) & 31);
-    const float r = __shfl_sync(0xffffffffu, x[0], (lane + 1) & 31);
-#pragma unroll
-    for (int c = 0; c < W; ++c) h[c] = (c ? x[c - 1] : l) + (c + 1 < W ? x[c + 1] : r);
-}
-
-// r <- p(Lap) r for the warp's H rows; halo(y, x) gives row y of r outside
-// them (-M <= y < 0 or H <= y < H + M).  Rows stream through the M stages; a
-// stage keeps its last row (p) and the three known neighbours of that row's
-// cells (s), so T = ((left + right) + above) + below for every cell.
-// SHIFT: plus `shift`, added to the small term: r + be0 r lies on the coarse
-// grid of its binade, where a shift below half a unit would be rounded away in
-// all of its cells alike.
-template <int W, int H, int M, bool SHIFT, class Halo>
-__device__ __forceinline__ void apply_poly(float (&r)[H][W], const Coef<float, M>& cf, int lane, float shift,
-                                           Halo halo) {
-    float s[M][W], p[M][W];
-#pragma unroll
-    for (int y = -M; y < H + M; ++y) {
-        float x[W];
-        if (y >= 0 && y < H) {
-#pragma unroll
-            for (int c = 0; c < W; ++c) x[c] = r[y][c];
-        } else {
-            halo(y, x);
-        }
-#pragma unroll
-        for (int k = 0; k < M; ++k) {
-            const int yk = y - k, first = k - M;  // x is row yk of the stage's input, whose first row is `first`
-            if (yk < first) break;
-            float nx[W];
-            const bool emit = yk >= first + 2;
-            if (emit) {
-                if (k < M - 1) {
-                    float rr[W];
-                    const int yr = yk - 1;
-                    if (k == 0) {
-#pragma unroll
-                        for (int c = 0; c < W; ++c) rr[c] = p[0][c];
-                    } else if (yr >= 0 && yr < H) {
-#pragma unroll
-                        for (int c = 0; c < W; ++c) rr[c] = r[yr][c];
-                    } else {
-                        halo(yr, rr);
-                    }
-#pragma unroll
-                    for (int c = 0; c < W; ++c) nx[c] = fmaf(cf.g[k], s[k][c] + x[c], rr[c]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < W; ++c) {
-                        const float t0 = fmaf(cf.be0, r[yk - 1][c], r[yk - 1][c]);
-                        r[yk - 1][c] = SHIFT ? t0 + fmaf(cf.b1, s[k][c] + x[c], shift) : fmaf(cf.b1, s[k][c] + x[c], t0);
-                    }
-                }
-            }
-            if (yk > first && yk < H + M - k - 1) {
-                float h[W];
-                hsum<W>(x, h, lane);
-#pragma unroll
-                for (int c = 0; c < W; ++c) s[k][c] = h[c] + p[k][c];
-            }
-#pragma unroll
-            for (int c = 0; c < W; ++c) p[k][c] = x[c];
-            if (!emit || k == M - 1) break;
-#pragma unroll
-            for (int c = 0; c < W; ++c) x[c] = nx[c];
-        }
-    }
-}
-
-constexpr float kFix = 16777216.f;  // 2^24: fixed point of the sums of r
-constexpr long long kBadSum = (long long)(1ULL << 63);
-
-// Sum over the warp's lanes of a 62-bit integer, on every lane.
-__device__ __forceinline__ long long warp_sum_s64(long long v) {
-    const int a0 = int(v & 0xfffff), a1 = int((v >> 20) & 0xfffff), a2 = int(v >> 40);
-    return (long long)__reduce_add_sync(0xffffffffu, a0) + ((long long)__reduce_add_sync(0xffffffffu, a1) << 20) +
-           ((long long)__reduce_add_sync(0xffffffffu, a2) << 40);
-}
-
-// Sum of the two rows' cells of a lane (the same order under every split).
-template <int W>
-__device__ __forceinline__ float pair_sum(const float (&x)[W], const float (&y)[W]) {
-    float t[W];
-#pragma unroll
-    for (int c = 0; c < W; ++c) t[c] = x[c] + y[c];
-#pragma unroll
-    for (int o = W / 2; o > 0; o /= 2)
-#pragma unroll
-        for (int c = 0; c < o; ++c) t[c] += t[c + o];
-    return t[0];
 }
 
 template <int N, int H, int NW, int P, int M>
@@ -497,7 +346,7 @@ int launch_reg_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t strea
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = P > 1 ? 1 : 0;
-    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<float, M>(args, poly)));
+    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<float, M>(args.a, args.dt, poly)));
     count_launch();
     return AC_OK;
 }
@@ -750,7 +599,7 @@ int launch_smem_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stre
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = P > 1 ? 1 : 0;
-    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<T, M>(args, poly)));
+    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<T, M>(args.a, args.dt, poly)));
     count_launch();
     return AC_OK;
 }
@@ -785,6 +634,10 @@ template <>
 int launch_stencil<float>(int n, const FineArgs& args, cudaStream_t stream, bool* taken) {
     *taken = false;
     if (n < 32 || n > 512) return AC_OK;
+    // rows move as vectors; callers that pass unaligned fields keep the Fourier kernels
+    if ((reinterpret_cast<uintptr_t>(args.in) | reinterpret_cast<uintptr_t>(args.out) |
+         reinterpret_cast<uintptr_t>(args.states) | reinterpret_cast<uintptr_t>(args.traj)) % 16)
+        return AC_OK;
     // degree 4 rows of 512 columns would need 262 KB of halo buffers
     const SolvePoly p = solve_poly(args.a, args.lam_scale, 2, AC_F32, 2, n == 512 ? 3 : 4);
     if (!p.degree) return AC_OK;

@@ -32,7 +32,7 @@ def params(n, prec, variant, lam, dt=1e-4):
     return G.FineParams(n, float(np.sqrt(lam / (4 * dt))) / n, 2.0, dt, variant=variant, precision=prec)
 
 
-# lam: float32 degrees 2, 3, 4 below 3.1e-3, 1.5e-2, 4e-2 (512: up to 3); float64 degrees 4, 5, 6 below 1.1e-3, 3.8e-3, 1e-2
+# lam: float32 degrees 2, 3, 4 below 4.9e-3, 2.2e-2, 5.5e-2 (512: up to 3); float64 degrees 4, 5, 6 below 1.1e-3, 3.8e-3, 1e-2
 CASES = [(n, F32, lam) for n in (32, 64, 128, 256, 512) for lam in (1.25e-3, 1e-2, 3e-2)]
 CASES += [(n, F64, lam) for n in (32, 64, 128, 256) for lam in (8e-4, 3e-3, 8e-3)]
 
@@ -112,3 +112,52 @@ def test_no_diffusion_and_not_a_number():
                 assert torch.isfinite(out[0]).all() and not torch.isfinite(out[1]).all()
                 if variant:  # the mean is not a number
                     assert torch.isnan(out[1]).all()
+
+
+def field_ref(u, fp, steps):
+    """The step with a float64 Fourier solve, 2D or 3D."""
+    n, dims = fp.n, u.dim() - 1
+    axes = tuple(range(1, dims + 1))
+    s2 = torch.sin(torch.pi * torch.arange(n, device="cuda", dtype=torch.float64) / n) ** 2
+    sym = 1 + fp.S * fp.dt
+    for a in range(dims):
+        m = s2[: n // 2 + 1] if a == dims - 1 else s2
+        sym = sym + fp.dt * fp.eps ** 2 * 4 * n * n * m.reshape([-1 if a == b else 1 for b in range(dims)])
+    v = u.double()
+    for _ in range(steps):
+        f = v - v ** 3
+        if fp.variant:
+            f = f - f.mean(dim=axes, keepdim=True)
+        v = torch.fft.irfftn(torch.fft.rfftn((1 + fp.S * fp.dt) * v + fp.dt * f, dim=axes) / sym, s=(n,) * dims, dim=axes)
+    return v
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("steps", [1, 3, 4, 5, 9])
+def test_tiles_1024(steps, variant):
+    """One to three launches of up to four steps, every tile edge: against
+    float64.  Tolerance: two roundings of values below 1 a step."""
+    n = 1024
+    fp = G.FineParams(n, 0.004, 2.0, 2e-5, variant=variant, precision=F32)
+    u = fields(n, 2, F32, shift=0.03)
+    out = G.ac_fine_propagate_slices(fp, steps, u)
+    assert (out.double() - field_ref(u, fp, steps)).abs().max().item() < 1.2e-7 * (steps + 1)
+    if variant:
+        assert (out.double().mean(dim=(1, 2)) - u.double().mean(dim=(1, 2))).abs().max().item() < 1e-8
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n,count,steps", [(32, 3, 1), (32, 41, 4), (64, 1, 3), (64, 5, 2), (128, 1, 3), (128, 9, 2)])
+def test_cube_stream(n, count, steps, variant):
+    """Chunk lengths from 8 to 32 planes, in place and out of place."""
+    dt = 1e-4
+    fp = G.FineParams(n, float(np.sqrt(2.5e-3 / (4 * dt))) / n, 2.0, dt, variant=variant, precision=F32)
+    g = torch.Generator(device="cuda").manual_seed(n + count)
+    u = torch.rand((count, n, n, n), generator=g, device="cuda") * 1.8 - 0.85
+    out = G.ac_fine3d_propagate(fp, steps, u)
+    assert (out.double() - field_ref(u, fp, steps)).abs().max().item() < 1.2e-7 * (steps + 1)
+    if variant:
+        assert (out.double().mean(dim=(1, 2, 3)) - u.double().mean(dim=(1, 2, 3))).abs().max().item() < 1e-8
+    v = u.clone()
+    G.ac_fine3d_propagate(fp, steps, v, v)
+    assert torch.equal(v, out)
