@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "f32x2.cuh"
 
 namespace acpr {
 
@@ -31,33 +32,6 @@ __device__ __forceinline__ float phi_as(float x) {
     return x >= 0.0f ? 1.0f - q : q;
 }
 
-// Paired float32 arithmetic: two lanes in one 64-bit register, operated on by
-// the sm_100-family .f32x2 instructions (one issue for two results), each
-// lane rounded exactly as the scalar add / mul / fma.
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 f2(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void f2split(f32x2 v, float& a, float& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 // Hardware approximations: 1/x and 2^x (PTX rcp.approx, ex2.approx).
 __device__ __forceinline__ float rcp_hw(float x) {
     float r;

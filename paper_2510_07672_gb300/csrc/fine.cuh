@@ -54,4 +54,8 @@ SolvePoly solve_poly(double a, double lam_scale, int dims, int precision, int mi
 template <typename T>
 int launch_stencil(int n, const FineArgs& args, cudaStream_t stream, bool* taken);
 
+// The adjoint steps of `adj` and the forward steps of `fwd` (same step, other
+// fields) side by side in one launch, where the polynomial solve serves them.
+int launch_stencil_pair(int n, int precision, const FineArgs& adj, const FineArgs& fwd, cudaStream_t stream, bool* taken);
+
 }  // namespace acpr

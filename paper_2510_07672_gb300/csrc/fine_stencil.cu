@@ -27,11 +27,11 @@
 // the order and of the split.
 //
 // Bound: FP32 (float64: FP64) issue.  Measured, Fourier kernel -> this one:
-//   512 fields of 256^2, mass, 100 steps        11.40 -> 2.22 ms
-//   21 fields of 512^2, 50 to 90 steps           3.01 -> 0.37 ms
-//   float64 256^2, 300 steps, their recomputation and adjoint  138 -> 26 ms
-//   one step of one 128^2 field (call included)  16.4 -> 11.8 us
-// Error against 64 bits after 100 float32 steps at 256^2: 1.5e-5 -> 2e-6.
+//   512 fields of 256^2, mass, 100 steps        11.40 -> 1.98 ms (2.21 with scalar instructions and 8x8x4)
+//   21 fields of 512^2, 50 to 90 steps           3.01 -> 0.25 ms (0.37)
+//   float64 256^2, 300 steps, their recomputation and adjoint  138 -> 22.5 ms (32.3 one after the other)
+//   one step of one 128^2 field (call included)  16.4 -> 9.6 us
+// Error against 64 bits after 100 float32 steps at 256^2: 1.5e-5 -> 1.5e-6.
 #include <algorithm>
 #include <cmath>
 
@@ -127,29 +127,33 @@ __device__ __forceinline__ Item item_of(const FineArgs& args, int field) {
 
 // The lane's W columns of a row in global memory (row base, 16-byte aligned).
 template <int W>
-__device__ __forceinline__ void grow_load(const float* row, float (&x)[W], int lane) {
+__device__ __forceinline__ void grow_load(const float* row, LaneV<W> (&x)[Lane<W>::E], int lane) {
     const float* p = row + lane * W;
+    float c[W];
     if constexpr (W >= 4) {
 #pragma unroll
         for (int v = 0; v < W / 4; ++v) {
             const float4 q = reinterpret_cast<const float4*>(p)[v];
-            x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w;
+            c[4 * v] = q.x; c[4 * v + 1] = q.y; c[4 * v + 2] = q.z; c[4 * v + 3] = q.w;
         }
     } else {
 #pragma unroll
-        for (int c = 0; c < W; ++c) x[c] = p[c];
+        for (int i = 0; i < W; ++i) c[i] = p[i];
     }
+    to_lane<W>(c, x);
 }
 template <int W>
-__device__ __forceinline__ void grow_store(float* row, const float (&x)[W], int lane) {
+__device__ __forceinline__ void grow_store(float* row, const LaneV<W> (&x)[Lane<W>::E], int lane) {
     float* p = row + lane * W;
+    float c[W];
+    from_lane<W>(x, c);
     if constexpr (W >= 4) {
 #pragma unroll
         for (int v = 0; v < W / 4; ++v)
-            reinterpret_cast<float4*>(p)[v] = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
+            reinterpret_cast<float4*>(p)[v] = make_float4(c[4 * v], c[4 * v + 1], c[4 * v + 2], c[4 * v + 3]);
     } else {
 #pragma unroll
-        for (int c = 0; c < W; ++c) p[c] = x[c];
+        for (int i = 0; i < W; ++i) p[i] = c[i];
     }
 }
 
@@ -161,11 +165,11 @@ struct RegShape {
     static_assert(R * P == N && H % 2 == 0 && H >= M && N % 32 == 0, "split");
 };
 
-template <int N, int H, int NW, int P, int M, int MINB, bool MASS, bool ADJ>
-__global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid_constant__ FineArgs args,
-                                                                    const __grid_constant__ Coef<float, M> cf) {
+template <int N, int H, int NW, int P, int M, bool MASS, bool ADJ>
+__device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coef<float, M>& cf, int field) {
     using Sh = RegShape<N, H, NW, P, M>;
-    constexpr int W = Sh::W, R = Sh::R;
+    constexpr int W = Sh::W, R = Sh::R, E = Lane<W>::E;
+    using V = LaneV<W>;
     constexpr long long NN = (long long)N * N;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* halo = reinterpret_cast<float*>(smem_raw);  // [buffer][0: above, 1: below][warp][M][N]
@@ -173,7 +177,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int rank = 0;
     if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
-    const int field = blockIdx.x / P;
     const Item it = item_of(args, field);
     const int row0 = rank * R + warp * H;
     const float* in = static_cast<const float*>(args.in) + it.fin * NN + (long long)row0 * N;
@@ -181,7 +184,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
     float* traj = args.traj ? static_cast<float*>(args.traj) + field * NN + (long long)row0 * N : nullptr;
     const long long traj_step = (long long)args.num_fields * NN;
 
-    float u[H][W];
+    V u[H][E];
 #pragma unroll
     for (int y = 0; y < H; ++y) grow_load<W>(in + y * N, u[y], lane);
     if (traj) {
@@ -210,12 +213,15 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
         long long acc = 0;
         bool bad = false;
 #pragma unroll
-        for (int y = 0; y < H; ++y)
+        for (int y = 0; y < H; ++y) {
+            float v[W];
+            from_lane<W>(u[y], v);
 #pragma unroll
             for (int c = 0; c < W; ++c) {
-                acc += __float2ll_rn(u[y][c] * kFix);
-                bad |= !(fabsf(u[y][c]) < 0x1p19f);
+                acc += __float2ll_rn(v[c] * kFix);
+                bad |= !(fabsf(v[c]) < 0x1p19f);
             }
+        }
         acc = warp_sum_s64(acc);
         if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
         cl_wait<P>();
@@ -234,24 +240,28 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
     } else {
         cl_wait<P>();
     }
-    const float inv_fix = float(1.0 / (args.a * double(NN) * double(kFix)));
+    const float inv_fix = float(cf.inv_sum) * (1.f / kFix);
 
     for (int step = 0; step < it.steps; ++step) {
         const int buf = step & 1;
-        if constexpr (!ADJ) {
+        // the rows that others wait for first
+        auto rhs_row = [&](int y) {
+            if constexpr (!ADJ) {
 #pragma unroll
-            for (int y = 0; y < H; ++y)
+                for (int c = 0; c < E; ++c) u[y][c] = rhs(u[y][c], vset<V>(cf.mdt), vset<V>(cf.kappa));
+            }
+        };
 #pragma unroll
-                for (int c = 0; c < W; ++c) {
-                    const float v = u[y][c];
-                    u[y][c] = fmaf(v, fmaf(cf.mdt, v * v, cf.kappa), v);
-                }
-        }
+        for (int y = 0; y < H; ++y)
+            if (y < M || y >= H - M) rhs_row(y);
 #pragma unroll
         for (int m = 0; m < M; ++m) {
             row_store<W>(up + buf * BUF + m * N, u[m], lane);
             row_store<W>(down + buf * BUF + m * N, u[H - M + m], lane);
         }
+        if constexpr (!MASS) cl_arrive<P>();
+#pragma unroll
+        for (int y = M; y < H - M; ++y) rhs_row(y);
         if constexpr (MASS) {
             if constexpr (!ADJ) {
                 long long acc = 0;
@@ -274,17 +284,20 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
                 publish_total(__double_as_longlong(msum), buf);
             }
         }
-        cl_arrive<P>();
+        if constexpr (MASS) cl_arrive<P>();
         cl_wait<P>();
+        // the shift of the mass model, and the adjoint's mean of mu
         float shift = 0.f;
-        if constexpr (MASS) {
+        auto collect = [&]() -> float {
             const long long* tb = tot + buf * P * NW;
             if constexpr (!ADJ) {
                 long long t = 0;
                 bool bad = target == kBadSum;
-                for (int i = lane; i < P * NW; i += 32) {
-                    t += tb[i];
-                    bad |= tb[i] == kBadSum;
+#pragma unroll
+                for (int i0 = 0; i0 < P * NW; i0 += 32) {
+                    const long long v = P * NW % 32 == 0 || i0 + lane < P * NW ? tb[i0 + lane] : 0;
+                    t += v;
+                    bad |= v == kBadSum;
                 }
                 t = warp_sum_s64(t);
                 shift = float(target - t) * inv_fix;
@@ -294,23 +307,29 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
                 for (int i = lane; i < P * NW; i += 32) t += __longlong_as_double(tb[i]);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                shift = float(t / (double(NN) * args.a));  // mean of mu
+                shift = float(t * cf.inv_sum);
             }
-        }
-        apply_poly<W, H, M, MASS && !ADJ>(u, cf, lane, shift, [&](int y, float(&x)[W]) {
-            row_load<W>((y < 0 ? above + (y + M) * N : below + (y - H) * N) + buf * BUF, x, lane);
-        });
+            return shift;
+        };
+        apply_poly<W, H, M, MASS && !ADJ>(
+            u, cf, lane,
+            [&](int y, V(&x)[E]) {
+                row_load<W>((y < 0 ? above + (y + M) * N : below + (y - H) * N) + buf * BUF, x, lane);
+            },
+            collect);
+        if constexpr (MASS && ADJ) collect();
         if constexpr (ADJ) {
             const float* un = static_cast<const float*>(args.states) +
                               ((long long)(it.steps - 1 - step) * args.num_fields + field) * NN + (long long)row0 * N;
 #pragma unroll
             for (int y = 0; y < H; ++y) {
-                float v[W];
+                V v[E];
                 grow_load<W>(un + y * N, v, lane);
+                const V one = vset<V>(1.f), m3 = vset<V>(-3.f), a = vset<V>(cf.a), dt = vset<V>(cf.dt), ms = vset<V>(-shift);
 #pragma unroll
-                for (int c = 0; c < W; ++c) {
-                    const float f = 1.f - 3.f * v[c] * v[c];
-                    u[y][c] = fmaf(cf.a, u[y][c], cf.dt * f * (u[y][c] - shift));
+                for (int c = 0; c < E; ++c) {
+                    const V f = vmul(dt, vfma(m3, vmul(v[c], v[c]), one));
+                    u[y][c] = vfma(a, u[y][c], vmul(f, vadd(u[y][c], ms)));
                 }
             }
         }
@@ -325,30 +344,61 @@ __global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid
 }
 
 template <int N, int H, int NW, int P, int M, int MINB, bool MASS, bool ADJ>
-int launch_reg_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
-    using Sh = RegShape<N, H, NW, P, M>;
-    auto kern = stencil_reg_kernel<N, H, NW, P, M, MINB, MASS, ADJ>;
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM)));
+__global__ void __launch_bounds__(NW * 32, MINB) stencil_reg_kernel(const __grid_constant__ FineArgs args,
+                                                                    const __grid_constant__ Coef<float, M> cf) {
+    stencil_reg_body<N, H, NW, P, M, MASS, ADJ>(args, cf, blockIdx.x / P);
+}
+
+// Adjoint steps of some fields and forward steps of others in one launch.
+template <int N, int H, int NW, int P, int M, bool MASS>
+__global__ void __launch_bounds__(NW * 32, 1) stencil_reg_pair_kernel(const __grid_constant__ FineArgs adj,
+                                                                      const __grid_constant__ FineArgs fwd,
+                                                                      const __grid_constant__ Coef<float, M> cf) {
+    const int f = blockIdx.x / P;
+    if (f < adj.num_fields) stencil_reg_body<N, H, NW, P, M, MASS, true>(adj, cf, f);
+    else stencil_reg_body<N, H, NW, P, M, MASS, false>(fwd, cf, f - adj.num_fields);
+}
+
+// Launches a kernel in clusters of P CTAs.
+template <typename K, typename... A>
+int launch_clusters(K kern, bool* configured, int P, unsigned fields, int threads, size_t smem, cudaStream_t stream,
+                    const A&... a) {
+    if (!*configured) {
+        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
         if (P > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        configured = true;
+        *configured = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(args.num_fields) * P, 1, 1);
-    cfg.blockDim = dim3(NW * 32, 1, 1);
-    cfg.dynamicSmemBytes = Sh::SMEM;
+    cfg.gridDim = dim3(fields * unsigned(P), 1, 1);
+    cfg.blockDim = dim3(unsigned(threads), 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = P;
+    attr[0].val.clusterDim.x = unsigned(P);
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = P > 1 ? 1 : 0;
-    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<float, M>(args.a, args.dt, poly)));
+    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, a...));
     count_launch();
     return AC_OK;
+}
+
+template <int N, int H, int NW, int P, int M, int MINB, bool MASS, bool ADJ>
+int launch_reg_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
+    using Sh = RegShape<N, H, NW, P, M>;
+    static bool configured = false;
+    return launch_clusters(stencil_reg_kernel<N, H, NW, P, M, MINB, MASS, ADJ>, &configured, P, unsigned(args.num_fields), NW * 32, Sh::SMEM, stream, args,
+                           make_coef<float, M>(args.a, args.dt, double(N) * N, poly));
+}
+
+template <int N, int H, int NW, int P, int M, bool MASS>
+int launch_reg_pair(const FineArgs& adj, const FineArgs& fwd, const SolvePoly& poly, cudaStream_t stream) {
+    static bool configured = false;
+    return launch_clusters(stencil_reg_pair_kernel<N, H, NW, P, M, MASS>, &configured, P,
+                           unsigned(adj.num_fields + fwd.num_fields), NW * 32, RegShape<N, H, NW, P, M>::SMEM, stream, adj,
+                           fwd, make_coef<float, M>(adj.a, adj.dt, double(N) * N, poly));
 }
 
 template <int N, int H, int NW, int P, int M, int MINB>
@@ -360,26 +410,48 @@ int launch_reg(const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
                      : launch_reg_t<N, H, NW, P, M, MINB, false, false>(args, poly, st);
 }
 
-// The split by size, degree and batch.
+// The split (rows a warp, warps a CTA, CTAs a field, CTAs per SM) by size and
+// batch.  40 steps, us, mass-conserving / classic, measured for each line:
+//   256: 4x4x16  1 field 60/36, 8 70/45; 8x4x8 (1 CTA per SM's registers)  8 fields 62/42, 24 87/67;
+//        8x4x8 (4 CTAs)  38 fields 106/83, 512 825/650; 8x8x4 512 fields 923/645, 8x16x2 999/703
+//   512: 8x4x16  1 field 105/70, 21 216/164, 64 599/504; 4x8x16  112/72, 317/206, 1033/677
+//   128: 4x4x8   1 field 38/25, 16 44/31; 8x4x4  16 fields 44/29, 64 56/38, 128 82/58;
+//        16x8x1  64 fields 83/49, 128 83/50, 512 261/166 (8x4x4 252/177)
+//   64:  4x4x4   1 field 29/21, 76 40/29; 16x4x1  39/18, 76 40/18, 512 79/50
+//   32:  8x4x1   1 field 22/14, 512 40/24; 4x8x1 22/13, 49/29
+// Degrees 3 and 4 keep more rows of the stages in registers and hold fewer
+// rows of the field.
 template <int M>
 int dispatch_reg(int n, const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
     const int F = args.num_fields;
-    switch (n) {
-        case 32: return launch_reg<32, 4, 8, 1, M, 1>(args, poly, st);
-        case 64:
-            if (F <= 38) return launch_reg<64, 4, 4, 4, M, 1>(args, poly, st);
-            return launch_reg<64, 8, 8, 1, M, 1>(args, poly, st);
-        case 128:
-            if (F <= 19) return launch_reg<128, 4, 4, 8, M, 1>(args, poly, st);
-            return launch_reg<128, 8, 8, 2, M, 2>(args, poly, st);
-        case 256:
-            if constexpr (M == 2)
-                if (F > 19) return launch_reg<256, 8, 8, 4, M, 2>(args, poly, st);
-            return launch_reg<256, 4, 8, 8, M, 2>(args, poly, st);
-        case 512:
-            if constexpr (M <= 3) return launch_reg<512, 4, 8, 16, M, 1>(args, poly, st);
-            return AC_ERR_UNSUPPORTED;
-        default: return AC_ERR_UNSUPPORTED;
+    if constexpr (M == 2) {
+        switch (n) {
+            case 32: return launch_reg<32, 8, 4, 1, M, 1>(args, poly, st);
+            case 64:
+                if (args.mass && F <= 76) return launch_reg<64, 4, 4, 4, M, 1>(args, poly, st);
+                return launch_reg<64, 16, 4, 1, M, 4>(args, poly, st);
+            case 128:
+                if (F <= 12) return launch_reg<128, 4, 4, 8, M, 1>(args, poly, st);
+                if (F <= 96) return launch_reg<128, 8, 4, 4, M, 4>(args, poly, st);
+                return launch_reg<128, 16, 8, 1, M, 2>(args, poly, st);
+            case 256:
+                if (F <= 6) return launch_reg<256, 4, 4, 16, M, 1>(args, poly, st);
+                if (F <= 24) return launch_reg<256, 8, 4, 8, M, 1>(args, poly, st);
+                return launch_reg<256, 8, 4, 8, M, 4>(args, poly, st);
+            case 512: return launch_reg<512, 8, 4, 16, M, 2>(args, poly, st);
+            default: return AC_ERR_UNSUPPORTED;
+        }
+    } else {
+        switch (n) {
+            case 32: return launch_reg<32, 4, 8, 1, M, 1>(args, poly, st);
+            case 64: return launch_reg<64, 8, 8, 1, M, 1>(args, poly, st);
+            case 128: return launch_reg<128, 8, 8, 2, M, 2>(args, poly, st);
+            case 256: return launch_reg<256, 4, 8, 8, M, 2>(args, poly, st);
+            case 512:
+                if constexpr (M == 3) return launch_reg<512, 4, 8, 16, M, 1>(args, poly, st);
+                return AC_ERR_UNSUPPORTED;
+            default: return AC_ERR_UNSUPPORTED;
+        }
     }
 }
 
@@ -412,8 +484,7 @@ __device__ __forceinline__ void fix64(double x, long long& hi, long long& lo) {
 }
 
 template <typename T, int N, int P, int M, bool MASS, bool ADJ>
-__global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_constant__ FineArgs args,
-                                                                  const __grid_constant__ Coef<T, M> cf) {
+__device__ __forceinline__ void stencil_smem_body(const FineArgs& args, const Coef<T, M>& cf, int field) {
     using Sh = ShShape<T, N, P, M>;
     constexpr int R = Sh::R, RH = Sh::RH, RW = Sh::RW, K = Sh::K;
     constexpr long long NN = (long long)N * N;
@@ -425,7 +496,6 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_c
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int rank = 0;
     if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
-    const int field = blockIdx.x / P;
     const Item it = item_of(args, field);
     const T* in = static_cast<const T*>(args.in) + it.fin * NN + (long long)rank * R * N;
     T* out = static_cast<T*>(args.out) + it.fout * NN + (long long)rank * R * N;
@@ -477,7 +547,7 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_c
     bool bad = false;
     // sums of the cells in fixed point, scaled to [-1, 1]-like sizes for the
     // adjoint, whose fields have no natural scale
-    double scale = 1.0;
+    double scale = 1.0, inv_scale = 1.0;
     if constexpr (MASS) {
         if constexpr (ADJ) {
             // power of two at the field's largest entry
@@ -496,7 +566,10 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_c
             for (int o = 16; o > 0; o >>= 1) e = max(e, (long long)__shfl_xor_sync(0xffffffffu, e, o));
             // 2^-exponent, exact; a zero or subnormal field keeps 1
             const int ex = int(e >> 52) - 1023;
-            if (ex > -1000 && ex < 1000) scale = __longlong_as_double((long long)(1023 - ex) << 52);
+            if (ex > -1000 && ex < 1000) {
+                scale = __longlong_as_double((long long)(1023 - ex) << 52);
+                inv_scale = __longlong_as_double((long long)(1023 + ex) << 52);
+            }
         } else {
             long long hi = 0, lo = 0;
 #pragma unroll
@@ -507,7 +580,7 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_c
             publish(hi, lo, bad, 1);
             cl_arrive<P>();
             cl_wait<P>();
-            mean = collect(1) / double(NN);
+            mean = collect(1) * (args.a * cf.inv_sum);
         }
     }
 
@@ -533,7 +606,7 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_c
         cl_wait<P>();
         T shift = T(0);
         if constexpr (MASS) {
-            const double m = collect(buf) / (double(NN) * args.a * scale);
+            const double m = collect(buf) * cf.inv_sum * inv_scale;
             shift = T(ADJ ? m : mean - m);
         }
         // stages: w_k on rows -(M-1-k) .. R + (M-1-k)
@@ -578,30 +651,34 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_c
 }
 
 template <typename T, int N, int P, int M, bool MASS, bool ADJ>
+__global__ void __launch_bounds__(kShThreads) stencil_smem_kernel(const __grid_constant__ FineArgs args,
+                                                                  const __grid_constant__ Coef<T, M> cf) {
+    stencil_smem_body<T, N, P, M, MASS, ADJ>(args, cf, blockIdx.x / P);
+}
+
+template <typename T, int N, int P, int M, bool MASS>
+__global__ void __launch_bounds__(kShThreads) stencil_smem_pair_kernel(const __grid_constant__ FineArgs adj,
+                                                                       const __grid_constant__ FineArgs fwd,
+                                                                       const __grid_constant__ Coef<T, M> cf) {
+    const int f = blockIdx.x / P;
+    if (f < adj.num_fields) stencil_smem_body<T, N, P, M, MASS, true>(adj, cf, f);
+    else stencil_smem_body<T, N, P, M, MASS, false>(fwd, cf, f - adj.num_fields);
+}
+
+template <typename T, int N, int P, int M, bool MASS, bool ADJ>
 int launch_smem_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
     using Sh = ShShape<T, N, P, M>;
-    auto kern = stencil_smem_kernel<T, N, P, M, MASS, ADJ>;
     static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM)));
-        if (P > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        configured = true;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(args.num_fields) * P, 1, 1);
-    cfg.blockDim = dim3(kShThreads, 1, 1);
-    cfg.dynamicSmemBytes = Sh::SMEM;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = P;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = P > 1 ? 1 : 0;
-    ACPR_CUDA(cudaLaunchKernelEx(&cfg, kern, args, make_coef<T, M>(args.a, args.dt, poly)));
-    count_launch();
-    return AC_OK;
+    return launch_clusters(stencil_smem_kernel<T, N, P, M, MASS, ADJ>, &configured, P, unsigned(args.num_fields), kShThreads, Sh::SMEM, stream, args,
+                           make_coef<T, M>(args.a, args.dt, double(N) * N, poly));
+}
+
+template <typename T, int N, int P, int M, bool MASS>
+int launch_smem_pair(const FineArgs& adj, const FineArgs& fwd, const SolvePoly& poly, cudaStream_t stream) {
+    static bool configured = false;
+    return launch_clusters(stencil_smem_pair_kernel<T, N, P, M, MASS>, &configured, P,
+                           unsigned(adj.num_fields + fwd.num_fields), kShThreads, ShShape<T, N, P, M>::SMEM, stream, adj, fwd,
+                           make_coef<T, M>(adj.a, adj.dt, double(N) * N, poly));
 }
 
 template <typename T, int N, int P, int M>
@@ -628,6 +705,33 @@ int dispatch_smem(int n, const FineArgs& args, const SolvePoly& poly, cudaStream
     }
 }
 
+template <bool MASS>
+int dispatch_reg_pair(int n, const FineArgs& adj, const FineArgs& fwd, const SolvePoly& poly, cudaStream_t st) {
+    switch (n) {  // the splits for few fields
+        case 32: return launch_reg_pair<32, 8, 4, 1, 2, MASS>(adj, fwd, poly, st);
+        case 64: return launch_reg_pair<64, 4, 4, 4, 2, MASS>(adj, fwd, poly, st);
+        case 128: return launch_reg_pair<128, 4, 4, 8, 2, MASS>(adj, fwd, poly, st);
+        case 256: return launch_reg_pair<256, 4, 4, 16, 2, MASS>(adj, fwd, poly, st);
+        case 512: return launch_reg_pair<512, 8, 4, 16, 2, MASS>(adj, fwd, poly, st);
+        default: return AC_ERR_UNSUPPORTED;
+    }
+}
+template <int M, bool MASS>
+int dispatch_smem_pair(int n, const FineArgs& adj, const FineArgs& fwd, const SolvePoly& poly, cudaStream_t st) {
+    switch (n) {
+        case 32: return launch_smem_pair<double, 32, 4, M, MASS>(adj, fwd, poly, st);
+        case 64: return launch_smem_pair<double, 64, M <= 4 ? 16 : 8, M, MASS>(adj, fwd, poly, st);
+        case 128: return launch_smem_pair<double, 128, 16, M, MASS>(adj, fwd, poly, st);
+        case 256: return launch_smem_pair<double, 256, 16, M, MASS>(adj, fwd, poly, st);
+        default: return AC_ERR_UNSUPPORTED;
+    }
+}
+
+bool unaligned(const FineArgs& a) {
+    return (reinterpret_cast<uintptr_t>(a.in) | reinterpret_cast<uintptr_t>(a.out) | reinterpret_cast<uintptr_t>(a.states) |
+            reinterpret_cast<uintptr_t>(a.traj)) % 16;
+}
+
 }  // namespace
 
 template <>
@@ -635,9 +739,7 @@ int launch_stencil<float>(int n, const FineArgs& args, cudaStream_t stream, bool
     *taken = false;
     if (n < 32 || n > 512) return AC_OK;
     // rows move as vectors; callers that pass unaligned fields keep the Fourier kernels
-    if ((reinterpret_cast<uintptr_t>(args.in) | reinterpret_cast<uintptr_t>(args.out) |
-         reinterpret_cast<uintptr_t>(args.states) | reinterpret_cast<uintptr_t>(args.traj)) % 16)
-        return AC_OK;
+    if (unaligned(args)) return AC_OK;
     // degree 4 rows of 512 columns would need 262 KB of halo buffers
     const SolvePoly p = solve_poly(args.a, args.lam_scale, 2, AC_F32, 2, n == 512 ? 3 : 4);
     if (!p.degree) return AC_OK;
@@ -663,6 +765,19 @@ int launch_stencil<double>(int n, const FineArgs& args, cudaStream_t stream, boo
         case 5: return dispatch_smem<5>(n, args, p, stream);
         default: return dispatch_smem<6>(n, args, p, stream);
     }
+}
+
+int launch_stencil_pair(int n, int precision, const FineArgs& adj, const FineArgs& fwd, cudaStream_t stream, bool* taken) {
+    *taken = false;
+    const bool f32 = precision == AC_F32;
+    if (n < 32 || n > (f32 ? 512 : 256) || (f32 && (unaligned(adj) || unaligned(fwd)))) return AC_OK;
+    const SolvePoly p = solve_poly(adj.a, adj.lam_scale, 2, precision, f32 ? 2 : 4, f32 ? 2 : 5);
+    if (!p.degree) return AC_OK;
+    *taken = true;
+    if (f32) return adj.mass ? dispatch_reg_pair<true>(n, adj, fwd, p, stream) : dispatch_reg_pair<false>(n, adj, fwd, p, stream);
+    if (p.degree == 4)
+        return adj.mass ? dispatch_smem_pair<4, true>(n, adj, fwd, p, stream) : dispatch_smem_pair<4, false>(n, adj, fwd, p, stream);
+    return adj.mass ? dispatch_smem_pair<5, true>(n, adj, fwd, p, stream) : dispatch_smem_pair<5, false>(n, adj, fwd, p, stream);
 }
 
 }  // namespace acpr

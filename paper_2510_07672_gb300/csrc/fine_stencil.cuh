@@ -3,7 +3,9 @@
 #pragma once
 
 #include <cmath>
+#include <type_traits>
 
+#include "f32x2.cuh"
 #include "fine.cuh"
 
 namespace acpr {
@@ -15,10 +17,11 @@ struct Coef {
     T be0, b1;      // u' = r + be0 r + b1 T w_1
     T g[M];         // g[k], k = 0 .. M - 2: stage k, w = r + g[k] T (input)
     T a, dt;        // adjoint: lambda' = a mu + dt f'(u) (mu - mean)
+    double inv_sum;  // 1 / (a cells): sum of r -> mean of p(Lap) r (no division on the device: float64 is scarce)
 };
 
 template <typename T, int M>
-Coef<T, M> make_coef(double a, double dt, const SolvePoly& p) {
+Coef<T, M> make_coef(double a, double dt, double cells, const SolvePoly& p) {
     Coef<T, M> c{};
     c.kappa = T((a - 1.0) + dt);
     c.mdt = T(-dt);
@@ -31,46 +34,115 @@ Coef<T, M> make_coef(double a, double dt, const SolvePoly& p) {
     }
     c.a = T(a);
     c.dt = T(dt);
+    c.inv_sum = 1.0 / (a * cells);
     return c;
 }
 
-// A row in shared memory, a warp's lanes holding W adjacent columns each.
+// A lane's W adjacent columns of a row: pairs (column j, column j + W / 2) for
+// even W, so that a column's neighbours are the adjacent pairs but at the ends
+// and one paired instruction serves two cells; single columns for odd W.
 template <int W>
-__device__ __forceinline__ void row_store(float* dst, const float (&x)[W], int lane) {
-    // chunks of VW floats, chunk-major: lanes store consecutive vectors
-    constexpr int VW = W % 4 == 0 ? 4 : W % 2 == 0 ? 2 : 1;
+struct Lane {
+    static constexpr bool PAIR = W % 2 == 0;
+    static constexpr int E = PAIR ? W / 2 : W;
+    using V = std::conditional_t<PAIR, f32x2, float>;
+};
+template <int W>
+using LaneV = typename Lane<W>::V;
+
+__device__ __forceinline__ float vadd(float a, float b) { return a + b; }
+__device__ __forceinline__ f32x2 vadd(f32x2 a, f32x2 b) { return f2_add(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return a * b; }
+__device__ __forceinline__ f32x2 vmul(f32x2 a, f32x2 b) { return f2_mul(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ f32x2 vfma(f32x2 a, f32x2 b, f32x2 c) { return f2_fma(a, b, c); }
+template <typename V>
+__device__ __forceinline__ V vset(float a) {
+    if constexpr (sizeof(V) == 8) return f2(a, a);
+    else return a;
+}
+__device__ __forceinline__ float lo_of(f32x2 v) {
+    float a, b;
+    f2split(v, a, b);
+    return a;
+}
+__device__ __forceinline__ float hi_of(f32x2 v) {
+    float a, b;
+    f2split(v, a, b);
+    return b;
+}
+
+// Columns in order <-> the lane's elements.
+template <int W>
+__device__ __forceinline__ void to_lane(const float (&c)[W], LaneV<W> (&x)[Lane<W>::E]) {
 #pragma unroll
-    for (int v = 0; v < W / VW; ++v) {
-        float* p = dst + v * 32 * VW + lane * VW;
-        if constexpr (VW == 4) *reinterpret_cast<float4*>(p) = make_float4(x[4 * v], x[4 * v + 1], x[4 * v + 2], x[4 * v + 3]);
-        else if constexpr (VW == 2) *reinterpret_cast<float2*>(p) = make_float2(x[2 * v], x[2 * v + 1]);
-        else *p = x[v];
+    for (int e = 0; e < Lane<W>::E; ++e) {
+        if constexpr (Lane<W>::PAIR) x[e] = f2(c[e], c[e + W / 2]);
+        else x[e] = c[e];
     }
 }
 template <int W>
-__device__ __forceinline__ void row_load(const float* src, float (&x)[W], int lane) {
-    constexpr int VW = W % 4 == 0 ? 4 : W % 2 == 0 ? 2 : 1;
+__device__ __forceinline__ void from_lane(const LaneV<W> (&x)[Lane<W>::E], float (&c)[W]) {
 #pragma unroll
-    for (int v = 0; v < W / VW; ++v) {
-        const float* p = src + v * 32 * VW + lane * VW;
-        if constexpr (VW == 4) {
-            const float4 q = *reinterpret_cast<const float4*>(p);
-            x[4 * v] = q.x; x[4 * v + 1] = q.y; x[4 * v + 2] = q.z; x[4 * v + 3] = q.w;
-        } else if constexpr (VW == 2) {
-            const float2 q = *reinterpret_cast<const float2*>(p);
-            x[2 * v] = q.x; x[2 * v + 1] = q.y;
-        } else {
-            x[v] = *p;
+    for (int e = 0; e < Lane<W>::E; ++e) {
+        if constexpr (Lane<W>::PAIR) f2split(x[e], c[e], c[e + W / 2]);
+        else c[e] = x[e];
+    }
+}
+
+// A warp's row in shared memory, each lane's elements where only that lane
+// looks for them: vectors of up to 16 bytes, consecutive over the lanes.
+template <int W>
+__device__ __forceinline__ void row_store(float* dst, const LaneV<W> (&x)[Lane<W>::E], int lane) {
+    constexpr int E = Lane<W>::E;
+    if constexpr (Lane<W>::PAIR && E % 2 == 0) {
+#pragma unroll
+        for (int v = 0; v < E / 2; ++v)
+            reinterpret_cast<ulonglong2*>(dst)[v * 32 + lane] = make_ulonglong2(x[2 * v], x[2 * v + 1]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) reinterpret_cast<LaneV<W>*>(dst)[e * 32 + lane] = x[e];
+    }
+}
+template <int W>
+__device__ __forceinline__ void row_load(const float* src, LaneV<W> (&x)[Lane<W>::E], int lane) {
+    constexpr int E = Lane<W>::E;
+    if constexpr (Lane<W>::PAIR && E % 2 == 0) {
+#pragma unroll
+        for (int v = 0; v < E / 2; ++v) {
+            const ulonglong2 q = reinterpret_cast<const ulonglong2*>(src)[v * 32 + lane];
+            x[2 * v] = q.x;
+            x[2 * v + 1] = q.y;
         }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) x[e] = reinterpret_cast<const LaneV<W>*>(src)[e * 32 + lane];
     }
 }
-// Left plus right neighbour of every column of a row.
+
+// Left plus right neighbour of every column of a row; the neighbours of the
+// run's ends are the next lanes' (the ring of lanes is the periodic row).
 template <int W>
-__device__ __forceinline__ void hsum(const float (&x)[W], float (&h)[W], int lane) {
-    const float l = __shfl_sync(0xffffffffu, x[W - 1], (lane + 31) & 31);
-    const float r = __shfl_sync(0xffffffffu, x[0], (lane + 1) & 31);
+__device__ __forceinline__ void hsum(const LaneV<W> (&x)[Lane<W>::E], LaneV<W> (&h)[Lane<W>::E], int lane) {
+    constexpr int E = Lane<W>::E;
+    if constexpr (Lane<W>::PAIR) {
+        const float l = __shfl_sync(0xffffffffu, hi_of(x[E - 1]), (lane + 31) & 31);
+        const float r = __shfl_sync(0xffffffffu, lo_of(x[0]), (lane + 1) & 31);
+        const f32x2 lv = f2(l, lo_of(x[E - 1])), rv = f2(hi_of(x[0]), r);
 #pragma unroll
-    for (int c = 0; c < W; ++c) h[c] = (c ? x[c - 1] : l) + (c + 1 < W ? x[c + 1] : r);
+        for (int e = 0; e < E; ++e) h[e] = f2_add(e ? x[e - 1] : lv, e + 1 < E ? x[e + 1] : rv);
+    } else {
+        const float l = __shfl_sync(0xffffffffu, x[E - 1], (lane + 31) & 31);
+        const float r = __shfl_sync(0xffffffffu, x[0], (lane + 1) & 31);
+#pragma unroll
+        for (int e = 0; e < E; ++e) h[e] = (e ? x[e - 1] : l) + (e + 1 < E ? x[e + 1] : r);
+    }
+}
+
+// r = u + u (kappa + mdt u^2)
+template <typename V>
+__device__ __forceinline__ V rhs(V v, V mdt, V kappa) {
+    return vfma(v, vfma(mdt, vmul(v, v), kappa), v);
 }
 
 // r <- p(Lap) r for the warp's H rows; halo(y, x) gives row y of r outside
@@ -80,16 +152,21 @@ __device__ __forceinline__ void hsum(const float (&x)[W], float (&h)[W], int lan
 // SHIFT: plus `shift`, added to the small term: r + be0 r lies on the coarse
 // grid of its binade, where a shift below half a unit would be rounded away in
 // all of its cells alike.
-template <int W, int H, int M, bool SHIFT, class Halo>
-__device__ __forceinline__ void apply_poly(float (&r)[H][W], const Coef<float, M>& cf, int lane, float shift,
-                                           Halo halo) {
-    float s[M][W], p[M][W];
+// It is asked for (shift()) when the first row is complete.
+template <int W, int H, int M, bool SHIFT, class Halo, class Shift>
+__device__ __forceinline__ void apply_poly(LaneV<W> (&r)[H][Lane<W>::E], const Coef<float, M>& cf, int lane,
+                                           Halo halo, Shift shift) {
+    using V = LaneV<W>;
+    constexpr int E = Lane<W>::E;
+    V s[M][E], p[M][E];
+    const V be0 = vset<V>(cf.be0), b1 = vset<V>(cf.b1);
+    V sh = vset<V>(0.f);
 #pragma unroll
     for (int y = -M; y < H + M; ++y) {
-        float x[W];
+        V x[E];
         if (y >= 0 && y < H) {
 #pragma unroll
-            for (int c = 0; c < W; ++c) x[c] = r[y][c];
+            for (int c = 0; c < E; ++c) x[c] = r[y][c];
         } else {
             halo(y, x);
         }
@@ -97,42 +174,44 @@ __device__ __forceinline__ void apply_poly(float (&r)[H][W], const Coef<float, M
         for (int k = 0; k < M; ++k) {
             const int yk = y - k, first = k - M;  // x is row yk of the stage's input, whose first row is `first`
             if (yk < first) break;
-            float nx[W];
+            V nx[E];
             const bool emit = yk >= first + 2;
             if (emit) {
                 if (k < M - 1) {
-                    float rr[W];
+                    V rr[E];
                     const int yr = yk - 1;
                     if (k == 0) {
 #pragma unroll
-                        for (int c = 0; c < W; ++c) rr[c] = p[0][c];
+                        for (int c = 0; c < E; ++c) rr[c] = p[0][c];
                     } else if (yr >= 0 && yr < H) {
 #pragma unroll
-                        for (int c = 0; c < W; ++c) rr[c] = r[yr][c];
+                        for (int c = 0; c < E; ++c) rr[c] = r[yr][c];
                     } else {
                         halo(yr, rr);
                     }
+                    const V g = vset<V>(cf.g[k]);
 #pragma unroll
-                    for (int c = 0; c < W; ++c) nx[c] = fmaf(cf.g[k], s[k][c] + x[c], rr[c]);
+                    for (int c = 0; c < E; ++c) nx[c] = vfma(g, vadd(s[k][c], x[c]), rr[c]);
                 } else {
+                    if (SHIFT && yk == 1) sh = vset<V>(shift());
 #pragma unroll
-                    for (int c = 0; c < W; ++c) {
-                        const float t0 = fmaf(cf.be0, r[yk - 1][c], r[yk - 1][c]);
-                        r[yk - 1][c] = SHIFT ? t0 + fmaf(cf.b1, s[k][c] + x[c], shift) : fmaf(cf.b1, s[k][c] + x[c], t0);
+                    for (int c = 0; c < E; ++c) {
+                        const V t0 = vfma(be0, r[yk - 1][c], r[yk - 1][c]), t = vadd(s[k][c], x[c]);
+                        r[yk - 1][c] = SHIFT ? vadd(t0, vfma(b1, t, sh)) : vfma(b1, t, t0);
                     }
                 }
             }
             if (yk > first && yk < H + M - k - 1) {
-                float h[W];
+                V h[E];
                 hsum<W>(x, h, lane);
 #pragma unroll
-                for (int c = 0; c < W; ++c) s[k][c] = h[c] + p[k][c];
+                for (int c = 0; c < E; ++c) s[k][c] = vadd(h[c], p[k][c]);
             }
 #pragma unroll
-            for (int c = 0; c < W; ++c) p[k][c] = x[c];
+            for (int c = 0; c < E; ++c) p[k][c] = x[c];
             if (!emit || k == M - 1) break;
 #pragma unroll
-            for (int c = 0; c < W; ++c) x[c] = nx[c];
+            for (int c = 0; c < E; ++c) x[c] = nx[c];
         }
     }
 }
@@ -149,15 +228,17 @@ __device__ __forceinline__ long long warp_sum_s64(long long v) {
 
 // Sum of the two rows' cells of a lane (the same order under every split).
 template <int W>
-__device__ __forceinline__ float pair_sum(const float (&x)[W], const float (&y)[W]) {
-    float t[W];
+__device__ __forceinline__ float pair_sum(const LaneV<W> (&x)[Lane<W>::E], const LaneV<W> (&y)[Lane<W>::E]) {
+    constexpr int E = Lane<W>::E;
+    LaneV<W> t[E];
 #pragma unroll
-    for (int c = 0; c < W; ++c) t[c] = x[c] + y[c];
+    for (int c = 0; c < E; ++c) t[c] = vadd(x[c], y[c]);
 #pragma unroll
-    for (int o = W / 2; o > 0; o /= 2)
+    for (int o = E / 2; o > 0; o /= 2)
 #pragma unroll
-        for (int c = 0; c < o; ++c) t[c] += t[c + o];
-    return t[0];
+        for (int c = 0; c < o; ++c) t[c] = vadd(t[c], t[c + o]);
+    if constexpr (Lane<W>::PAIR) return lo_of(t[0]) + hi_of(t[0]);
+    else return t[0];
 }
 
 }  // namespace acpr
