@@ -12,6 +12,8 @@
 
 namespace acpr {
 
+int fine_run_adjoint_beside(const ac_params* p, int adj_steps, const void* states, const void* lam, void* lam_out,
+                            int fwd_steps, const void* u, void* u_out, void* traj, cudaStream_t stream, bool* taken);
 int fine_run(const ac_params* p, int groups, int per_group, int steps, const void* in, long long in_gs,
              long long in_off, void* out, long long out_gs, long long out_off, const int* map, int adjoint,
              const void* states, void* traj, cudaStream_t stream, void* big_ws = nullptr, size_t big_ws_bytes = 0);
@@ -97,10 +99,12 @@ int energy_grad(const ac_params* p, int fields, const void* u, void* g, cudaStre
     return AC_OK;
 }
 
-static size_t grad_ws_bytes(const ac_params* p, int steps, int K) {
+// Checkpoints, `segments` segments' states (two: one is recomputed while the
+// adjoint runs through the other) and two gradients.
+static size_t grad_ws_bytes(const ac_params* p, int steps, int K, int segments) {
     const size_t fb = elem_size(p->precision) * size_t(p->n) * p->n;
     const int nseg = (steps + K - 1) / K;
-    return fb * (size_t(nseg + 1) + size_t(K + 1) + 2);
+    return fb * (size_t(nseg + 1) + size_t(segments) * size_t(K + 1) + 2);
 }
 
 int energy_gradient_ic(const ac_params* p, int steps, int K, const void* u0, void* grad, void* ws, size_t ws_bytes,
@@ -108,29 +112,51 @@ int energy_gradient_ic(const ac_params* p, int steps, int K, const void* u0, voi
     int rc = check_p(p);
     if (rc) return rc;
     ACPR_CHECK_ARG(steps >= 0 && K >= 1 && u0 && grad && ws, "bad gradient arguments");
-    ACPR_CHECK_ARG(ws_bytes >= grad_ws_bytes(p, steps, K), "workspace too small: need %zu bytes",
-                   grad_ws_bytes(p, steps, K));
+    // (a workspace with room for one segment still runs, without the overlap)
+    ACPR_CHECK_ARG(ws_bytes >= grad_ws_bytes(p, steps, K, 1), "workspace too small: need %zu bytes",
+                   grad_ws_bytes(p, steps, K, 1));
+    const int segments = ws_bytes >= grad_ws_bytes(p, steps, K, 2) ? 2 : 1;
     const size_t fb = elem_size(p->precision) * size_t(p->n) * p->n;
     const int nseg = (steps + K - 1) / K;
     char* cp = static_cast<char*>(ws);                 // checkpoints c_0 .. c_nseg
-    char* traj = cp + fb * (nseg + 1);                 // one segment's states
-    char* lam[2] = {traj + fb * (K + 1), traj + fb * (K + 2)};
+    char* traj[2];                                     // one or two segments' states
+    traj[0] = cp + fb * (nseg + 1);
+    traj[1] = traj[0] + (segments - 1) * fb * (K + 1);
+    char* lam[2] = {traj[1] + fb * (K + 1), traj[1] + fb * (K + 2)};
+    auto len_of = [&](int i) { return (i + 1) * K <= steps ? K : steps - i * K; };
+    auto states = [&](int i, char* to) {
+        return fine_run(p, 1, 1, len_of(i), cp + fb * i, 0, 0, to + fb * len_of(i), 0, 0, nullptr, 0, nullptr, to, st);
+    };
     ACPR_CUDA(cudaMemcpyAsync(cp, u0, fb, cudaMemcpyDeviceToDevice, st));
-    for (int i = 0; i < nseg; ++i) {
-        const int len = (i + 1) * K <= steps ? K : steps - i * K;
-        rc = fine_run(p, 1, 1, len, cp + fb * i, 0, 0, cp + fb * (i + 1), 0, 0, nullptr, 0, nullptr, nullptr, st);
+    for (int i = 0; i + 1 < nseg; ++i) {
+        rc = fine_run(p, 1, 1, len_of(i), cp + fb * i, 0, 0, cp + fb * (i + 1), 0, 0, nullptr, 0, nullptr, nullptr, st);
         if (rc) return rc;
     }
-    rc = energy_grad(p, 1, cp + fb * nseg, lam[0], st);
+    // the last segment's states are kept on the way forward
+    const char* last = cp;
+    if (nseg > 0) {
+        if ((rc = states(nseg - 1, traj[0]))) return rc;
+        last = traj[0] + fb * len_of(nseg - 1);
+    }
+    rc = energy_grad(p, 1, last, lam[0], st);
     if (rc) return rc;
-    int cur = 0;
+    int cur = 0, have = 0;  // traj[have]: the states of segment i
     for (int i = nseg - 1; i >= 0; --i) {
-        const int len = (i + 1) * K <= steps ? K : steps - i * K;
-        // recompute the segment's states u_{iK} .. u_{iK+len} (traj[len] is not needed)
-        rc = fine_run(p, 1, 1, len, cp + fb * i, 0, 0, traj + fb * len, 0, 0, nullptr, 0, nullptr, traj, st);
-        if (rc) return rc;
-        rc = fine_run(p, 1, 1, len, lam[cur], 0, 0, lam[cur ^ 1], 0, 0, nullptr, 1, traj, nullptr, st);
-        if (rc) return rc;
+        // the adjoint through segment i, beside it the states of segment i - 1
+        // from its checkpoint (one field's steps fill 16 SMs at most)
+        char* next = traj[segments == 2 ? have ^ 1 : 0];
+        bool beside = false;
+        if (i > 0 && segments == 2) {
+            rc = fine_run_adjoint_beside(p, len_of(i), traj[have], lam[cur], lam[cur ^ 1], len_of(i - 1), cp + fb * (i - 1),
+                                         next + fb * len_of(i - 1), next, st, &beside);
+            if (rc) return rc;
+        }
+        if (!beside) {
+            rc = fine_run(p, 1, 1, len_of(i), lam[cur], 0, 0, lam[cur ^ 1], 0, 0, nullptr, 1, traj[have], nullptr, st);
+            if (rc) return rc;
+            if (i > 0 && (rc = states(i - 1, next))) return rc;
+        }
+        if (segments == 2) have ^= 1;
         cur ^= 1;
     }
     ACPR_CUDA(cudaMemcpyAsync(grad, lam[cur], fb, cudaMemcpyDeviceToDevice, st));
@@ -151,7 +177,7 @@ extern "C" int ac_energy_grad(const ac_params* params, int num_fields, const voi
 
 extern "C" size_t ac_energy_gradient_workspace(const ac_params* params, int steps, int checkpoint_every) {
     if (!params || steps < 0 || checkpoint_every < 1 || params->n < 2) return 0;
-    return acpr::grad_ws_bytes(params, steps, checkpoint_every);
+    return acpr::grad_ws_bytes(params, steps, checkpoint_every, 2);
 }
 
 extern "C" int ac_energy_gradient_ic(const ac_params* params, int steps, int checkpoint_every, const void* u0,

@@ -638,6 +638,35 @@ static int dispatch_fine(int n, const FineArgs& args, cudaStream_t stream) {
     return v[idx].launch(args, stream);
 }
 
+// One field's adjoint steps through `states` (lam -> lam_out) and another's
+// forward steps (u -> u_out, every state into traj) in one launch; *taken =
+// false and nothing launched where only separate launches are built.
+int fine_run_adjoint_beside(const ac_params* p, int adj_steps, const void* states, const void* lam, void* lam_out,
+                            int fwd_steps, const void* u, void* u_out, void* traj, cudaStream_t stream, bool* taken) {
+    *taken = false;
+    int count = 0;
+    const FineVariant* v = is_pow2(p->n) && p->n <= 512 ? pick_variant(p->n, p->precision, &count) : nullptr;
+    if (!v || !count || v[g_variant[p->precision][ilog2(p->n)]].launch) return AC_OK;
+    FineArgs a{};
+    a.num_fields = a.per_group = 1;
+    a.mass = p->variant == AC_MASS_CONSERVING;
+    a.a = 1.0 + p->S * p->dt;
+    a.dt = p->dt;
+    const double h = p->length / p->n;
+    a.lam_scale = p->dt * p->eps * p->eps * 4.0 / (h * h);
+    FineArgs b = a;
+    a.in = lam;
+    a.out = lam_out;
+    a.steps = adj_steps;
+    a.adjoint = 1;
+    a.states = states;
+    b.in = u;
+    b.out = u_out;
+    b.steps = fwd_steps;
+    b.traj = traj;
+    return launch_stencil_pair(p->n, p->precision, a, b, stream, taken);
+}
+
 // Device-side timeout flag of the fine kernels' bounded exchange waits:
 // AC_ERR_TIMEOUT (and the flag cleared) if one gave up since the last call.
 // Synchronises the stream.

@@ -161,3 +161,26 @@ def test_cube_stream(n, count, steps, variant):
     v = u.clone()
     G.ac_fine3d_propagate(fp, steps, v, v)
     assert torch.equal(v, out)
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("n,prec,steps,every", [(32, F32, 7, 3), (128, F32, 9, 4), (64, F64, 11, 4), (128, F64, 6, 6), (32, F64, 5, 8)])
+def test_energy_gradient_with_and_without_the_overlap(n, prec, steps, every, variant):
+    """The states of a segment recomputed beside the adjoint of the next one:
+    the same bits as one after the other (a workspace with one segment's room)."""
+    import ctypes
+    from paper_2510_07672_gb300 import abi
+    fp = params(n, prec, variant, 1e-3)
+    u = fields(n, 1, prec)[0]
+    got = G.ac_energy_gradient_ic(fp, steps, u, checkpoint_every=every)
+    p = fp.c()
+    full = G.load().ac_energy_gradient_workspace(ctypes.byref(p), steps, every)
+    nbytes = full - u.numel() * u.element_size() * (every + 1)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    ref = torch.empty_like(u)
+    args = (ctypes.byref(p), steps, every, u.data_ptr(), ref.data_ptr(), ws.data_ptr())
+    stream = torch.cuda.current_stream().cuda_stream
+    assert G.load().ac_energy_gradient_ic(*args, nbytes, stream) == abi.AC_OK
+    torch.cuda.synchronize()
+    assert torch.equal(got, ref)
+    assert G.load().ac_energy_gradient_ic(*args, nbytes - 1, stream) == -1
