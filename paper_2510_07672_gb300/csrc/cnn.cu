@@ -22,7 +22,6 @@ namespace acpr {
 __device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
 // ---------------------------------------------------------------- float64 --
-// One thread per output pixel, all output channels.
 // Batch entry b of the input field starts at in + fi(b) * in_bs with
 // fi(b) = in_map ? in_map[b] : b; the output field at out + fo(b) * out_bs with
 // fo(b) = out_map ? out_map[b] : b.  Hidden activations are compact
@@ -37,12 +36,29 @@ struct BatchIO {
 
 __device__ __forceinline__ long long bsel(const int* map, int b) { return map ? map[b] : b; }
 
-template <int COUT_MAX>
-__global__ void conv_f64_kernel(const double* __restrict__ in, double* __restrict__ out,
-                                const double* __restrict__ W, const double* __restrict__ bias,
-                                int batch, int n, int cin, int cout, int act, int apply_act,
-                                const double* __restrict__ resid, BatchIO io) {
-    const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// A thread computes G output channels of one pixel, blockIdx.y picks which; the
+// block's weights are staged in shared memory.  Each output is its own chain
+// (bias, then channels and taps in order), so G does not change the bits.
+// Bound: FP64 issue (two lanes per SM and cycle), so the work has to reach every
+// SM: a 64^2 field is 64 blocks of pixels, and 8 blocks of 2 channels each make
+// 512 (one thread per pixel with all 16 channels: 84 us per layer of one field;
+// split 22 us).
+constexpr int kF64Threads = 64;
+
+template <int G>
+__global__ void __launch_bounds__(kF64Threads) conv_f64_kernel(const double* __restrict__ in, double* __restrict__ out,
+                                                               const double* __restrict__ W,
+                                                               const double* __restrict__ bias, int batch, int n, int cin,
+                                                               int cout, int act, int apply_act,
+                                                               const double* __restrict__ resid, BatchIO io) {
+    extern __shared__ double ws[];  // [cin][G][9]
+    const int o0 = blockIdx.y * G;
+    for (int i = threadIdx.x; i < G * cin * 9; i += kF64Threads) {
+        const int g = i / (cin * 9), r = i % (cin * 9);
+        ws[((r / 9) * G + g) * 9 + r % 9] = o0 + g < cout ? W[(long long)(o0 + g) * cin * 9 + r] : 0.0;
+    }
+    __syncthreads();
+    const long long pix = (long long)blockIdx.x * kF64Threads + threadIdx.x;
     const long long nn = (long long)n * n;
     if (pix >= nn * batch) return;
     const int b = int(pix / nn);
@@ -50,29 +66,44 @@ __global__ void conv_f64_kernel(const double* __restrict__ in, double* __restric
     const long long fi = bsel(io.in_map, b), fo = bsel(io.out_map, b);
     const double* inb = io.in_mapped ? in + fi * io.in_bs : in + (long long)b * cin * nn;
     double* outb = io.out_mapped ? out + fo * io.out_bs : out + (long long)b * cout * nn;
-    double acc[COUT_MAX];
-    for (int o = 0; o < cout; ++o) acc[o] = bias[o];
+    int off[9];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) off[t] = wrap(y + t / 3 - 1, n) * n + wrap(x + t % 3 - 1, n);
+    double acc[G];
+#pragma unroll
+    for (int g = 0; g < G; ++g) acc[g] = o0 + g < cout ? bias[o0 + g] : 0.0;
     for (int c = 0; c < cin; ++c) {
         const double* plane = inb + (long long)c * nn;
+        const double* w = ws + c * G * 9;
         double v[9];
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+        for (int t = 0; t < 9; ++t) v[t] = plane[off[t]];
 #pragma unroll
-            for (int e = 0; e < 3; ++e) v[a * 3 + e] = plane[(long long)wrap(y + a - 1, n) * n + wrap(x + e - 1, n)];
-        for (int o = 0; o < cout; ++o) {
-            const double* w = W + ((long long)o * cin + c) * 9;
-            double s = acc[o];
+        for (int t = 0; t < 9; ++t)
 #pragma unroll
-            for (int t = 0; t < 9; ++t) s += w[t] * v[t];
-            acc[o] = s;
-        }
+            for (int g = 0; g < G; ++g) acc[g] += w[g * 9 + t] * v[t];
     }
-    for (int o = 0; o < cout; ++o) {
-        double z = acc[o];
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+        if (o0 + g >= cout) break;
+        double z = acc[g];
         if (apply_act) z = act_apply<double>(act, z);
         if (resid) z += resid[fi * io.in_bs + (long long)y * n + x];
-        outb[(long long)o * nn + (long long)y * n + x] = z;
+        outb[(long long)(o0 + g) * nn + (long long)y * n + x] = z;
     }
+}
+
+template <int G>
+static int launch_conv_f64(const double* in, double* out, const double* W, const double* bias, int batch, int n, int cin,
+                           int cout, int act, int apply_act, const double* resid, const BatchIO& io, cudaStream_t st) {
+    const long long pixels = (long long)n * n * batch;
+    const size_t smem = sizeof(double) * G * cin * 9;
+    if (smem > 48 * 1024)
+        ACPR_CUDA(cudaFuncSetAttribute(conv_f64_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    const dim3 grid(unsigned((pixels + kF64Threads - 1) / kF64Threads), unsigned((cout + G - 1) / G));
+    conv_f64_kernel<G><<<grid, kF64Threads, smem, st>>>(in, out, W, bias, batch, n, cin, cout, act, apply_act, resid, io);
+    ACPR_LAUNCH_CHECK();
+    return AC_OK;
 }
 
 // ------------------------------------------------------------ bf16 / f32 --
@@ -497,8 +528,6 @@ static int run_f32(const cnn_desc* d, int n, int batch, const float* u, float* o
 static int run_f64(const cnn_desc* d, int n, int batch, const double* u, double* out, const BatchIO& io,
                    cudaStream_t st) {
     const long long pixels = (long long)n * n * batch;
-    const int threads = 128;
-    const unsigned blocks = unsigned((pixels + threads - 1) / threads);
     const double* W = static_cast<const double*>(d->w);
     const double* Bv = static_cast<const double*>(d->b);
     const size_t act_elems = size_t(batch) * d->channels * n * n;
@@ -514,9 +543,17 @@ static int run_f64(const cnn_desc* d, int n, int batch, const double* u, double*
         BatchIO lio = io;
         lio.in_mapped = l == 0;
         lio.out_mapped = last;
-        conv_f64_kernel<64><<<blocks, threads, 0, st>>>(cur, dst, W + woff, Bv + boff, batch, n, cin, cout,
-                                                        d->act, last ? 0 : 1, (last && d->residual) ? u : nullptr, lio);
-        ACPR_LAUNCH_CHECK();
+        const double* rs = (last && d->residual) ? u : nullptr;
+        // four channels a thread share the loads once the batch fills the SMs
+        // without the split (152 SMs x 32 warps); two spread a small one
+        int rc;
+        if (cout == 1)
+            rc = launch_conv_f64<1>(cur, dst, W + woff, Bv + boff, batch, n, cin, cout, d->act, !last, rs, lio, st);
+        else if (pixels * cout / 4 < 152LL * 1024)
+            rc = launch_conv_f64<2>(cur, dst, W + woff, Bv + boff, batch, n, cin, cout, d->act, !last, rs, lio, st);
+        else
+            rc = launch_conv_f64<4>(cur, dst, W + woff, Bv + boff, batch, n, cin, cout, d->act, !last, rs, lio, st);
+        if (rc) return rc;
         cur = dst;
         woff += size_t(cin) * cout * 9;
         boff += cout;
