@@ -249,23 +249,19 @@ __global__ void __launch_bounds__(kThreads) post_kernel(T* __restrict__ out, Acn
                                                         int limiter, double lo, double hi, T* __restrict__ s_save,
                                                         int lg, int per_block) {
     const int b = blockIdx.y;
-    __shared__ double shift;
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        if (mass_fix)
-            for (int k = 0; k < parts; ++k) t += part[(long long)b * parts + k];
-        shift = -t / double(1LL << (2 * lg));
-    }
-    __syncthreads();
+    __shared__ double red[kThreads / 32];
+    const double sum = mass_fix ? acnn_sum_parts(part + (long long)b * parts, parts, 1, red) : 0.0;
+    const AcnnShift<T> shift(-sum * (1.0 / double(1LL << (2 * lg))));
+    const T tlo = T(lo), thi = T(hi);
     T* ob = out + acnn_sel(io.out_map, b) * io.out_bs;
     const long long nn = 1LL << (2 * lg);
     const long long first = (long long)blockIdx.x * per_block;
     for (int k = threadIdx.x; k < per_block; k += kThreads) {
         const long long q = first + k;
-        double v = double(ob[q]) + shift;
-        if (s_save) s_save[b * nn + q] = T(v);
-        if (limiter) v = v < lo ? lo : (v > hi ? hi : v);
-        ob[q] = T(v);
+        T v = mass_fix ? shift.add(ob[q]) : ob[q];
+        if (s_save) s_save[b * nn + q] = v;
+        if (limiter) v = v < tlo ? tlo : (v > thi ? thi : v);
+        ob[q] = v;
     }
 }
 
@@ -314,18 +310,11 @@ __global__ void __launch_bounds__(kThreads) loss_resid_kernel(const T* __restric
                                                               double* __restrict__ rpart, int parts, int lg,
                                                               double half_dt, double e2_h2, int mass) {
     __shared__ double red[kThreads / 32];
-    __shared__ double gsum;
     const long long nn = 1LL << (2 * lg);
     const long long first = (long long)blockIdx.x * kThreads * kLossPix;
     const long long b = first >> (2 * lg);
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        if (mass)
-            for (int k = 0; k < parts; ++k) t += fpart[2 * (b * parts + k)] + fpart[2 * (b * parts + k) + 1];
-        gsum = t / double(nn);
-    }
-    __syncthreads();
-    const T g = T(gsum);
+    const double gsum = mass ? acnn_sum_parts(fpart + 2 * b * parts, 2 * parts, 1, red) : 0.0;
+    const T g = T(gsum * (1.0 / double(nn)));  // nn is a power of two: exact
     const int n = 1 << lg, mask = n - 1;
     const T* a0 = U0 + b * nn;
     const T* a1 = U1 + b * nn;
@@ -359,23 +348,17 @@ __global__ void __launch_bounds__(kThreads) loss_grad_kernel(const T* __restrict
                                                              int total_blocks, T* __restrict__ grad,
                                                              double* __restrict__ loss, int lg, double half_dt,
                                                              double e2_h2, int mass, double scale) {
-    __shared__ double rmean;
+    __shared__ double red[kThreads / 32];
     const long long nn = 1LL << (2 * lg);
     const long long first = (long long)blockIdx.x * kThreads * kLossPix;
     const long long b = first >> (2 * lg);
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < parts; ++k) t += rpart[2 * (b * parts + k)];
-        rmean = t / double(nn);
-        if (blockIdx.x == 0) {
-            double l = 0.0;
-            for (int k = 0; k < total_blocks; ++k) l += rpart[2 * k + 1];
-            *loss = l * scale * 0.5;
-        }
+    const double rsum = mass ? acnn_sum_parts(rpart + 2 * b * parts, parts, 2, red) : 0.0;
+    if (blockIdx.x == 0) {
+        const double l = acnn_sum_parts(rpart + 1, total_blocks, 2, red);
+        if (threadIdx.x == 0) *loss = l * scale * 0.5;
     }
-    __syncthreads();
     if (!grad) return;
-    const T rm = T(rmean);
+    const T rm = T(rsum * (1.0 / double(nn)));
     const int n = 1 << lg, mask = n - 1;
     const T* rb = r + b * nn;
     for (int k = 0; k < kLossPix; ++k) {

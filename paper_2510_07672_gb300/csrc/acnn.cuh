@@ -25,6 +25,44 @@ __device__ __forceinline__ long long acnn_sel(const int* map, int b) { return ma
 __device__ __forceinline__ float acnn_tanh(float x) { return 1.0f - __fdividef(2.0f, 1.0f + __expf(2.0f * x)); }
 __device__ __forceinline__ double acnn_tanh(double x) { return tanh(x); }
 
+// Sum of count float64 values p[0], p[stride], ..., on every thread of a block
+// of 8 warps, in an order fixed by count alone.  red: 8 shared values.  (One
+// thread adding them in turn waits out a memory latency per value: 14 us for
+// the 64 partials of a 256^2 field.)
+__device__ __forceinline__ double acnn_sum_parts(const double* __restrict__ p, int count, int stride, double* red) {
+    double s = 0.0;
+    for (int k = threadIdx.x; k < count; k += 256) s += p[(long long)k * stride];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += red[w];
+    __syncthreads();  // the caller may reuse `red`
+    return t;
+}
+
+// x + shift rounded once.  float32: shift = hi + lo and the exact error of
+// x + hi (TwoSum, Knuth) in place of float64 instructions, scarce on this GPU.
+template <typename T>
+struct AcnnShift {
+    double v;
+    __device__ explicit AcnnShift(double s) : v(s) {}
+    __device__ T add(T x) const { return T(double(x) + v); }
+};
+template <>
+struct AcnnShift<float> {
+    float hi, lo;
+    __device__ explicit AcnnShift(double s) : hi(float(s)), lo(float(s - double(float(s)))) {}
+    __device__ float add(float x) const {
+        const float s = __fadd_rn(x, hi), bb = __fsub_rn(s, x);
+        const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(hi, bb));
+        return __fadd_rn(s, __fadd_rn(e, lo));
+    }
+};
+
 inline int acnn_convs(int blocks) { return 2 + 2 * blocks; }
 
 inline void acnn_dims(int C, int blocks, int l, int* cin, int* cout) {
