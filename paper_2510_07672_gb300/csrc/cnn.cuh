@@ -13,25 +13,6 @@ __device__ __forceinline__ float bf16r(float x) {
     return __bfloat162float(__float2bfloat16_rn(x));
 }
 
-// Standard normal CDF Phi(x) in float32 from the rational approximation of
-// Abramowitz & Stegun, Handbook of Mathematical Functions, eq. 7.1.26 (after
-// Hastings): for z >= 0, erfc(z) = t (a1 + t (a2 + t (a3 + t (a4 + t a5))))
-// exp(-z^2) + e(z), t = 1 / (1 + p z), |e(z)| <= 1.5e-7.  With z = |x| / sqrt 2,
-// Phi(-|x|) = erfc(z) / 2 and Phi(|x|) = 1 - Phi(-|x|): the negative tail is
-// formed without the cancellation of 1 + erf.  Absolute error about 1e-7,
-// far under the bf16 rounding the activations then take, in about a third of
-// the instructions of 0.5 (1 + erff(x / sqrt 2)).
-__device__ __forceinline__ float phi_as(float x) {
-    const float z = fabsf(x) * 0.70710678118654752440f;
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, z, 1.0f));
-    float p = fmaf(t, 1.061405429f, -1.453152027f);
-    p = fmaf(t, p, 1.421413741f);
-    p = fmaf(t, p, -0.284496736f);
-    p = fmaf(t, p, 0.254829592f);
-    const float q = 0.5f * (p * t) * __expf(-z * z);  // Phi(-|x|)
-    return x >= 0.0f ? 1.0f - q : q;
-}
-
 // Hardware approximations: 1/x and 2^x (PTX rcp.approx, ex2.approx).
 __device__ __forceinline__ float rcp_hw(float x) {
     float r;
@@ -44,11 +25,15 @@ __device__ __forceinline__ float ex2_hw(float x) {
     return r;
 }
 
-// GELU x Phi(x) of two lanes with the paired instructions: the same
-// Abramowitz & Stegun 7.1.26 form as phi_as, q = Phi(-|x|) = erfc(z)/2 with
-// the 1/2 folded into the coefficients (exact: a power of two) and
-// exp(-z^2) = 2^(-x^2 log2(e) / 2); then x Phi(x) = max(x, 0) - |x| q for
-// either sign of x.
+// GELU x Phi(x) of two lanes with the paired instructions.  Phi(-|x|) =
+// erfc(z) / 2, z = |x| / sqrt 2, from the rational approximation of Abramowitz &
+// Stegun, Handbook of Mathematical Functions, eq. 7.1.26 (after Hastings):
+// erfc(z) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2) + e(z), t =
+// 1 / (1 + p z), |e(z)| <= 1.5e-7, the 1/2 folded into the coefficients (exact:
+// a power of two) and exp(-z^2) = 2^(-x^2 log2(e) / 2); then x Phi(x) =
+// max(x, 0) - |x| q for either sign of x.  Absolute error about 1e-7, far under
+// the bf16 rounding the activations then take, in about a third of the
+// instructions of 0.5 (1 + erff(x / sqrt 2)).
 __device__ __forceinline__ f32x2 gelu2(f32x2 x) {
     float x0, x1;
     f2split(x, x0, x1);
@@ -140,8 +125,39 @@ int pack_hidden_weights(const cnn_desc* d, cudaStream_t st);
 // in/out are [batch][C/8][n][n][8] bf16.  Returns AC_ERR_UNSUPPORTED when the
 // shape has no tensor-core kernel.
 // Derivative of act_apply: 1 - tanh^2, or Phi(x) + x phi(x).
+// Phi(x) + x phi(x) with Phi as in gelu2 and one 2^(-x^2 log2(e) / 2) for both
+// terms; the scalar form has the same roundings as the paired one.
+__device__ __forceinline__ f32x2 gelu_grad2(f32x2 x) {
+    float x0, x1;
+    f2split(x, x0, x1);
+    const f32x2 z = f2_mul(f2(fabsf(x0), fabsf(x1)), f2(0.70710678118654752440f, 0.70710678118654752440f));
+    float d0, d1;
+    f2split(f2_fma(z, f2(0.3275911f, 0.3275911f), f2(1.0f, 1.0f)), d0, d1);
+    const f32x2 t = f2(rcp_hw(d0), rcp_hw(d1));
+    f32x2 p = f2_fma(t, f2(0.5307027145f, 0.5307027145f), f2(-0.7265760135f, -0.7265760135f));
+    p = f2_fma(t, p, f2(0.7107068705f, 0.7107068705f));
+    p = f2_fma(t, p, f2(-0.142248368f, -0.142248368f));
+    p = f2_fma(t, p, f2(0.127414796f, 0.127414796f));
+    float w0, w1;
+    f2split(f2_mul(f2_mul(x, x), f2(-0.72134752044448170368f, -0.72134752044448170368f)), w0, w1);
+    const f32x2 e = f2(ex2_hw(w0), ex2_hw(w1));
+    const f32x2 q = f2_mul(f2_mul(p, t), e);  // Phi(-|x|)
+    float q0, q1, r0, r1;
+    f2split(q, q0, q1);
+    f2split(f2_fma(q, f2(-1.0f, -1.0f), f2(1.0f, 1.0f)), r0, r1);
+    const f32x2 phi = f2(x0 >= 0.0f ? r0 : q0, x1 >= 0.0f ? r1 : q1);
+    return f2_fma(f2_mul(x, e), f2(0.39894228040143267794f, 0.39894228040143267794f), phi);
+}
 __device__ __forceinline__ float act_grad_gelu(float x) {
-    return phi_as(x) + x * __expf(-0.5f * x * x) * 0.39894228040143267794f;
+    const float z = __fmul_rn(fabsf(x), 0.70710678118654752440f);
+    const float t = rcp_hw(__fmaf_rn(z, 0.3275911f, 1.0f));
+    float p = __fmaf_rn(t, 0.5307027145f, -0.7265760135f);
+    p = __fmaf_rn(t, p, 0.7107068705f);
+    p = __fmaf_rn(t, p, -0.142248368f);
+    p = __fmaf_rn(t, p, 0.127414796f);
+    const float e = ex2_hw(__fmul_rn(__fmul_rn(x, x), -0.72134752044448170368f));
+    const float q = __fmul_rn(__fmul_rn(p, t), e);
+    return __fmaf_rn(__fmul_rn(x, e), 0.39894228040143267794f, x >= 0.0f ? __fsub_rn(1.0f, q) : q);
 }
 __device__ __forceinline__ double act_grad_gelu(double x) {
     return 0.5 * (1.0 + erf(x * 0.70710678118654752440)) + x * exp(-0.5 * x * x) * 0.39894228040143267794;
@@ -163,6 +179,17 @@ __device__ __forceinline__ float act_grad_c(float x) {
         return 1.0f - t * t;
     } else {
         return act_grad_gelu(x);
+    }
+}
+
+template <int ACT>
+__device__ __forceinline__ f32x2 act_grad2(f32x2 x) {
+    if constexpr (ACT == AC_ACT_TANH) {
+        float a, b;
+        f2split(x, a, b);
+        return f2(act_grad_c<ACT>(a), act_grad_c<ACT>(b));
+    } else {
+        return gelu_grad2(x);
     }
 }
 

@@ -582,15 +582,14 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
                                     }
                                 }
                             } else {
-                                const float4 za = reinterpret_cast<const float4*>(zio + off)[0];
-                                const float4 zb = reinterpret_cast<const float4*>(zio + off)[1];
-                                const float zz[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
+                                const ulonglong2 za = reinterpret_cast<const ulonglong2*>(zio + off)[0];
+                                const ulonglong2 zb = reinterpret_cast<const ulonglong2*>(zio + off)[1];
+                                const f32x2 zz[4] = {za.x, za.y, zb.x, zb.y};
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) {
                                     float a0, a1;
-                                    f2split(z[e], a0, a1);
-                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(a0 * act_grad_c<ACT>(zz[2 * e]),
-                                                                                    a1 * act_grad_c<ACT>(zz[2 * e + 1]));
+                                    f2split(f2_mul(z[e], act_grad2<ACT>(zz[e])), a0, a1);
+                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
                                     packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
                                 }
                             }

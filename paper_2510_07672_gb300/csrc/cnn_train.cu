@@ -31,6 +31,7 @@
 namespace acpr {
 
 constexpr int kChunks = 64;      // pixel chunks of the weight-gradient reduction
+constexpr int kTcChunks = 152;   // of the tensor-core kernel: one CTA per SM
 constexpr int kWgThreads = 256;
 
 __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
@@ -52,7 +53,7 @@ static TrainLayout train_layout(const cnn_desc* d, int n, int batch) {
     t.off_wt = t.off_dz + 2 * t.a_bytes;
     const size_t wt = size_t(L > 2 ? L - 2 : 0) * 9 * d->channels * d->channels * 2;
     t.off_part = (t.off_wt + wt + 255) / 256 * 256;
-    t.off_gc = t.off_part + size_t(kChunks) * 9 * (size_t(d->channels) * d->channels + d->channels) * 4;
+    t.off_gc = t.off_part + size_t(d->channels == 64 ? kTcChunks : kChunks) * 9 * (size_t(d->channels) * d->channels + d->channels) * 4;
     t.off_zpart = t.off_gc + size_t(batch) * n * n * 4;
     t.off_maps = t.off_zpart + size_t(batch) * n * n * sizeof(double);  // >= the last layer's block partials
     t.total = t.off_maps + size_t(batch) * 9 * n * n * sizeof(float);
@@ -60,37 +61,68 @@ static TrainLayout train_layout(const cnn_desc* d, int n, int batch) {
 }
 
 // ------------------------------------------------------------- forward ----
-// First layer with the float32 pre-activations saved (1 -> C, K = 9).
+// Two horizontally adjacent pixels of a thread as the lanes of the paired
+// instructions: window[a][e] = (v[y + a - 1][x + e - 1], v[y + a - 1][x + e]),
+// bf16-rounded; the weights in shared memory as pairs of equal values.
+__device__ __forceinline__ void pair_window(const float* __restrict__ f, int y, int x, int n, f32x2 (&vp)[3][3]) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = bf16r(f[(long long)wrapi(y + a - 1, n) * n + wrapi(x + e - 1, n)]);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) vp[a][e] = f2(v[e], v[e + 1]);
+    }
+}
 template <int C>
-__global__ void first_fwd_save_kernel(const float* __restrict__ u, __nv_bfloat16* __restrict__ a1,
-                                      float* __restrict__ z0, const float* __restrict__ W,
-                                      const float* __restrict__ bias, int batch, int n, int act) {
-    const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void pair_weights(f32x2* ws, const float* __restrict__ W) {
+    for (int i = threadIdx.x; i < C * 9; i += blockDim.x) ws[i] = f2(bf16r(W[i]), bf16r(W[i]));
+}
+
+// First layer with the float32 pre-activations saved (1 -> C, K = 9): the sums
+// of conv_first_bf16_kernel.  Bound: its stores (6 C bytes a pixel) and GELU; C = 64, 16 fields of 256^2: a pixel a
+// thread with the weights read and rounded per use 179 us, pairs 102 us.
+template <int C, int ACT>
+__global__ void __launch_bounds__(128) first_fwd_save_kernel(const float* __restrict__ u, __nv_bfloat16* __restrict__ a1,
+                                                             float* __restrict__ z0, const float* __restrict__ W,
+                                                             const float* __restrict__ bias, int batch, int n) {
+    __shared__ f32x2 ws[C * 9];
+    __shared__ float bs[C];
+    pair_weights<C>(ws, W);
+    for (int i = threadIdx.x; i < C; i += blockDim.x) bs[i] = bias[i];
+    __syncthreads();
+    const long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 2;
     const long long nn = (long long)n * n;
     if (pix >= nn * batch) return;
-    const int b = int(pix / nn);
-    const int y = int((pix % nn) / n), x = int(pix % n);
-    const float* f = u + (long long)b * nn;
-    float v[9];
-#pragma unroll
-    for (int t = 0; t < 9; ++t) v[t] = bf16r(f[(long long)wrapi(y + t / 3 - 1, n) * n + wrapi(x + t % 3 - 1, n)]);
-#pragma unroll
+    const int lg = __ffs(n) - 1;  // n is a power of two
+    const int b = int(pix >> (2 * lg));
+    const int y = int(pix >> lg) & (n - 1), x = int(pix) & (n - 1);
+    f32x2 vp[3][3];
+    pair_window(u + (long long)b * nn, y, x, n, vp);
+#pragma unroll 1
     for (int kc = 0; kc < C / 8; ++kc) {
-        __align__(16) __nv_bfloat16 o8[8];
-        __align__(16) float z8[8];
+        __align__(16) __nv_bfloat16 o8[2][8];
+        __align__(16) float z8[2][8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int o = kc * 8 + i;
-            float s = 0.f;
+            f32x2 s2 = f2(0.f, 0.f);
 #pragma unroll
-            for (int t = 0; t < 9; ++t) s = fmaf(bf16r(W[o * 9 + t]), v[t], s);
-            z8[i] = s + bias[o];
-            o8[i] = __float2bfloat16_rn(act_apply<float>(act, z8[i]));
+            for (int t = 0; t < 9; ++t) s2 = f2_fma(ws[o * 9 + t], vp[t / 3][t % 3], s2);
+            s2 = f2_add(s2, f2(bs[o], bs[o]));
+            f2split(s2, z8[0][i], z8[1][i]);
+            float a0, a1v;
+            f2split(act2<ACT>(s2), a0, a1v);
+            o8[0][i] = __float2bfloat16_rn(a0);
+            o8[1][i] = __float2bfloat16_rn(a1v);
         }
-        const long long off = (((long long)b * (C / 8) + kc) * nn + pix % nn) * 8;
-        *reinterpret_cast<uint4*>(a1 + off) = *reinterpret_cast<const uint4*>(o8);
-        reinterpret_cast<float4*>(z0 + off)[0] = *reinterpret_cast<const float4*>(z8);
-        reinterpret_cast<float4*>(z0 + off)[1] = *reinterpret_cast<const float4*>(z8 + 4);
+#pragma unroll
+        for (int px = 0; px < 2; ++px) {
+            const long long off = (((long long)b * (C / 8) + kc) * nn + ((pix + px) & (nn - 1))) * 8;
+            *reinterpret_cast<uint4*>(a1 + off) = *reinterpret_cast<const uint4*>(o8[px]);
+            reinterpret_cast<float4*>(z0 + off)[0] = *reinterpret_cast<const float4*>(z8[px]);
+            reinterpret_cast<float4*>(z0 + off)[1] = *reinterpret_cast<const float4*>(z8[px] + 4);
+        }
     }
 }
 
@@ -117,32 +149,45 @@ __global__ void center_kernel(const float* __restrict__ g, float* __restrict__ g
 }
 
 // Last layer: dz_{L-2} = bf16(act'(z_{L-2}) * sum_tap W_L[c][tap] g[p - off(tap)]).
-template <int C>
-__global__ void last_dgrad_kernel(const float* __restrict__ g, const float* __restrict__ W,
-                                  const float* __restrict__ zprev, __nv_bfloat16* __restrict__ dz, int batch,
-                                  int n, int act) {
-    const long long pix = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+// Bound: reading z and writing dz (6 C bytes a pixel); C = 64, 16 fields of
+// 256^2: a pixel a thread 197 us, pairs 88 us.
+template <int C, int ACT>
+__global__ void __launch_bounds__(128) last_dgrad_kernel(const float* __restrict__ g, const float* __restrict__ W,
+                                                         const float* __restrict__ zprev, __nv_bfloat16* __restrict__ dz,
+                                                         int batch, int n) {
+    __shared__ f32x2 ws[C * 9];
+    pair_weights<C>(ws, W);
+    __syncthreads();
+    const long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 2;
     const long long nn = (long long)n * n;
     if (pix >= nn * batch) return;
-    const int b = int(pix / nn);
-    const int y = int((pix % nn) / n), x = int(pix % n);
-    float gv[9];
-#pragma unroll
-    for (int t = 0; t < 9; ++t)  // input p feeds output p - off(tap)
-        gv[t] = bf16r(g[(long long)b * nn + (long long)wrapi(y - (t / 3 - 1), n) * n + wrapi(x - (t % 3 - 1), n)]);
-#pragma unroll
+    const int lg = __ffs(n) - 1;
+    const int b = int(pix >> (2 * lg));
+    const int y = int(pix >> lg) & (n - 1), x = int(pix) & (n - 1);
+    f32x2 vp[3][3];
+    pair_window(g + (long long)b * nn, y, x, n, vp);
+#pragma unroll 1
     for (int kc = 0; kc < C / 8; ++kc) {
-        const long long off = (((long long)b * (C / 8) + kc) * nn + pix % nn) * 8;
-        __align__(16) __nv_bfloat16 o8[8];
+        const long long off = (((long long)b * (C / 8) + kc) * nn + (pix & (nn - 1))) * 8;
+        __align__(16) float z8[2][8];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)  // the two pixels' channels are adjacent
+            reinterpret_cast<float4*>(&z8[0][0])[q] = reinterpret_cast<const float4*>(zprev + off)[q];
+        __align__(16) __nv_bfloat16 o8[2][8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int c = kc * 8 + i;
-            float s = 0.f;
+            f32x2 s2 = f2(0.f, 0.f);
 #pragma unroll
-            for (int t = 0; t < 9; ++t) s = fmaf(bf16r(W[c * 9 + t]), gv[t], s);
-            o8[i] = __float2bfloat16_rn(s * act_grad<float>(act, zprev[off + i]));
+            for (int t = 0; t < 9; ++t)  // input p feeds output p - off(tap)
+                s2 = f2_fma(ws[c * 9 + t], vp[2 - t / 3][2 - t % 3], s2);
+            float a0, a1;
+            f2split(f2_mul(s2, act_grad2<ACT>(f2(z8[0][i], z8[1][i]))), a0, a1);
+            o8[0][i] = __float2bfloat16_rn(a0);
+            o8[1][i] = __float2bfloat16_rn(a1);
         }
-        *reinterpret_cast<uint4*>(dz + off) = *reinterpret_cast<const uint4*>(o8);
+        reinterpret_cast<uint4*>(dz + off)[0] = *reinterpret_cast<const uint4*>(o8[0]);
+        reinterpret_cast<uint4*>(dz + off)[1] = *reinterpret_cast<const uint4*>(o8[1]);
     }
 }
 
@@ -290,119 +335,138 @@ wgrad_kernel(const void* __restrict__ a_src, const void* __restrict__ dz_src, fl
     if (tap == 0 && threadIdx.x < COUT) out[C * C + threadIdx.x] = bacc;
 }
 // The same partials for the first (CIN = 1) and last (COUT = 1) layers, where
-// one side has K = C channels and the other one: a thread walks its own pixels
-// of the (tap, chunk) block with all K channel sums in registers (the K-side
-// operand comes as 16-byte chunk vectors), then the block sums its threads in
-// a fixed order (a shuffle tree per warp, then the warps in order).
+// one side is a float32 field and the other K channels: per pixel q,
+//   first: sum of dz(q, k) u(q + off(tap)),   last: sum of a(q, k) g(q - off(tap)).
+// A block takes one chunk of 8 channels and a range of strips of 8 rows; a
+// thread walks its column with the field's 3 x 3 window sliding, so each 16-byte
+// channel vector is read once for all nine taps (a block per tap read it nine
+// times: 331 and 118 us for 64 channels, 16 fields of 256^2; now 85 and 77).  The threads' sums are folded by exchanging halves, then the warps in
+// order.  Bound: latency of the loads (12 warps per SM).
+constexpr int kThinRows = 8, kThinThreads = 128;
+
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kWgThreads)
-wgrad_thin_kernel(const void* __restrict__ a_src, const void* __restrict__ dz_src, float* __restrict__ part,
-                  int batch, int n, int C) {
+__global__ void __launch_bounds__(kThinThreads) wgrad_thin_kernel(const void* __restrict__ a_src,
+                                                                  const void* __restrict__ dz_src,
+                                                                  float* __restrict__ part, int batch, int n, int C) {
     static_assert(CIN == 1 || COUT == 1, "one side of the layer has one channel");
-    constexpr int K = CIN > COUT ? CIN : COUT;
-    constexpr int KC = K / 8;
-    constexpr int NW = kWgThreads / 32;
-    __shared__ float red[NW][K + 1];
-    const int tap = blockIdx.x % 9;
-    const int chunk = blockIdx.x / 9;
-    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-    const int lg = __ffs(n) - 1;  // n is a power of two
+    constexpr bool FIRST = CIN == 1;
+    constexpr int KC = (FIRST ? COUT : CIN) / 8, NV = 9 * 8 + 8, PAD = 96;
+    __shared__ float red[kThinThreads / 32][PAD];
+    const int kc = blockIdx.y, chunk = blockIdx.x;
+    const int lg = __ffs(n) - 1;  // n is a power of two, at least kThinRows
+    const int mask = n - 1;
     const long long nn = (long long)n * n;
-    const long long total = nn * batch;
-    const long long per_chunk = (total + kChunks - 1) / kChunks;
-    const long long p0 = chunk * per_chunk;
-    const long long p1 = p0 + per_chunk < total ? p0 + per_chunk : total;
-    const bool bias = tap == 0;
-    float acc[K], bacc[CIN == 1 ? K : 1];
+    const long long strips = nn * batch / kThinRows;
+    const long long s0 = strips * chunk / gridDim.x, s1 = strips * (chunk + 1) / gridDim.x;
+    const float* field = static_cast<const float*>(FIRST ? a_src : dz_src);
+    const __nv_bfloat16* vec = static_cast<const __nv_bfloat16*>(FIRST ? dz_src : a_src);
+    f32x2 acc[9][4], bacc[4];
 #pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] = 0.f;
+    for (int h = 0; h < 4; ++h) {
+        bacc[h] = f2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < (CIN == 1 ? K : 1); ++k) bacc[k] = 0.f;
-    for (long long p = p0 + threadIdx.x; p < p1; p += kWgThreads) {
-        const int b = int(p >> (2 * lg));
-        const long long pl = p & (nn - 1);
-        const int y = wrapi((int(p >> lg) & (n - 1)) + dy, n), x = wrapi((int(p) & (n - 1)) + dx, n);
-        const long long q = (long long)y * n + x;
-        if constexpr (CIN == 1) {
-            // first layer: a = the float32 field (bf16-rounded), dz = C bf16 channels at p
-            const float av = bf16r(static_cast<const float*>(a_src)[(long long)b * nn + q]);
-            const __nv_bfloat16* dz = static_cast<const __nv_bfloat16*>(dz_src);
+        for (int t = 0; t < 9; ++t) acc[t][h] = f2(0.f, 0.f);
+    }
+    float gsum = 0.f;
+    const int per = n / kThinRows;
+    for (long long s = s0 + threadIdx.x; s < s1; s += kThinThreads) {
+        const int j = int(s) & mask;
+        const long long r = s >> lg;
+        const int i0 = int(r % per) * kThinRows, b = int(r / per);
+        const float* f = field + b * nn;
+        const uint4* v = reinterpret_cast<const uint4*>(vec) + ((long long)b * KC + kc) * nn;
+        const int jl = (j - 1) & mask, jr = (j + 1) & mask;
+        float w[3][3];
+        auto row = [&](int i, float(&x)[3]) {
+            const float* p = f + (long long)(i & mask) * n;
+            x[0] = bf16r(p[jl]);
+            x[1] = bf16r(p[j]);
+            x[2] = bf16r(p[jr]);
+        };
+        row(i0 - 1, w[0]);
+        row(i0, w[1]);
 #pragma unroll
-            for (int kc = 0; kc < KC; ++kc) {
-                const uint4 raw = *reinterpret_cast<const uint4*>(dz + (((long long)b * KC + kc) * nn + pl) * 8);
-                const __nv_bfloat16* v8 = reinterpret_cast<const __nv_bfloat16*>(&raw);
+        for (int k = 0; k < kThinRows; ++k) {
+            row(i0 + k + 1, w[(k + 2) % 3]);
+            const uint4 raw = v[(long long)(i0 + k) * n + j];
+            const uint32_t word[4] = {raw.x, raw.y, raw.z, raw.w};
+            f32x2 x[4];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const float dv = __bfloat162float(v8[i]);
-                    acc[kc * 8 + i] = fmaf(dv, av, acc[kc * 8 + i]);
-                    if (bias) bacc[kc * 8 + i] += dv;
-                }
+            for (int h = 0; h < 4; ++h)
+                x[h] = f2(__uint_as_float(word[h] << 16), __uint_as_float(word[h] & 0xffff0000u));
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const float u = FIRST ? w[(k + t / 3) % 3][t % 3] : w[(k + 2 - t / 3) % 3][2 - t % 3];
+                const f32x2 u2 = f2(u, u);
+#pragma unroll
+                for (int h = 0; h < 4; ++h) acc[t][h] = f2_fma(u2, x[h], acc[t][h]);
             }
-        } else {
-            // last layer: dz = the float32 output gradient (bf16-rounded), a = C bf16 channels at q
-            const float dv = bf16r(static_cast<const float*>(dz_src)[(long long)b * nn + pl]);
-            const __nv_bfloat16* a = static_cast<const __nv_bfloat16*>(a_src);
+            if constexpr (FIRST) {
 #pragma unroll
-            for (int kc = 0; kc < KC; ++kc) {
-                const uint4 raw = *reinterpret_cast<const uint4*>(a + (((long long)b * KC + kc) * nn + q) * 8);
-                const __nv_bfloat16* v8 = reinterpret_cast<const __nv_bfloat16*>(&raw);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc[kc * 8 + i] = fmaf(dv, __bfloat162float(v8[i]), acc[kc * 8 + i]);
+                for (int h = 0; h < 4; ++h) bacc[h] = f2_add(bacc[h], x[h]);
+            } else {
+                gsum += w[(k + 1) % 3][1];
             }
-            if (bias) bacc[0] += dv;
         }
     }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* out = part + ((long long)chunk * 9 + tap) * (C * C + C);
-    // weight partials: index o * CIN + c is k on both sides (the other index is 0)
+    float val[PAD];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        float v = acc[k];
+    for (int i = 0; i < PAD; ++i) val[i] = 0.f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[warp][k] = v;
+    for (int h = 0; h < 4; ++h) {
+#pragma unroll
+        for (int t = 0; t < 9; ++t) f2split(acc[t][h], val[t * 8 + 2 * h], val[t * 8 + 2 * h + 1]);
+        f2split(bacc[h], val[72 + 2 * h], val[72 + 2 * h + 1]);
     }
+    if constexpr (!FIRST) val[72] = gsum;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int base = 0;
+#pragma unroll
+    for (int o = 16, half = PAD / 2; o > 0; o >>= 1, half /= 2) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float keep = hi ? val[i + half] : val[i], send = hi ? val[i] : val[i + half];
+            val[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        base += hi ? half : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < PAD / 32; ++i) red[warp][base + i] = val[i];
     __syncthreads();
-    if (threadIdx.x < K) {
+    float* out = part + (long long)chunk * 9 * (C * C + C);
+    for (int k = threadIdx.x; k < NV; k += kThinThreads) {
         float t = 0.f;
-        for (int w = 0; w < NW; ++w) t += red[w][threadIdx.x];
-        out[threadIdx.x] = t;
-    }
-    if (bias) {
-        __syncthreads();
 #pragma unroll
-        for (int k = 0; k < COUT; ++k) {
-            float v = bacc[CIN == 1 ? k : 0];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) red[warp][k] = v;
-        }
-        __syncthreads();
-        if (threadIdx.x < COUT) {
-            float t = 0.f;
-            for (int w = 0; w < NW; ++w) t += red[w][threadIdx.x];
-            out[C * C + threadIdx.x] = t;
-        }
+        for (int w = 0; w < kThinThreads / 32; ++w) t += red[w][k];
+        // weight partials: index o * CIN + c is the channel on both sides (the other index is 0)
+        if (k < 72) out[(long long)(k / 8) * (C * C + C) + kc * 8 + k % 8] = t;
+        else if (FIRST) out[C * C + kc * 8 + k - 72] = t;
+        else if (k == 72 && kc == 0) out[C * C] = t;
     }
 }
 
-// Fixed-order sum of the chunk partials into the float32 gradients
-// (W[o][c][tap] layout of the masters; overwrite or accumulate).
-__global__ void wgrad_reduce_kernel(const float* __restrict__ part, float* __restrict__ gw, float* __restrict__ gb,
-                                    int cin, int cout, int C, int accumulate) {
-    const int nw = cout * cin * 9;
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < nw) {
-        const int o = idx / (cin * 9), c = (idx / 9) % cin, tap = idx % 9;
-        float s = 0.f;
-        for (int ch = 0; ch < kChunks; ++ch) s += part[((long long)ch * 9 + tap) * (C * C + C) + o * cin + c];
-        gw[idx] = accumulate ? gw[idx] + s : s;
-    } else if (idx < nw + cout) {
-        const int o = idx - nw;
-        float s = 0.f;
-        for (int ch = 0; ch < kChunks; ++ch) s += part[((long long)ch * 9) * (C * C + C) + C * C + o];
-        gb[o] = accumulate ? gb[o] + s : s;
+// Fixed-order sum of the chunk partials into the float32 gradients: 64
+// parameters a block (neighbouring in the partials), four threads each sum a
+// quarter of the chunks, the quarters in order.
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ part, float* __restrict__ gw,
+                                                           float* __restrict__ gb, int cin, int cout, int C, int chunks,
+                                                           int accumulate) {
+    __shared__ float quarter[4][64];
+    const int cc = cin * cout, nw = cc * 9, g = threadIdx.x >> 6, l = threadIdx.x & 63;
+    const int idx = blockIdx.x * 64 + l;  // [tap][o][c], then the biases
+    float s = 0.f;
+    if (idx < nw + cout) {
+        const long long at = idx < nw ? (long long)(idx / cc) * (C * C + C) + idx % cc : C * C + idx - nw;
+#pragma unroll 4
+        for (int ch = chunks * g / 4; ch < chunks * (g + 1) / 4; ++ch) s += part[(long long)ch * 9 * (C * C + C) + at];
     }
+    quarter[g][l] = s;
+    __syncthreads();
+    if (g || idx >= nw + cout) return;
+    s = ((quarter[0][l] + quarter[1][l]) + quarter[2][l]) + quarter[3][l];
+    float* dst = idx < nw ? gw + (long long)(idx % cc) * 9 + idx / cc : gb + idx - nw;
+    *dst = accumulate ? *dst + s : s;
 }
 
 // ------------------------------------------------------------- host side --
@@ -419,13 +483,16 @@ static int check_train(const cnn_desc* d) {
 template <int CIN, int COUT>
 static int wgrad(const void* a, const void* dz, float* part, float* gw, float* gb, int batch, int n, int C,
                  int accumulate, cudaStream_t st) {
-    if constexpr (CIN == 1 || COUT == 1)
-        wgrad_thin_kernel<CIN, COUT><<<kChunks * 9, kWgThreads, 0, st>>>(a, dz, part, batch, n, C);
-    else
+    int chunks = kChunks;
+    if constexpr (CIN == 1 || COUT == 1) {
+        if (C == 64) chunks = kTcChunks;
+        wgrad_thin_kernel<CIN, COUT><<<dim3(chunks, C / 8), kThinThreads, 0, st>>>(a, dz, part, batch, n, C);
+    } else {
         wgrad_kernel<CIN, COUT><<<kChunks * 9, kWgThreads, 0, st>>>(a, dz, part, batch, n, C);
+    }
     ACPR_LAUNCH_CHECK();
     const int total = COUT * CIN * 9 + COUT;
-    wgrad_reduce_kernel<<<(total + 255) / 256, 256, 0, st>>>(part, gw, gb, CIN, COUT, C, accumulate);
+    wgrad_reduce_kernel<<<(total + 63) / 64, 256, 0, st>>>(part, gw, gb, CIN, COUT, C, chunks, accumulate);
     ACPR_LAUNCH_CHECK();
     return AC_OK;
 }
@@ -435,12 +502,15 @@ static int forward_train(const cnn_desc* d, int n, int batch, const float* u, fl
                          cudaStream_t st) {
     const TrainLayout t = train_layout(d, n, batch);
     const long long pixels = (long long)n * n * batch;
-    const unsigned blocks = unsigned((pixels + 127) / 128);
     const float* W = static_cast<const float*>(d->w);
     const float* Bv = static_cast<const float*>(d->b);
     auto A = [&](int l) { return reinterpret_cast<__nv_bfloat16*>(ws + t.off_a + t.a_bytes * (l - 1)); };
     auto Z = [&](int l) { return reinterpret_cast<float*>(ws + t.off_z + t.z_bytes * l); };
-    first_fwd_save_kernel<C><<<blocks, 128, 0, st>>>(u, A(1), Z(0), W, Bv, batch, n, d->act);
+    const unsigned pair_blocks = unsigned((pixels / 2 + 127) / 128);
+    if (d->act == AC_ACT_TANH)
+        first_fwd_save_kernel<C, AC_ACT_TANH><<<pair_blocks, 128, 0, st>>>(u, A(1), Z(0), W, Bv, batch, n);
+    else
+        first_fwd_save_kernel<C, AC_ACT_GELU><<<pair_blocks, 128, 0, st>>>(u, A(1), Z(0), W, Bv, batch, n);
     ACPR_LAUNCH_CHECK();
     size_t woff = size_t(C) * 9, boff = C;
     for (int l = 1; l < d->layers - 1; ++l) {
@@ -462,12 +532,15 @@ static int forward_train_fused(const cnn_desc* d, int n, int batch, const float*
                                cudaStream_t st) {
     const TrainLayout t = train_layout(d, n, batch);
     const long long pixels = (long long)n * n * batch;
-    const unsigned blocks = unsigned((pixels + 127) / 128);
     const float* W = static_cast<const float*>(d->w);
     const float* Bv = static_cast<const float*>(d->b);
     auto A = [&](int l) { return reinterpret_cast<__nv_bfloat16*>(ws + t.off_a + t.a_bytes * (l - 1)); };
     auto Z = [&](int l) { return reinterpret_cast<float*>(ws + t.off_z + t.z_bytes * l); };
-    first_fwd_save_kernel<C><<<blocks, 128, 0, st>>>(u, A(1), Z(0), W, Bv, batch, n, d->act);
+    const unsigned pair_blocks = unsigned((pixels / 2 + 127) / 128);
+    if (d->act == AC_ACT_TANH)
+        first_fwd_save_kernel<C, AC_ACT_TANH><<<pair_blocks, 128, 0, st>>>(u, A(1), Z(0), W, Bv, batch, n);
+    else
+        first_fwd_save_kernel<C, AC_ACT_GELU><<<pair_blocks, 128, 0, st>>>(u, A(1), Z(0), W, Bv, batch, n);
     ACPR_LAUNCH_CHECK();
     size_t woff = size_t(C) * 9, boff = C;
     const int L = d->layers;
@@ -519,17 +592,23 @@ static int backward(const cnn_desc* d, int n, int batch, const float* u, const f
     // last layer
     rc = wgrad<C, 1>(A(L - 1), gs, part, gw + woffs[L - 1], gb + boffs[L - 1], batch, n, C, accumulate, st);
     if (rc) return rc;
-    last_dgrad_kernel<C><<<blocks, 128, 0, st>>>(gs, W + woffs[L - 1], Z(L - 2), dz[0], batch, n, d->act);
+    const unsigned pair_blocks = unsigned((pixels / 2 + 127) / 128);
+    if (d->act == AC_ACT_TANH)
+        last_dgrad_kernel<C, AC_ACT_TANH><<<pair_blocks, 128, 0, st>>>(gs, W + woffs[L - 1], Z(L - 2), dz[0], batch, n);
+    else
+        last_dgrad_kernel<C, AC_ACT_GELU><<<pair_blocks, 128, 0, st>>>(gs, W + woffs[L - 1], Z(L - 2), dz[0], batch, n);
     ACPR_LAUNCH_CHECK();
     int cur = 0;
     // hidden layers L-2 .. 1: dz[cur] holds dz_l
     for (int l = L - 2; l >= 1; --l) {
         if (wgrad_tc_supported(C, n)) {
-            rc = wgrad_tc_partials(n, batch, A(l), dz[cur], part, kChunks, conv_status(ws), st);
+            const long long units = (long long)batch * (n / 128) * n;
+            const int chunks = int(units < kTcChunks ? units : kTcChunks);
+            rc = wgrad_tc_partials(n, batch, A(l), dz[cur], part, chunks, conv_status(ws), st);
             if (rc) return rc;
             const int tot = C * C * 9 + C;
-            wgrad_reduce_kernel<<<(tot + 255) / 256, 256, 0, st>>>(part, gw + woffs[l], gb + boffs[l], C, C, C,
-                                                                   accumulate);
+            wgrad_reduce_kernel<<<(tot + 63) / 64, 256, 0, st>>>(part, gw + woffs[l], gb + boffs[l], C, C, C, chunks,
+                                                                 accumulate);
             ACPR_LAUNCH_CHECK();
         } else {
             rc = wgrad<C, C>(A(l), dz[cur], part, gw + woffs[l], gb + boffs[l], batch, n, C, accumulate, st);

@@ -9,24 +9,30 @@
 // "MN-major" no-swizzle core-matrix layout of the tcgen05 operands (a core
 // matrix = 8 pixels x 8 channels, 128 contiguous bytes); A and B are read
 // transposed (instruction descriptor bits 15 and 16), LBO = 128 bytes between
-// pixel groups, SBO = the chunk-plane stride.  One MMA = 64 x 64 x 16 (16
-// pixels); the M = 64 accumulator puts rows 16 q .. 16 q + 15 in TMEM lanes
-// 32 q .. 32 q + 15.
+// pixel groups, SBO = the chunk-plane stride.
 //
-// Work: units (field, 128-column block, row) in order, split into kChunks
-// contiguous ranges; each range is run by two CTAs, one for taps 0..4 and one
-// for taps 5..8 (5 or 4 accumulators of 64 columns), so every CTA keeps its
-// accumulators in TMEM over its whole range and writes one partial per tap at
-// the end.  The CTA of taps 0..4 also forms the bias gradient sum_p dz(p, co)
-// as one more 64 x 16 x 16 MMA per pixel group against a B of ones.  The
-// partials are summed in a fixed order by the same reduction as the CUDA-core
-// weight gradient, so the result is deterministic.
-//   warp 0, producer: the input rows y - 1, y, y + 1 of a run start and then
-//     row y + 1 per unit (128 columns plus one pixel each side, wrapped at the
-//     field's edge: bulk copy per chunk plane, wrapped pixel by cp.async) into
-//     a ring of activation rows, and row y of dz into a ring of dz rows;
-//   warp 1 (lane 0), MMA issuer: per unit 8 pixel groups x its taps, then
-//     releases the dz row and the activation row no later unit reads;
+// Work unit: one activation row y of a 128-column block.  Tap row dy pairs it
+// with the gradient row y + 1 - dy, so the unit's operand A is
+//   rows y and y + 1 of dz side by side, M = 128 (dy = 1 and 0), and
+//   row y - 1, M = 64 (dy = 2);
+// dx is a shift of B's start address by one pixel.  Per 16 pixels that is three
+// MMAs of 128 x 64 x 16 and three of 64 x 64 x 16 for all nine taps (one MMA of
+// 64 x 64 x 16 per tap issued nine, and the pipe takes about as long for each).
+// Two gradient rows are one operand when they lie in neighbouring ring slots:
+// the ring has one more slot that repeats slot 0.  The bias gradient rides in
+// the dx = 1 MMA: B there has two more planes, of ones, and the accumulator 16
+// more columns, each sum_p dz(p, co).  One CTA per SM takes a contiguous range
+// of units and keeps all accumulators in TMEM (448 columns); it reads every
+// activation row and every gradient row of its range once.  The partials of the
+// CTAs are summed in a fixed order, so the result is deterministic.
+// Measured, a layer on 16 fields of 256^2: two CTAs per range with 5 and 4 taps
+// each, M = 64, 64 ranges: 289 us; this form 127 us = 608 TFLOP/s.
+//   warp 0, producer: gradient rows y - 1, y, y + 1 at a run's start, then row
+//     y + 1 per unit, and activation row y (128 columns plus one pixel each
+//     side, wrapped at the field's edge: bulk copy per chunk plane, wrapped
+//     pixel by cp.async);
+//   warp 1 (lane 0), MMA issuer: per unit 8 pixel groups, then releases the
+//     activation row and the gradient row no later unit reads;
 //   warps 2..5, epilogue: after the last MMA, read the accumulators and store
 //     the partials.
 // Every wait is bounded and sets the caller's status word when it gives up.
@@ -41,15 +47,17 @@ constexpr int kWC = 64;                          // channels
 constexpr int kWKC = kWC / 8;                    // chunk planes
 constexpr int kWThreads = 32 * 6;                // producer, MMA, 4 epilogue warps
 constexpr uint32_t kWAPlane = 130u * 16u;        // activation row: 128 pixels + 2 guard pixels
-constexpr uint32_t kWASlot = kWKC * kWAPlane;
+constexpr uint32_t kWASlot = (kWKC + 2) * kWAPlane;  // and two planes of ones
 constexpr uint32_t kWDPlane = 128u * 16u;        // dz row: 128 pixels
 constexpr uint32_t kWDSlot = kWKC * kWDPlane;
-constexpr int kWRA = 7;                          // activation-row ring
-constexpr int kWRD = 4;                          // dz-row ring
-constexpr size_t kWOnesOff = size_t(kWRA) * kWASlot + size_t(kWRD) * kWDSlot;
-constexpr uint32_t kWOnesPlane = 16u * 16u;      // B = ones for the bias: N = 16, K = 16, MN-major
-constexpr size_t kWCtlOff = kWOnesOff + 2 * kWOnesPlane;
+constexpr int kWRA = 5;                          // activation-row ring
+constexpr int kWRD = 6;                          // dz-row ring (and one slot that repeats the first)
+constexpr size_t kWCtlOff = size_t(kWRA) * kWASlot + size_t(kWRD + 1) * kWDSlot;
 constexpr size_t kWSmem = kWCtlOff + 256;
+// accumulator columns: dy = 0, 1 for dx = 0, 2, 1 (the last with the bias), dy = 2 for dx = 0, 1, 2
+__host__ __device__ constexpr uint32_t w_col01(int dx) { return dx == 0 ? 0u : (dx == 1 ? 128u : 64u); }
+__host__ __device__ constexpr uint32_t w_col2(int dx) { return 256u + 64u * uint32_t(dx); }
+constexpr uint32_t kWColBias = 128 + kWC;
 
 struct WCtl {
     uint64_t afull[kWRA], aempty[kWRA], dfull[kWRD], dempty[kWRD];
@@ -58,6 +66,7 @@ struct WCtl {
     int abort;
 };
 static_assert(sizeof(WCtl) <= 256, "control block");
+static_assert(kWSmem <= 227 * 1024, "shared memory");
 
 bool g_wgrad_tc = true;
 }  // namespace
@@ -73,9 +82,7 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
     WCtl* ctl = reinterpret_cast<WCtl*>(smem + kWCtlOff);
     volatile int* abort_flag = &ctl->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int group = blockIdx.x & 1;                 // taps 0..4 or 5..8
-    const int tap0 = group ? 5 : 0, ntap = group ? 4 : 5;
-    const int ch = blockIdx.x >> 1;                   // pixel chunk of the reduction
+    const int ch = blockIdx.x;
     const int NB = n / 128;
     const size_t nn = size_t(n) * n;
     const long long total = (long long)batch * NB * n;
@@ -95,11 +102,12 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
         ctl->abort = 0;
         tc::fence_mbar_init();
     }
-    if (group == 0) {
-        uint32_t* ones = reinterpret_cast<uint32_t*>(smem + kWOnesOff);
-        for (int i = tid; i < int(2 * kWOnesPlane / 4); i += blockDim.x) ones[i] = 0x3F803F80u;  // bf16 1.0 pairs
-        tc::fence_proxy_async_smem();
+    // the planes of ones (bf16 pairs) behind every activation row
+    for (int i = tid; i < kWRA * int(2 * kWAPlane / 4); i += blockDim.x) {
+        const int s = i / int(2 * kWAPlane / 4), e = i % int(2 * kWAPlane / 4);
+        reinterpret_cast<uint32_t*>(aring + size_t(s) * kWASlot + kWKC * kWAPlane)[e] = 0x3F803F80u;
     }
+    tc::fence_proxy_async_smem();
     if (warp == 1) tc::tmem_alloc(&ctl->tmem, 512u);
     tc::fence_before_sync();
     __syncthreads();
@@ -121,18 +129,14 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
             const int bx = wl ? x0 : x0 - 1;
             const uint32_t bbytes = uint32_t(130 - int(wl) - int(wr)) * 16u;
             const uint32_t boff = wl ? 16u : 0u;
-            for (int k = start ? 0 : 2; k < 3; ++k) {
-                int yin = y - 1 + k;
-                yin = yin < 0 ? yin + n : (yin >= n ? yin - n : yin);
+            // activation row y
+            {
                 const int slot = ra.idx;
                 bool free_slot = true;
                 if (lane == 0 && ja >= kWRA) free_slot = p_wait(&ctl->aempty[slot], ra.phase ^ 1u, abort_flag, status);
-                if (!__shfl_sync(0xffffffffu, free_slot, 0)) {
-                    ok = false;
-                    break;
-                }
+                if (!__shfl_sync(0xffffffffu, free_slot, 0)) break;
                 unsigned char* dst = aring + size_t(slot) * kWASlot;
-                const __nv_bfloat16* src = a + (size_t(f) * kWKC * nn + size_t(yin) * n) * 8;
+                const __nv_bfloat16* src = a + (size_t(f) * kWKC * nn + size_t(y) * n) * 8;
                 if (lane == 0) {
                     tc::mbar_arrive_expect_tx(&ctl->afull[slot], uint32_t(kWKC) * bbytes);
                     for (int kc = 0; kc < kWKC; ++kc)
@@ -149,21 +153,31 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
                 ++ja;
                 ra.next();
             }
-            if (!ok) break;
-            // dz row y of this unit
-            const int slot = rd.idx;
-            bool free_slot = true;
-            if (lane == 0 && jd >= kWRD) free_slot = p_wait(&ctl->dempty[slot], rd.phase ^ 1u, abort_flag, status);
-            if (!__shfl_sync(0xffffffffu, free_slot, 0)) break;
-            if (lane == 0) {
-                unsigned char* dst = dring + size_t(slot) * kWDSlot;
-                const __nv_bfloat16* src = dz + (size_t(f) * kWKC * nn + size_t(y) * n + size_t(x0)) * 8;
-                tc::mbar_arrive_expect_tx(&ctl->dfull[slot], kWDSlot);
-                for (int kc = 0; kc < kWKC; ++kc)
-                    tc::bulk_g2s(dst + size_t(kc) * kWDPlane, src + size_t(kc) * nn * 8, kWDPlane, &ctl->dfull[slot]);
+            // gradient rows y - 1, y, y + 1 or y + 1
+            for (int k = start ? 0 : 2; k < 3; ++k) {
+                int yin = y - 1 + k;
+                yin = yin < 0 ? yin + n : (yin >= n ? yin - n : yin);
+                const int slot = rd.idx;
+                bool free_slot = true;
+                if (lane == 0 && jd >= kWRD) free_slot = p_wait(&ctl->dempty[slot], rd.phase ^ 1u, abort_flag, status);
+                if (!__shfl_sync(0xffffffffu, free_slot, 0)) {
+                    ok = false;
+                    break;
+                }
+                if (lane == 0) {
+                    const __nv_bfloat16* src = dz + (size_t(f) * kWKC * nn + size_t(yin) * n + size_t(x0)) * 8;
+                    const int copies = slot == 0 ? 2 : 1;  // slot 0 also behind the last one
+                    tc::mbar_arrive_expect_tx(&ctl->dfull[slot], uint32_t(copies) * kWDSlot);
+                    for (int c = 0; c < copies; ++c) {
+                        unsigned char* dst = dring + size_t(c ? kWRD : slot) * kWDSlot;
+                        for (int kc = 0; kc < kWKC; ++kc)
+                            tc::bulk_g2s(dst + size_t(kc) * kWDPlane, src + size_t(kc) * nn * 8, kWDPlane,
+                                         &ctl->dfull[slot]);
+                    }
+                }
+                ++jd;
+                rd.next();
             }
-            ++jd;
-            rd.next();
         }
         // drain: every issued copy lands before the CTA may exit
         if (lane == 0) {
@@ -177,63 +191,55 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
     } else if (warp == 1) {
         if (lane == 0) {
             // ---- MMA issuer
-            // bf16 A and B, f32 D, both operands MN-major (transposed), M = 64, N = 64
-            constexpr uint32_t idesc = tc::idesc_bf16_f32(64, 64) | (1u << 15) | (1u << 16);
-            constexpr uint32_t idesc_b = tc::idesc_bf16_f32(64, 16) | (1u << 15) | (1u << 16);
-            const uint64_t ones_d = tc::smem_desc(tc::smem_u32(smem + kWOnesOff), 128, kWOnesPlane);
+            // bf16 A and B, f32 D, both operands MN-major (transposed)
+            constexpr uint32_t tr = (1u << 15) | (1u << 16);
+            constexpr uint32_t id01 = tc::idesc_bf16_f32(128, kWC) | tr, id01b = tc::idesc_bf16_f32(128, kWC + 16) | tr;
+            constexpr uint32_t id2 = tc::idesc_bf16_f32(64, kWC) | tr;
             const uint64_t a_hi = tc::smem_desc(0, 128, kWDPlane);  // A = dz rows
             const uint64_t b_hi = tc::smem_desc(0, 128, kWAPlane);  // B = activation rows
             const uint32_t aring_u = tc::smem_u32(aring) >> 4, dring_u = tc::smem_u32(dring) >> 4;
             RingPos ra(kWRA), rd(kWRD);
-            // ring positions of the unit's rows y - 1, y, y + 1
-            int pos[3] = {0, 0, 0};
-            uint32_t par[3] = {0, 0, 0};
-            bool ok = true, first = true;
+            int pos[3] = {0, 0, 0};  // ring slots of the gradient rows y - 1, y, y + 1
+            bool ok = true;
+            uint32_t acc = 0;
             int y = int(u0 % n);
             for (long long u = u0; u < u1 && ok; ++u, y = (y + 1 == n ? 0 : y + 1)) {
                 const bool start = (u == u0) || (y == 0);
-                if (start) {
-                    for (int k = 0; k < 3; ++k, ra.next()) {
-                        pos[k] = ra.idx;
-                        par[k] = ra.phase;
-                    }
-                } else {
-                    pos[0] = pos[1];
-                    par[0] = par[1];
-                    pos[1] = pos[2];
-                    par[1] = par[2];
-                    pos[2] = ra.idx;
-                    par[2] = ra.phase;
-                    ra.next();
+                pos[0] = pos[1];
+                pos[1] = pos[2];
+                for (int k = start ? 0 : 2; k < 3 && ok; ++k) {
+                    pos[k] = rd.idx;
+                    ok = p_wait(&ctl->dfull[rd.idx], rd.phase, abort_flag, status);
+                    rd.next();
                 }
-                for (int k = start ? 0 : 2; k < 3 && ok; ++k) ok = p_wait(&ctl->afull[pos[k]], par[k], abort_flag, status);
-                if (ok) ok = p_wait(&ctl->dfull[rd.idx], rd.phase, abort_flag, status);
+                if (ok) ok = p_wait(&ctl->afull[ra.idx], ra.phase, abort_flag, status);
                 if (!ok) break;
                 // the wrapped pixels came by cp.async (generic proxy); the MMAs read through the async proxy
                 tc::fence_proxy_async_smem();
                 tc::fence_after_sync();
-                const uint32_t d_u = dring_u + uint32_t(rd.idx) * (kWDSlot >> 4);
+                const uint32_t d01 = dring_u + uint32_t(pos[1]) * (kWDSlot >> 4);  // rows y, y + 1: slot pos[1] and the next
+                const uint32_t d2 = dring_u + uint32_t(pos[0]) * (kWDSlot >> 4);
+                const uint32_t r_u = aring_u + uint32_t(ra.idx) * (kWASlot >> 4);
 #pragma unroll 1
                 for (int kg = 0; kg < 8; ++kg) {
-                    const uint64_t ad = a_hi | uint64_t(d_u + uint32_t(kg * 16));
-                    for (int t = 0; t < ntap; ++t) {
-                        const int tap = tap0 + t, dy = tap / 3, dx = tap % 3;
-                        const uint32_t r_u = aring_u + uint32_t(pos[dy]) * (kWASlot >> 4);
+                    const uint64_t a01 = a_hi | uint64_t(d01 + uint32_t(kg * 16));
+                    const uint64_t a2 = a_hi | uint64_t(d2 + uint32_t(kg * 16));
+#pragma unroll
+                    for (int dx = 0; dx < 3; ++dx) {
                         const uint64_t bd = b_hi | uint64_t(r_u + uint32_t(kg * 16 + dx));
-                        tc::mma_bf16(tmem + uint32_t(t * kWC), ad, bd, idesc, (first && kg == 0) ? 0u : 1u);
+                        tc::mma_bf16(tmem + w_col01(dx), a01, bd, dx == 1 ? id01b : id01, acc);
+                        tc::mma_bf16(tmem + w_col2(dx), a2, bd, id2, acc);
                     }
-                    if (group == 0)  // bias: every column of this accumulator is sum_p dz(p, co)
-                        tc::mma_bf16(tmem + uint32_t(5 * kWC), ad, ones_d, idesc_b, (first && kg == 0) ? 0u : 1u);
+                    acc = 1;
                 }
-                first = false;
-                tc::mma_commit(&ctl->dempty[rd.idx]);
-                rd.next();
+                tc::mma_commit(&ctl->aempty[ra.idx]);
+                ra.next();
                 // row y - 1 is read by no later unit; at the end of a run neither are y, y + 1
                 const bool cont = (u + 1 < u1) && (y + 1 != n);
-                tc::mma_commit(&ctl->aempty[pos[0]]);
+                tc::mma_commit(&ctl->dempty[pos[0]]);
                 if (!cont) {
-                    tc::mma_commit(&ctl->aempty[pos[1]]);
-                    tc::mma_commit(&ctl->aempty[pos[2]]);
+                    tc::mma_commit(&ctl->dempty[pos[1]]);
+                    tc::mma_commit(&ctl->dempty[pos[2]]);
                 }
             }
             // every MMA issued completes before the accumulators are read and TMEM is freed
@@ -241,21 +247,22 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
             if (!ok) *abort_flag = 1;
         }
     } else {
-        // ---- epilogue: the accumulators of this CTA's taps -> partials
+        // ---- epilogue: the accumulators -> partials
         const int q = warp & 3;
         const bool ok = tc::mbar_wait_bounded(&ctl->fin, 0, kTcSpin);
         if (!ok) atomicExch(status, 3);
         tc::fence_after_sync();
         if (ok && !*abort_flag) {
-            const int co = 16 * q + lane;  // valid for lanes 0..15
-            for (int t = 0; t < ntap; ++t) {
-                float* dst = part + (size_t(ch) * 9 + size_t(tap0 + t)) * (kWC * kWC + kWC) + size_t(co) * kWC;
+            constexpr size_t kTapFloats = kWC * kWC + kWC;
+            float* base = part + size_t(ch) * 9 * kTapFloats;
+            auto store = [&](uint32_t col, int tap, int co, bool valid) {
+                float* dst = base + size_t(tap) * kTapFloats + size_t(co) * kWC;
 #pragma unroll 1
                 for (int c0 = 0; c0 < kWC; c0 += 8) {
                     uint32_t v[8];
-                    tc::tmem_ld8(tmem + (uint32_t(q * 32) << 16) + uint32_t(t * kWC + c0), v);
+                    tc::tmem_ld8(tmem + (uint32_t(q * 32) << 16) + col + uint32_t(c0), v);
                     tc::tmem_wait_ld();
-                    if (lane < 16) {
+                    if (valid) {
                         reinterpret_cast<float4*>(dst + c0)[0] =
                             make_float4(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]),
                                         __uint_as_float(v[3]));
@@ -264,13 +271,17 @@ wgrad_tc_kernel(const __nv_bfloat16* __restrict__ a, const __nv_bfloat16* __rest
                                         __uint_as_float(v[7]));
                     }
                 }
+            };
+            // M = 128: lane m holds row m (m < 64: dy = 1, else dy = 0); M = 64: rows 16 q .. 16 q + 15 in lanes 32 q ..
+            const int m = 32 * q + lane;
+            for (int dx = 0; dx < 3; ++dx) {
+                store(w_col01(dx), (m < kWC ? 3 : 0) + dx, m & (kWC - 1), true);
+                store(w_col2(dx), 6 + dx, 16 * q + (lane & 15), lane < 16);
             }
-            if (group == 0) {
-                uint32_t v[8];
-                tc::tmem_ld8(tmem + (uint32_t(q * 32) << 16) + uint32_t(5 * kWC), v);
-                tc::tmem_wait_ld();
-                if (lane < 16) part[(size_t(ch) * 9) * (kWC * kWC + kWC) + kWC * kWC + co] = __uint_as_float(v[0]);
-            }
+            uint32_t v[8];
+            tc::tmem_ld8(tmem + (uint32_t(q * 32) << 16) + kWColBias, v);
+            tc::tmem_wait_ld();
+            if (m < kWC) base[kWC * kWC + m] = __uint_as_float(v[0]);  // sum of dz over the rows y (dy = 1)
         }
     }
     tc::fence_before_sync();
@@ -296,7 +307,7 @@ int wgrad_tc_partials(int n, int batch, const __nv_bfloat16* a, const __nv_bfloa
         ACPR_CUDA(cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kWSmem)));
         configured = true;
     }
-    wgrad_tc_kernel<<<2 * chunks, kWThreads, kWSmem, st>>>(a, dz, part, n, batch, chunks, status);
+    wgrad_tc_kernel<<<chunks, kWThreads, kWSmem, st>>>(a, dz, part, n, batch, chunks, status);
     ACPR_LAUNCH_CHECK();
     return AC_OK;
 }
