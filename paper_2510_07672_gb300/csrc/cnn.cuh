@@ -25,86 +25,50 @@ __device__ __forceinline__ float ex2_hw(float x) {
     return r;
 }
 
-// GELU x Phi(x) = max(x, 0) + a 2^P(a), a = -min(|x|, 8): Phi(-|x|) = 2^P with
-// P the polynomial of degree 9 fitted to log2 Phi on [-8, 0], P(0) = -1 (linear
-// program on 5000 points, the error weighted by |x| Phi^0.8).  Against float64
-// the absolute error is below that of the rational form of gelu_tail on every
-// unit interval of [-6, 5] (at most 6e-8 for x < 1; relative 1.5e-7 near zero), far
-// under the bf16 rounding the activations then take, with one exponential and
-// no reciprocal.  Beyond 8, Phi(-|x|) < 1e-15.  NaN gives NaN.
-constexpr int kGeluTerms = 10;
-__device__ __forceinline__ constexpr float gelu_coef(int i) {
-    constexpr float c[kGeluTerms] = {-1.0f,           1.151106358e+00f, -4.592000544e-01f, 5.250946805e-02f,  7.057531737e-03f,
-                                     1.028008701e-04f, -2.209950180e-04f, -5.545776730e-05f, -6.374868462e-06f, -3.000669153e-07f};
-    return c[i];
-}
-__device__ __forceinline__ float max_nan(float a, float b) {
-    float r;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float gelu1(float x) {
-    const float a = fmaxf(-fabsf(x), -8.0f);
-    float p = gelu_coef(kGeluTerms - 1);
-#pragma unroll
-    for (int i = kGeluTerms - 2; i >= 0; --i) p = __fmaf_rn(a, p, gelu_coef(i));
-    return __fmaf_rn(a, ex2_hw(p), max_nan(x, 0.0f));
-}
-
-// The coefficients as pairs of equal values for the paired instructions, which
-// take no immediates: a load from shared memory keeps them in registers
-// (gelu_stage by the block before a barrier, gelu_load by the threads after it).
-// Instructions per pair of a hidden layer's outputs, C = 64: 51 with the rational
-// form (in pairs or not), 53 with this polynomial one lane at a time, 43 in
-// pairs; first layer 48 -> 40.
-struct GeluK {
-    f32x2 c[kGeluTerms];
-};
-__device__ __forceinline__ void gelu_stage(f32x2* sm) {
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int i = 0; i < kGeluTerms; ++i) sm[i] = f2(gelu_coef(i), gelu_coef(i));
-}
-__device__ __forceinline__ GeluK gelu_load(const f32x2* sm) {
-    GeluK k;
-    const uint32_t at = static_cast<uint32_t>(__cvta_generic_to_shared(sm));
-    static_assert(kGeluTerms % 2 == 0, "vectors of two pairs");
-#pragma unroll
-    for (int i = 0; i < kGeluTerms; i += 2)
-        asm volatile("ld.volatile.shared.v2.b64 {%0, %1}, [%2];" : "=l"(k.c[i]), "=l"(k.c[i + 1]) : "r"(at + 8u * i) : "memory");
-    return k;
-}
-// Two lanes of gelu1 with the same roundings.
-__device__ __forceinline__ f32x2 gelu2(f32x2 x, const GeluK& k) {
-    float x0, x1, p0, p1;
+// GELU x Phi(x) of two lanes with the paired instructions.  Phi(-|x|) =
+// erfc(z) / 2, z = |x| / sqrt 2, from the rational approximation of Abramowitz &
+// Stegun, Handbook of Mathematical Functions, eq. 7.1.26 (after Hastings):
+// erfc(z) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2) + e(z), t =
+// 1 / (1 + p z), |e(z)| <= 1.5e-7, the 1/2 folded into the coefficients (exact:
+// a power of two) and exp(-z^2) = 2^(-x^2 log2(e) / 2); then x Phi(x) =
+// max(x, 0) - |x| q for either sign of x.  Absolute error about 1e-7, far under
+// the bf16 rounding the activations then take, in about a third of the
+// instructions of 0.5 (1 + erff(x / sqrt 2)).
+__device__ __forceinline__ f32x2 gelu2(f32x2 x) {
+    float x0, x1;
     f2split(x, x0, x1);
-    const f32x2 a = f2(fmaxf(-fabsf(x0), -8.0f), fmaxf(-fabsf(x1), -8.0f));
-    f32x2 p = k.c[kGeluTerms - 1];
-#pragma unroll
-    for (int i = kGeluTerms - 2; i >= 0; --i) p = f2_fma(a, p, k.c[i]);
-    f2split(p, p0, p1);
-    return f2_fma(a, f2(ex2_hw(p0), ex2_hw(p1)), f2(max_nan(x0, 0.0f), max_nan(x1, 0.0f)));
+    const f32x2 nx = f2(-fabsf(x0), -fabsf(x1));
+    const f32x2 rx = f2(fmaxf(x0, 0.0f), fmaxf(x1, 0.0f));
+    const f32x2 z = f2_mul(nx, f2(-0.70710678118654752440f, -0.70710678118654752440f));
+    float d0, d1;
+    f2split(f2_fma(z, f2(0.3275911f, 0.3275911f), f2(1.0f, 1.0f)), d0, d1);
+    const f32x2 t = f2(rcp_hw(d0), rcp_hw(d1));
+    f32x2 p = f2_fma(t, f2(0.5307027145f, 0.5307027145f), f2(-0.7265760135f, -0.7265760135f));
+    p = f2_fma(t, p, f2(0.7107068705f, 0.7107068705f));
+    p = f2_fma(t, p, f2(-0.142248368f, -0.142248368f));
+    p = f2_fma(t, p, f2(0.127414796f, 0.127414796f));
+    float w0, w1;  // -x^2 log2(e) / 2
+    f2split(f2_mul(f2_mul(x, x), f2(-0.72134752044448170368f, -0.72134752044448170368f)), w0, w1);
+    const f32x2 q = f2_mul(f2_mul(p, t), f2(ex2_hw(w0), ex2_hw(w1)));  // Phi(-|x|)
+    return f2_fma(nx, q, rx);
 }
 
-// Phi(-|x|) = erfc(z) / 2, z = |x| / sqrt 2, and exp(-z^2), for the derivative:
-// the rational approximation of Abramowitz & Stegun, Handbook of Mathematical
-// Functions, eq. 7.1.26 (after Hastings): erfc(z) = t (a1 + t (a2 + t (a3 +
-// t (a4 + t a5)))) exp(-z^2) + e(z), t = 1 / (1 + p z), |e(z)| <= 1.5e-7, the 1/2
-// folded into the coefficients (exact: a power of two), 1 / sqrt 2 into p, and
-// exp(-z^2) = 2^-(x sqrt(log2(e) / 2))^2.
-__device__ __forceinline__ void gelu_tail(float x, float& e, float& q) {
-    const float t = rcp_hw(__fmaf_rn(fabsf(x), 0.23164188841f, 1.0f));
+// One lane of gelu2 with the same roundings (scalar kernels and the paired
+// ones give the same bits for the same input).
+__device__ __forceinline__ float gelu1(float x) {
+    const float nx = -fabsf(x);
+    const float z = __fmul_rn(nx, -0.70710678118654752440f);
+    const float t = rcp_hw(__fmaf_rn(z, 0.3275911f, 1.0f));
     float p = __fmaf_rn(t, 0.5307027145f, -0.7265760135f);
     p = __fmaf_rn(t, p, 0.7107068705f);
     p = __fmaf_rn(t, p, -0.142248368f);
     p = __fmaf_rn(t, p, 0.127414796f);
-    const float s = __fmul_rn(x, 0.84932180028801904f);
-    e = ex2_hw(-__fmul_rn(s, s));
-    q = __fmul_rn(__fmul_rn(p, t), e);
+    const float q = __fmul_rn(__fmul_rn(p, t), ex2_hw(__fmul_rn(__fmul_rn(x, x), -0.72134752044448170368f)));
+    return __fmaf_rn(nx, q, fmaxf(x, 0.0f));
 }
 
 // Activation after every conv but the last: tanh, or GELU x * Phi(x)
-// (float32: gelu1; float64: 0.5 (1 + erf(x / sqrt 2))).
+// (float32: gelu1 / gelu2; float64: 0.5 (1 + erf(x / sqrt 2))).
 __device__ __forceinline__ float act_apply_gelu(float x) { return gelu1(x); }
 __device__ __forceinline__ double act_apply_gelu(double x) {
     return 0.5 * x * (1.0 + erf(x * 0.70710678118654752440));
@@ -124,40 +88,16 @@ __device__ __forceinline__ float act_c(float x) {
     else return act_apply_gelu(x);
 }
 
-// act_c of two lanes.
+// act_c of two lanes (GELU with the paired instructions).
 template <int ACT>
-__device__ __forceinline__ f32x2 act2(f32x2 x, const GeluK& k) {
+__device__ __forceinline__ f32x2 act2(f32x2 x) {
     if constexpr (ACT == AC_ACT_TANH) {
         float a, b;
         f2split(x, a, b);
         return f2(tanhf(a), tanhf(b));
     } else {
-        return gelu2(x, k);
+        return gelu2(x);
     }
-}
-
-// First layer (1 -> C): weights (bf16-rounded) and bias of an output channel as
-// ten pairs of equal values in shared memory, read as five 16-byte vectors,
-// for two adjacent pixels as the lanes of the paired instructions.
-template <int C>
-__device__ __forceinline__ void first_weights(f32x2* ws, const float* __restrict__ W, const float* __restrict__ bias) {
-    for (int i = threadIdx.x; i < C * 10; i += blockDim.x) {
-        const float v = i % 10 < 9 ? bf16r(W[i / 10 * 9 + i % 10]) : bias[i / 10];
-        ws[i] = f2(v, v);
-    }
-}
-// The taps in order from zero, then the bias.
-__device__ __forceinline__ f32x2 first_pair(const f32x2* ws, int o, const f32x2 (&vp)[3][3]) {
-    const ulonglong2* w = reinterpret_cast<const ulonglong2*>(ws + o * 10);
-    f32x2 s = f2(0.f, 0.f);
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        const ulonglong2 q = w[m];
-        s = f2_fma(q.x, vp[2 * m / 3][2 * m % 3], s);
-        s = f2_fma(q.y, vp[(2 * m + 1) / 3][(2 * m + 1) % 3], s);
-    }
-    const ulonglong2 q = w[4];
-    return f2_add(f2_fma(q.x, vp[2][2], s), q.y);
 }
 
 int check_cnn(const cnn_desc* d);
@@ -181,11 +121,42 @@ int last_layer_bf16(const cnn_desc* d, int n, int batch, const __nv_bfloat16* a,
 size_t packed_hidden_bytes(const cnn_desc* d);
 int pack_hidden_weights(const cnn_desc* d, cudaStream_t st);
 
-// Derivative of act_apply: 1 - tanh^2, or Phi(x) + x phi(x) with one
-// exponential for both terms.
+// Hidden layer l (1 <= l <= layers - 2) on the tensor cores:
+// in/out are [batch][C/8][n][n][8] bf16.  Returns AC_ERR_UNSUPPORTED when the
+// shape has no tensor-core kernel.
+// Derivative of act_apply: 1 - tanh^2, or Phi(x) + x phi(x).
+// Phi(x) + x phi(x) with Phi as in gelu2 and one 2^(-x^2 log2(e) / 2) for both
+// terms; the scalar form has the same roundings as the paired one.
+__device__ __forceinline__ f32x2 gelu_grad2(f32x2 x) {
+    float x0, x1;
+    f2split(x, x0, x1);
+    const f32x2 z = f2_mul(f2(fabsf(x0), fabsf(x1)), f2(0.70710678118654752440f, 0.70710678118654752440f));
+    float d0, d1;
+    f2split(f2_fma(z, f2(0.3275911f, 0.3275911f), f2(1.0f, 1.0f)), d0, d1);
+    const f32x2 t = f2(rcp_hw(d0), rcp_hw(d1));
+    f32x2 p = f2_fma(t, f2(0.5307027145f, 0.5307027145f), f2(-0.7265760135f, -0.7265760135f));
+    p = f2_fma(t, p, f2(0.7107068705f, 0.7107068705f));
+    p = f2_fma(t, p, f2(-0.142248368f, -0.142248368f));
+    p = f2_fma(t, p, f2(0.127414796f, 0.127414796f));
+    float w0, w1;
+    f2split(f2_mul(f2_mul(x, x), f2(-0.72134752044448170368f, -0.72134752044448170368f)), w0, w1);
+    const f32x2 e = f2(ex2_hw(w0), ex2_hw(w1));
+    const f32x2 q = f2_mul(f2_mul(p, t), e);  // Phi(-|x|)
+    float q0, q1, r0, r1;
+    f2split(q, q0, q1);
+    f2split(f2_fma(q, f2(-1.0f, -1.0f), f2(1.0f, 1.0f)), r0, r1);
+    const f32x2 phi = f2(x0 >= 0.0f ? r0 : q0, x1 >= 0.0f ? r1 : q1);
+    return f2_fma(f2_mul(x, e), f2(0.39894228040143267794f, 0.39894228040143267794f), phi);
+}
 __device__ __forceinline__ float act_grad_gelu(float x) {
-    float e, q;
-    gelu_tail(x, e, q);
+    const float z = __fmul_rn(fabsf(x), 0.70710678118654752440f);
+    const float t = rcp_hw(__fmaf_rn(z, 0.3275911f, 1.0f));
+    float p = __fmaf_rn(t, 0.5307027145f, -0.7265760135f);
+    p = __fmaf_rn(t, p, 0.7107068705f);
+    p = __fmaf_rn(t, p, -0.142248368f);
+    p = __fmaf_rn(t, p, 0.127414796f);
+    const float e = ex2_hw(__fmul_rn(__fmul_rn(x, x), -0.72134752044448170368f));
+    const float q = __fmul_rn(__fmul_rn(p, t), e);
     return __fmaf_rn(__fmul_rn(x, e), 0.39894228040143267794f, x >= 0.0f ? __fsub_rn(1.0f, q) : q);
 }
 __device__ __forceinline__ double act_grad_gelu(double x) {
@@ -213,9 +184,13 @@ __device__ __forceinline__ float act_grad_c(float x) {
 
 template <int ACT>
 __device__ __forceinline__ f32x2 act_grad2(f32x2 x) {
-    float a, b;
-    f2split(x, a, b);
-    return f2(act_grad_c<ACT>(a), act_grad_c<ACT>(b));
+    if constexpr (ACT == AC_ACT_TANH) {
+        float a, b;
+        f2split(x, a, b);
+        return f2(act_grad_c<ACT>(a), act_grad_c<ACT>(b));
+    } else {
+        return gelu_grad2(x);
+    }
 }
 
 // Every conv workspace (cnn_desc.work and the training workspace) starts
@@ -235,9 +210,6 @@ int conv_check_status_uncaptured(int* status, cudaStream_t st);
 // waits on an mbarrier that nothing arrives on, for `polls` polls.
 void set_test_stall(int polls);
 
-// Hidden layer l (1 <= l <= layers - 2) on the tensor cores:
-// in/out are [batch][C/8][n][n][8] bf16.  Returns AC_ERR_UNSUPPORTED when the
-// shape has no tensor-core kernel.
 int hidden_layer_bf16(const cnn_desc* d, int l, int n, int batch, const __nv_bfloat16* in,
                       __nv_bfloat16* out, const float* w_master, const float* bias, int* status, cudaStream_t st,
                       float* zsave = nullptr);

@@ -21,7 +21,6 @@
 // conv_check_status() reports as AC_ERR_TIMEOUT.
 // Fields with n >= 128 take the persistent, warp-specialised kernel below.
 #include <algorithm>
-#include <type_traits>
 
 #include "cnn.cuh"
 #include "tc_pipe.cuh"
@@ -293,16 +292,9 @@ conv_hidden_tc_kernel(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __res
 //     Every output is ((D(y-1)[0] + b) + D(y)[1]) + D(y+1)[2] with each
 //     D accumulated over (dx, K-step) in order, whatever the ring depth, TMEM
 //     slot count or CTA count: G is bitwise the same under every shape.
-// kFwdLast: the nine-tap projection of a row's activations is one more GEMM
-// (M = 128 pixels, N = 16 with seven zero columns, K = C).  The epilogue warps
-// leave the bf16 activations in shared memory in the A layout (two buffers), one
-// more warp issues the C/16 MMAs into 16 of the columns a TMEM slot pads with,
-// and the epilogue warps store the maps of row r - 1 while row r's are formed.
-// On the CUDA cores the projection was 5 C paired fmas and loads a pixel: last
-// hidden layer of one 1024^2 field, C = 64: 123 -> 88 us, of 16 of 256^2, C = 32:
-// 76 -> 58 us (a layer without it: 73 and 53).
-// What bounds the epilogue: without its GELU the layers take 58 and 45 us, with one
-// twelfth of the MMAs 70 and 52, without the stores 73 and 52 (73 and 54 in full).
+// kFwdLast: the nine-tap projection of each pixel's activations is summed
+// per warp over its channels and then over the warps of a lane quarter in a
+// fixed order through shared memory.
 constexpr int kRMaxRing = 24;
 constexpr int kRMaxD = 5;
 
@@ -312,18 +304,15 @@ struct RCtl {
     uint64_t empty[kRMaxRing];
     uint64_t dfull[kRMaxD];
     uint64_t dempty[kRMaxD];
-    uint64_t pfull[2];  // kFwdLast: a row's activations are in buffer r % 2
-    uint64_t pdone[2];  // kFwdLast: its projection is in TMEM
+    uint64_t qbar[2][4];  // kFwdLast: the partial projections of a lane quarter are in shared memory
     uint64_t fin;  // completion of every MMA the CTA issued
     uint32_t tmem;
     int abort;
     alignas(16) float bias[64];
-    alignas(16) f32x2 gelu[kGeluTerms];
+    alignas(16) float wl[64 * 10];  // kFwdLast: bf16-rounded last-layer weights [channel][tap], tap 9 = 0
 };
-constexpr size_t kRCtlBytes = 1024;
-// kFwdLast: activation buffers [2][C/8][128 pixels][8] and last-layer weights [C/8][16 taps][8], bf16
-__host__ __device__ constexpr uint32_t r_act_bytes(int C) { return uint32_t(C / 8) * 128u * 16u; }
-__host__ __device__ constexpr uint32_t r_last_bytes(int C) { return 2u * r_act_bytes(C) + uint32_t(C / 8) * 16u * 16u; }
+constexpr size_t kRCtlBytes = 4096;
+constexpr size_t kRScratchBytes = size_t(2) * 4 * 4 * 9 * 32 * sizeof(float);  // [2][quarter][warp][tap][lane]
 
 // TMEM columns of one slot: 3C rounded up to a power of two, so that every
 // slot starts on a multiple of its own width.
@@ -331,18 +320,17 @@ __host__ __device__ constexpr int r_dcols(int C) { return C <= 16 ? 64 : (C <= 3
 __host__ __device__ constexpr uint32_t r_slot_bytes(int C) { return uint32_t(C / 8) * 130u * 16u; }
 
 // Epilogue geometry: CPW 8-channel chunks per warp, EPW warps per TMEM lane
-// quarter, THREADS = producer warp + two MMA warps + 4 EPW epilogue warps
-// (+ the projection's issuer with kFwdLast).
-template <int C, int mode>
+// quarter, THREADS = producer warp + two MMA warps + 4 EPW epilogue warps.
+template <int C>
 struct RGeom {
     static constexpr int KC = C / 8;
     static constexpr int CPW = KC >= 4 ? KC / 4 : 1;
     static constexpr int EPW = KC / CPW;
-    static constexpr int THREADS = 32 * (3 + 4 * EPW + (mode == kFwdLast));
+    static constexpr int THREADS = 32 * (3 + 4 * EPW);
 };
 
 template <int C, int ACT, int mode>
-__global__ void __launch_bounds__(RGeom<C, mode>::THREADS, 1)
+__global__ void __launch_bounds__(RGeom<C>::THREADS, 1)
 conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ out,
              const __nv_bfloat16* __restrict__ wpk, const float* __restrict__ bias, int n, int batch, int RING,
              int DS, float* __restrict__ zio, int* __restrict__ status, int stall,
@@ -350,8 +338,8 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
     constexpr int KC = C / 8;
     constexpr int N3 = 3 * C;
     constexpr int DCOLS = r_dcols(C);
-    constexpr int CPW = RGeom<C, mode>::CPW;  // chunks per epilogue warp
-    constexpr int EPW = RGeom<C, mode>::EPW;  // epilogue warps per lane quarter
+    constexpr int CPW = RGeom<C>::CPW;  // chunks per epilogue warp
+    constexpr int EPW = RGeom<C>::EPW;  // epilogue warps per lane quarter
     constexpr uint32_t WBYTES = 9u * C * C * 2u;
     constexpr uint32_t PLANE = 130u * 16u;
     constexpr uint32_t SLOT = r_slot_bytes(C);
@@ -359,8 +347,7 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
     unsigned char* w_tile = smem;  // [dx][kc][dy][cout][8]: B of the (dx, K-step) MMA is one block
     unsigned char* ring = smem + WBYTES;
     RCtl* ctl = reinterpret_cast<RCtl*>(ring + size_t(RING) * SLOT);
-    unsigned char* act_buf = reinterpret_cast<unsigned char*>(ctl) + kRCtlBytes;
-    unsigned char* wl_tile = act_buf + 2 * r_act_bytes(C);
+    float* scratch = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(ctl) + kRCtlBytes);
     volatile int* abort_flag = &ctl->abort;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int NB = n / 128;
@@ -378,16 +365,12 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
             tc::mbar_init(&ctl->dfull[i], 1);
             tc::mbar_init(&ctl->dempty[i], 4 * EPW);
         }
-        for (int i = 0; i < 2; ++i) {
-            tc::mbar_init(&ctl->pfull[i], 4 * EPW);
-            tc::mbar_init(&ctl->pdone[i], 1);
-        }
-        tc::mbar_init(&ctl->fin, mode == kFwdLast ? 3 : 2);
+        for (int i = 0; i < 8; ++i) tc::mbar_init(&ctl->qbar[i / 4][i % 4], EPW);
+        tc::mbar_init(&ctl->fin, 2);
         tc::mbar_init(&ctl->never, 1);
         ctl->abort = 0;
         tc::fence_mbar_init();
     }
-    gelu_stage(ctl->gelu);
     static_assert(sizeof(RCtl) <= kRCtlBytes, "control block");
     __syncthreads();
 
@@ -455,13 +438,13 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
             const int co = e % C, kc = (e / C) % KC, tap = e / (C * KC);
             wdst[((tap % 3) * KC + kc) * N3 + (tap / 3) * C + co] = wsrc[e];
         }
-        if constexpr (mode == kFwdLast)
-            for (int e = tid - 32; e < 16 * C; e += blockDim.x - 32) {
-                const int tap = (e / 8) % 16, c = e / 128 * 8 + e % 8;
-                reinterpret_cast<__nv_bfloat16*>(wl_tile)[e] = __float2bfloat16_rn(tap < 9 ? wlast[c * 9 + tap] : 0.f);
-            }
         tc::fence_proxy_async_smem();
         if (tid - 32 < C) ctl->bias[tid - 32] = (mode != kDgrad) ? bias[tid - 32] : 0.f;
+        if constexpr (mode == kFwdLast)
+            for (int e = tid - 32; e < 10 * C; e += blockDim.x - 32) {
+                const int tap = e % 10, c = e / 10;
+                ctl->wl[e] = tap < 9 ? bf16r(wlast[c * 9 + tap]) : 0.f;
+            }
         if (warp == 1) tc::tmem_alloc(&ctl->tmem, 512u);
         tc::fence_before_sync();
         tc::bar_sync(1, blockDim.x - 32);
@@ -516,34 +499,10 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
                 tc::mma_commit(&ctl->fin);
                 tc::mbar_wait_bounded(&ctl->fin, 0, kTcSpin);
             }
-        } else if (mode == kFwdLast && warp == 3 + 4 * EPW) {
-            // ---- projection: a row's activations times the nine taps
-            if (lane == 0) {
-                const uint32_t idesc = tc::idesc_bf16_f32(128, 16);
-                const uint64_t a_hi = tc::smem_desc(0, 128 * 16, 128), b_hi = tc::smem_desc(0, 16 * 16, 128);
-                const uint32_t act_u = tc::smem_u32(act_buf) >> 4, wl_u = tc::smem_u32(wl_tile) >> 4;
-                const int rows = int(u1 - u0);
-                for (int r = 0; r < rows; ++r) {
-                    const int par = r & 1;
-                    if (!p_wait(&ctl->pfull[par], uint32_t(r >> 1) & 1u, abort_flag, status)) break;
-                    tc::fence_after_sync();
-                    for (int ks = 0; ks < C / 16; ++ks)
-                        tc::mma_bf16(tmem + uint32_t(par * DCOLS + N3),
-                                     a_hi | uint64_t(act_u + uint32_t(par) * (r_act_bytes(C) >> 4) + uint32_t(2 * ks) * 128u),
-                                     b_hi | uint64_t(wl_u + uint32_t(2 * ks) * 16u), idesc, ks != 0);
-                    tc::mma_commit(&ctl->pdone[par]);
-                }
-                tc::mma_commit(&ctl->fin);
-                tc::mbar_wait_bounded(&ctl->fin, 0, kTcSpin);
-            }
         } else if (warp >= 3) {
             // ---- epilogue
             const int q = warp & 3;         // TMEM lane quarter: pixels 32 q .. 32 q + 31
             const int g = (warp - 3) >> 2;  // chunk group: chunks g CPW .. g CPW + CPW - 1
-            // with two chunks a warp there are no registers for them beside P and
-            // Pn: they are read again for each chunk (five broadcast loads)
-            GeluK gk;
-            if constexpr (CPW == 1) gk = gelu_load(ctl->gelu);
             const f32x2* bias2 = reinterpret_cast<const f32x2*>(ctl->bias);
             f32x2 P[CPW][4], Pn[CPW][4];  // partial sums of output rows y and y + 1, channel pairs
 #pragma unroll
@@ -554,115 +513,124 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
             RowCursor cur(u0, n, NB);
             int rows_done = 0;
             bool ok = true;
-            float* map_row = nullptr;  // kFwdLast: this lane's pixel of the previous row in the first map
-            // the maps of row `r` from TMEM: warp g < 3 of a quarter stores taps 3 g .. 3 g + 2
-            auto store_maps = [&](int r) {
-                if (!p_wait(&ctl->pdone[r & 1], uint32_t(r >> 1) & 1u, abort_flag, status)) return false;
-                if (g < 3) {
-                    uint32_t v[4];
+            for (long long u = u0; u < u1 && ok; ++u, cur.next()) {
+                const int y = cur.y;
+                const long long f = cur.f;
+                const bool start = (u == u0) || (y == 0);
+                const size_t pix = size_t(y) * n + size_t(cur.cb * 128 + q * 32 + lane);
+                for (int k = start ? 0 : 2; k < 3; ++k, dp.next()) {
+                    const int ds = dp.idx;
+                    if (!(ok = p_wait(&ctl->dfull[ds], dp.phase, abort_flag, status))) break;
                     tc::fence_after_sync();
-                    tc::tmem_ld4(tmem + (uint32_t(q * 32) << 16) + uint32_t((r & 1) * DCOLS + N3 + 3 * g), v);
-                    tc::tmem_wait_ld();
-                    tc::fence_before_sync();
+                    const uint32_t trow = tmem + (uint32_t(q * 32) << 16) + uint32_t(ds * DCOLS);
+                    f32x2 pt2[5];  // kFwdLast: the nine-tap projection, tap pairs
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) map_row[size_t(3 * g + t) * nn] = __uint_as_float(v[t]);
-                }
-                return true;
-            };
-            static_assert(mode != kFwdLast || (EPW == 4 && DCOLS >= N3 + 16), "projection columns and map warps");
-            const size_t kc_stride = nn * 8;
-            size_t off = 0;  // this lane's pixel of output row y in chunk g CPW
-            // One input row of the stream; FIN: it completes output row y.
-            auto take = [&](auto fin_tag) {
-                constexpr bool FIN = decltype(fin_tag)::value;
-                ulonglong2 zz[CPW][2];
-                if constexpr (FIN && mode == kDgrad) {  // in flight while the MMAs finish
+                    for (int m = 0; m < 5; ++m) pt2[m] = f2(0.f, 0.f);
 #pragma unroll
-                    for (int c = 0; c < CPW; ++c)
+                    for (int c = 0; c < CPW; ++c) {
+                        const int kc = g * CPW + c;
+                        uint32_t v[3][8];
 #pragma unroll
-                        for (int h = 0; h < 2; ++h)
-                            zz[c][h] = reinterpret_cast<const ulonglong2*>(zio + off + c * kc_stride)[h];
-                }
-                const int ds = dp.idx;
-                if (!p_wait(&ctl->dfull[ds], dp.phase, abort_flag, status)) return false;
-                tc::fence_after_sync();
-                const uint32_t trow = tmem + (uint32_t(q * 32) << 16) + uint32_t(ds * DCOLS + g * CPW * 8);
+                        for (int dy = 0; dy < 3; ++dy) tc::tmem_ld8(trow + uint32_t(dy * C + kc * 8), v[dy]);
+                        tc::tmem_wait_ld();
+                        if (c == CPW - 1) {
+                            // the slot is in registers: the MMA issuer may refill it
+                            tc::fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0) tc::mbar_arrive(&ctl->dempty[ds]);
+                        }
+                        f32x2 d[3][4];
 #pragma unroll
-                for (int c = 0; c < CPW; ++c) {
-                    const int kc = g * CPW + c;
-                    uint32_t v[3][8];
+                        for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
-                    for (int dy = 0; dy < 3; ++dy) tc::tmem_ld8(trow + uint32_t(dy * C + c * 8), v[dy]);
-                    tc::tmem_wait_ld();
-                    if (c == CPW - 1) {
-                        // the slot is in registers: the MMA issuer may refill it
-                        tc::fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(&ctl->dempty[ds]);
-                    }
-                    f32x2 d[3][4];
+                            for (int e = 0; e < 4; ++e)
+                                d[dy][e] = f2(__uint_as_float(v[dy][2 * e]), __uint_as_float(v[dy][2 * e + 1]));
+                        if (k == 2) {
+                            // output row y is complete: ((D(y-1)[0] + b) + D(y)[1]) + D(y+1)[2]
+                            const size_t off = ((size_t(f) * KC + kc) * nn + pix) * 8;
+                            f32x2 z[4];
 #pragma unroll
-                    for (int dy = 0; dy < 3; ++dy)
+                            for (int e = 0; e < 4; ++e) z[e] = f2_add(P[c][e], d[2][e]);
+                            uint32_t packed[4];
+                            if constexpr (mode != kDgrad) {
+                                float a8[8];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            d[dy][e] = f2(__uint_as_float(v[dy][2 * e]), __uint_as_float(v[dy][2 * e + 1]));
-                    f32x2 z[4];
+                                for (int e = 0; e < 4; ++e) {
+                                    float a0, a1;
+                                    f2split(act2<ACT>(z[e]), a0, a1);
+                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
+                                    packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
+                                    if constexpr (mode == kFwdLast) {
+                                        a8[2 * e] = __low2float(hh);
+                                        a8[2 * e + 1] = __high2float(hh);
+                                    }
+                                }
+                                if (zio) {
+                                    f32x2* z2 = reinterpret_cast<f32x2*>(zio + off);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if constexpr (FIN) z[e] = f2_add(P[c][e], d[2][e]);
-                        P[c][e] = f2_add(Pn[c][e], d[1][e]);
-                        if constexpr (mode == kDgrad) Pn[c][e] = d[0][e];
-                        else Pn[c][e] = f2_add(d[0][e], bias2[kc * 4 + e]);  // the bias enters first
-                    }
-                    if constexpr (FIN) {
-                        // output row y is complete: ((D(y-1)[0] + b) + D(y)[1]) + D(y+1)[2]
-                        uint32_t packed[4];
-                        if constexpr (CPW > 1 && mode != kDgrad) gk = gelu_load(ctl->gelu);
+                                    for (int e = 0; e < 4; ++e) z2[e] = z[e];
+                                }
+                                if constexpr (mode == kFwdLast) {
+                                    // channels in order, taps in pairs: each tap's sum is the
+                                    // same fma chain as one tap at a time
+#pragma unroll
+                                    for (int i = 0; i < 8; ++i) {
+                                        const f32x2* w2 = reinterpret_cast<const f32x2*>(ctl->wl + (kc * 8 + i) * 10);
+                                        const f32x2 ai = f2(a8[i], a8[i]);
+#pragma unroll
+                                        for (int m = 0; m < 5; ++m) pt2[m] = f2_fma(w2[m], ai, pt2[m]);
+                                    }
+                                }
+                            } else {
+                                const ulonglong2 za = reinterpret_cast<const ulonglong2*>(zio + off)[0];
+                                const ulonglong2 zb = reinterpret_cast<const ulonglong2*>(zio + off)[1];
+                                const f32x2 zz[4] = {za.x, za.y, zb.x, zb.y};
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    float a0, a1;
+                                    f2split(f2_mul(z[e], act_grad2<ACT>(zz[e])), a0, a1);
+                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
+                                    packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
+                                }
+                            }
+                            // kFwdLast stores the activations only for training (zio)
+                            if (mode != kFwdLast || zio)
+                                *reinterpret_cast<uint4*>(out + off) =
+                                    make_uint4(packed[0], packed[1], packed[2], packed[3]);
+                        }
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            f32x2 a;
-                            if constexpr (mode == kDgrad)
-                                a = f2_mul(z[e], act_grad2<ACT>(e % 2 ? zz[c][e / 2].y : zz[c][e / 2].x));
-                            else a = act2<ACT>(z[e], gk);
-                            float a0, a1;
-                            f2split(a, a0, a1);
-                            const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
-                            packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
+                            P[c][e] = f2_add(Pn[c][e], d[1][e]);
+                            if constexpr (mode == kDgrad) Pn[c][e] = d[0][e];
+                            else Pn[c][e] = f2_add(d[0][e], bias2[kc * 4 + e]);  // the bias enters first
                         }
-                        const uint4 o = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                        if (mode != kDgrad && zio) {
-                            ulonglong2* z2 = reinterpret_cast<ulonglong2*>(zio + off + c * kc_stride);
-                            z2[0] = make_ulonglong2(z[0], z[1]);
-                            z2[1] = make_ulonglong2(z[2], z[3]);
-                        }
-                        // buffer r % 2 is free: the projection of row r - 2 was waited for
-                        if constexpr (mode == kFwdLast)
-                            *reinterpret_cast<uint4*>(act_buf + (rows_done & 1) * r_act_bytes(C) +
-                                                      (kc * 128 + q * 32 + lane) * 16) = o;
-                        // kFwdLast stores the activations only for training (zio)
-                        if (mode != kFwdLast || zio) *reinterpret_cast<uint4*>(out + off + c * kc_stride) = o;
                     }
+                    if (mode == kFwdLast && k == 2) {
+                        // the quarter's EPW partial projections, summed in warp order
+                        const int par = rows_done & 1;
+                        float* sc = scratch + size_t(par * 4 + q) * (4 * 9 * 32);
+#pragma unroll
+                        for (int m = 0; m < 5; ++m) {
+                            float t0, t1;
+                            f2split(pt2[m], t0, t1);
+                            sc[(g * 9 + 2 * m) * 32 + lane] = t0;
+                            if (m < 4) sc[(g * 9 + 2 * m + 1) * 32 + lane] = t1;
+                        }
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&ctl->qbar[par][q]);
+                        if (!(ok = p_wait(&ctl->qbar[par][q], uint32_t((rows_done >> 1) & 1), abort_flag,
+                                          status)))
+                            break;
+                        for (int tp = g; tp < 9; tp += EPW) {
+                            float s_ = sc[tp * 32 + lane];
+#pragma unroll
+                            for (int w = 1; w < EPW; ++w) s_ = __fadd_rn(s_, sc[(w * 9 + tp) * 32 + lane]);
+                            maps[(size_t(f) * 9 + tp) * nn + pix] = s_;
+                        }
+                    }
+                    if (k == 2) ++rows_done;
                 }
-                dp.next();
-                return true;
-            };
-            for (int left = int(u1 - u0); left > 0; --left, cur.next()) {
-                if (rows_done == 0 || cur.y == 0) {  // a new run of rows: its first two input rows complete none
-                    off = ((size_t(cur.f) * KC + g * CPW) * nn + size_t(cur.y) * n + size_t(cur.cb * 128 + q * 32 + lane)) * 8;
-                    if (!(ok = take(std::false_type{}) && take(std::false_type{}))) break;
-                }
-                if (!(ok = take(std::true_type{}))) break;
-                if constexpr (mode == kFwdLast) {
-                    tc::fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0) tc::mbar_arrive(&ctl->pfull[rows_done & 1]);
-                    if (rows_done > 0 && !(ok = store_maps(rows_done - 1))) break;
-                    map_row = maps + size_t(cur.f) * 9 * nn + size_t(cur.y) * n + size_t(cur.cb * 128 + q * 32 + lane);
-                }
-                off += size_t(n) * 8;
-                ++rows_done;
             }
-            if (mode == kFwdLast && ok && rows_done > 0) store_maps(rows_done - 1);
         }
     }
     tc::fence_before_sync();
@@ -683,7 +651,7 @@ static RShape r_shape_with(int n, int C, int ring_mode, int ds, bool last) {
     const int dmax = std::min(kRMaxD, 512 / r_dcols(C));
     s.DS = ds ? ds : dmax;
     if (s.DS < 2 || s.DS > dmax) return RShape{};
-    const size_t fixed = size_t(9) * C * C * 2 + kRCtlBytes + (last ? r_last_bytes(C) : 0);
+    const size_t fixed = size_t(9) * C * C * 2 + kRCtlBytes + (last ? kRScratchBytes : 0);
     int ring = int((size_t(227) * 1024 - fixed) / r_slot_bytes(C));
     ring = std::min(ring, kRMaxRing);
     if (ring_mode == 1) ring = std::min(ring, 12);
@@ -789,7 +757,7 @@ static int launch_rows_mode(const RShape& s, int n, int batch, const __nv_bfloat
     }
     const long long units = (long long)batch * (n / 128) * n;
     const int grid = int(units < num_sms() ? units : num_sms());
-    kern<<<grid, RGeom<C, MODE>::THREADS, s.smem, st>>>(in, out, w, bias, n, batch, s.RING, s.DS, zio, status,
+    kern<<<grid, RGeom<C>::THREADS, s.smem, st>>>(in, out, w, bias, n, batch, s.RING, s.DS, zio, status,
                                                   g_test_stall, wlast, maps);
     ACPR_LAUNCH_CHECK();
     return AC_OK;
