@@ -100,6 +100,30 @@ __device__ __forceinline__ f32x2 act2(f32x2 x) {
     }
 }
 
+// First layer (1 -> C): weights (bf16-rounded) and bias of an output channel as
+// ten pairs of equal values in shared memory, read as five 16-byte vectors,
+// for two adjacent pixels as the lanes of the paired instructions.
+template <int C>
+__device__ __forceinline__ void first_weights(f32x2* ws, const float* __restrict__ W, const float* __restrict__ bias) {
+    for (int i = threadIdx.x; i < C * 10; i += blockDim.x) {
+        const float v = i % 10 < 9 ? bf16r(W[i / 10 * 9 + i % 10]) : bias[i / 10];
+        ws[i] = f2(v, v);
+    }
+}
+// The taps in order from zero, then the bias.
+__device__ __forceinline__ f32x2 first_pair(const f32x2* ws, int o, const f32x2 (&vp)[3][3]) {
+    const ulonglong2* w = reinterpret_cast<const ulonglong2*>(ws + o * 10);
+    f32x2 s = f2(0.f, 0.f);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const ulonglong2 q = w[m];
+        s = f2_fma(q.x, vp[2 * m / 3][2 * m % 3], s);
+        s = f2_fma(q.y, vp[(2 * m + 1) / 3][(2 * m + 1) % 3], s);
+    }
+    const ulonglong2 q = w[4];
+    return f2_add(f2_fma(q.x, vp[2][2], s), q.y);
+}
+
 int check_cnn(const cnn_desc* d);
 int coarse_step(const cnn_desc* d, int n, int batch, const void* u_in, void* u_out, cudaStream_t st);
 // Batch entry b reads the field at u_in + in_map[b] * in_bs and writes the
@@ -121,9 +145,6 @@ int last_layer_bf16(const cnn_desc* d, int n, int batch, const __nv_bfloat16* a,
 size_t packed_hidden_bytes(const cnn_desc* d);
 int pack_hidden_weights(const cnn_desc* d, cudaStream_t st);
 
-// Hidden layer l (1 <= l <= layers - 2) on the tensor cores:
-// in/out are [batch][C/8][n][n][8] bf16.  Returns AC_ERR_UNSUPPORTED when the
-// shape has no tensor-core kernel.
 // Derivative of act_apply: 1 - tanh^2, or Phi(x) + x phi(x).
 // Phi(x) + x phi(x) with Phi as in gelu2 and one 2^(-x^2 log2(e) / 2) for both
 // terms; the scalar form has the same roundings as the paired one.
@@ -210,6 +231,9 @@ int conv_check_status_uncaptured(int* status, cudaStream_t st);
 // waits on an mbarrier that nothing arrives on, for `polls` polls.
 void set_test_stall(int polls);
 
+// Hidden layer l (1 <= l <= layers - 2) on the tensor cores:
+// in/out are [batch][C/8][n][n][8] bf16.  Returns AC_ERR_UNSUPPORTED when the
+// shape has no tensor-core kernel.
 int hidden_layer_bf16(const cnn_desc* d, int l, int n, int batch, const __nv_bfloat16* in,
                       __nv_bfloat16* out, const float* w_master, const float* bias, int* status, cudaStream_t st,
                       float* zsave = nullptr);

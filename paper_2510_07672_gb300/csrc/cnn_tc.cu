@@ -21,6 +21,7 @@
 // conv_check_status() reports as AC_ERR_TIMEOUT.
 // Fields with n >= 128 take the persistent, warp-specialised kernel below.
 #include <algorithm>
+#include <type_traits>
 
 #include "cnn.cuh"
 #include "tc_pipe.cuh"
@@ -376,11 +377,12 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
 
     if (warp == 0) {
         // ---- producer warp: starts at once; the other warps stage the weights
-        // meanwhile.  Per streamed row and chunk plane lane 0 issues one bulk
-        // copy from the first to the last pixel that lies in the row (guard
-        // pixels included where they are interior); a wrapped guard pixel is a
-        // 16-byte cp.async by lane kc (a 16-byte bulk copy costs the copy
-        // engine about as much as a 2 KB one).  Every lane then arrives on
+        // meanwhile.  Per streamed row lane kc issues one bulk copy of chunk
+        // plane kc from the first to the last pixel that lies in the row (guard
+        // pixels included where they are interior; one lane issuing them all
+        // cost a C = 32 layer 4 us of 53, 16 fields of 256^2); a wrapped guard
+        // pixel is a 16-byte cp.async by lane kc (a 16-byte bulk copy costs the
+        // copy engine about as much as a 2 KB one).  Every lane then arrives on
         // full[slot] once its cp.async copies have landed.
         long long j = 0;
         RingPos rp(RING);
@@ -407,12 +409,11 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
                 }
                 unsigned char* dst = ring + size_t(slot) * SLOT;
                 const __nv_bfloat16* src = in + (size_t(f) * KC * nn + size_t(yin) * n) * 8;
-                if (lane == 0) {
-                    tc::mbar_arrive_expect_tx(&ctl->full[slot], uint32_t(KC) * bbytes);
-                    for (int kc = 0; kc < KC; ++kc)
-                        tc::bulk_g2s(dst + size_t(kc) * PLANE + boff, src + (size_t(kc) * nn + size_t(bx)) * 8, bbytes,
-                                     &ctl->full[slot]);
-                }
+                if (lane == 0) tc::mbar_arrive_expect_tx(&ctl->full[slot], uint32_t(KC) * bbytes);
+                __syncwarp();
+                if (lane < KC)
+                    tc::bulk_g2s(dst + size_t(lane) * PLANE + boff, src + (size_t(lane) * nn + size_t(bx)) * 8, bbytes,
+                                 &ctl->full[slot]);
                 if (lane < KC) {
                     unsigned char* d = dst + size_t(lane) * PLANE;
                     const __nv_bfloat16* r = src + size_t(lane) * nn * 8;
@@ -512,124 +513,142 @@ conv_rows_tc(const __nv_bfloat16* __restrict__ in, __nv_bfloat16* __restrict__ o
             RingPos dp(DS);
             RowCursor cur(u0, n, NB);
             int rows_done = 0;
-            bool ok = true;
-            for (long long u = u0; u < u1 && ok; ++u, cur.next()) {
-                const int y = cur.y;
-                const long long f = cur.f;
-                const bool start = (u == u0) || (y == 0);
-                const size_t pix = size_t(y) * n + size_t(cur.cb * 128 + q * 32 + lane);
-                for (int k = start ? 0 : 2; k < 3; ++k, dp.next()) {
-                    const int ds = dp.idx;
-                    if (!(ok = p_wait(&ctl->dfull[ds], dp.phase, abort_flag, status))) break;
-                    tc::fence_after_sync();
-                    const uint32_t trow = tmem + (uint32_t(q * 32) << 16) + uint32_t(ds * DCOLS);
-                    f32x2 pt2[5];  // kFwdLast: the nine-tap projection, tap pairs
+            const size_t kc_stride = nn * 8;
+            size_t off = 0;  // this lane's pixel of output row y in chunk g CPW
+            // One input row of the stream; FIN: it completes output row y.
+            auto take = [&](auto fin_tag) {
+                constexpr bool FIN = decltype(fin_tag)::value;
+                ulonglong2 zz[CPW][2];
+                if constexpr (FIN && mode == kDgrad) {
+                    // in flight while the MMAs finish: a C = 64 layer of 16 fields of
+                    // 256^2 130 -> 107 us
 #pragma unroll
-                    for (int m = 0; m < 5; ++m) pt2[m] = f2(0.f, 0.f);
+                    for (int c = 0; c < CPW; ++c)
 #pragma unroll
-                    for (int c = 0; c < CPW; ++c) {
-                        const int kc = g * CPW + c;
-                        uint32_t v[3][8];
+                        for (int h = 0; h < 2; ++h)
+                            zz[c][h] = reinterpret_cast<const ulonglong2*>(zio + off + c * kc_stride)[h];
+                }
+                const int ds = dp.idx;
+                if (!p_wait(&ctl->dfull[ds], dp.phase, abort_flag, status)) return false;
+                tc::fence_after_sync();
+                const uint32_t trow = tmem + (uint32_t(q * 32) << 16) + uint32_t(ds * DCOLS + g * CPW * 8);
+                f32x2 pt2[5];  // kFwdLast: the nine-tap projection, tap pairs
 #pragma unroll
-                        for (int dy = 0; dy < 3; ++dy) tc::tmem_ld8(trow + uint32_t(dy * C + kc * 8), v[dy]);
-                        tc::tmem_wait_ld();
-                        if (c == CPW - 1) {
-                            // the slot is in registers: the MMA issuer may refill it
-                            tc::fence_before_sync();
-                            __syncwarp();
-                            if (lane == 0) tc::mbar_arrive(&ctl->dempty[ds]);
-                        }
-                        f32x2 d[3][4];
+                for (int m = 0; m < 5; ++m) pt2[m] = f2(0.f, 0.f);
 #pragma unroll
-                        for (int dy = 0; dy < 3; ++dy)
+                for (int c = 0; c < CPW; ++c) {
+                    const int kc = g * CPW + c;
+                    uint32_t v[3][8];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                d[dy][e] = f2(__uint_as_float(v[dy][2 * e]), __uint_as_float(v[dy][2 * e + 1]));
-                        if (k == 2) {
-                            // output row y is complete: ((D(y-1)[0] + b) + D(y)[1]) + D(y+1)[2]
-                            const size_t off = ((size_t(f) * KC + kc) * nn + pix) * 8;
-                            f32x2 z[4];
+                    for (int dy = 0; dy < 3; ++dy) tc::tmem_ld8(trow + uint32_t(dy * C + c * 8), v[dy]);
+                    tc::tmem_wait_ld();
+                    if (c == CPW - 1) {
+                        // the slot is in registers: the MMA issuer may refill it
+                        tc::fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) tc::mbar_arrive(&ctl->dempty[ds]);
+                    }
+                    f32x2 d[3][4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) z[e] = f2_add(P[c][e], d[2][e]);
-                            uint32_t packed[4];
-                            if constexpr (mode != kDgrad) {
-                                float a8[8];
+                    for (int dy = 0; dy < 3; ++dy)
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    float a0, a1;
-                                    f2split(act2<ACT>(z[e]), a0, a1);
-                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
-                                    packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
-                                    if constexpr (mode == kFwdLast) {
-                                        a8[2 * e] = __low2float(hh);
-                                        a8[2 * e + 1] = __high2float(hh);
-                                    }
-                                }
-                                if (zio) {
-                                    f32x2* z2 = reinterpret_cast<f32x2*>(zio + off);
+                        for (int e = 0; e < 4; ++e)
+                            d[dy][e] = f2(__uint_as_float(v[dy][2 * e]), __uint_as_float(v[dy][2 * e + 1]));
+                    f32x2 z[4];
 #pragma unroll
-                                    for (int e = 0; e < 4; ++e) z2[e] = z[e];
-                                }
-                                if constexpr (mode == kFwdLast) {
-                                    // channels in order, taps in pairs: each tap's sum is the
-                                    // same fma chain as one tap at a time
-#pragma unroll
-                                    for (int i = 0; i < 8; ++i) {
-                                        const f32x2* w2 = reinterpret_cast<const f32x2*>(ctl->wl + (kc * 8 + i) * 10);
-                                        const f32x2 ai = f2(a8[i], a8[i]);
-#pragma unroll
-                                        for (int m = 0; m < 5; ++m) pt2[m] = f2_fma(w2[m], ai, pt2[m]);
-                                    }
-                                }
-                            } else {
-                                const ulonglong2 za = reinterpret_cast<const ulonglong2*>(zio + off)[0];
-                                const ulonglong2 zb = reinterpret_cast<const ulonglong2*>(zio + off)[1];
-                                const f32x2 zz[4] = {za.x, za.y, zb.x, zb.y};
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    float a0, a1;
-                                    f2split(f2_mul(z[e], act_grad2<ACT>(zz[e])), a0, a1);
-                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
-                                    packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
-                                }
-                            }
-                            // kFwdLast stores the activations only for training (zio)
-                            if (mode != kFwdLast || zio)
-                                *reinterpret_cast<uint4*>(out + off) =
-                                    make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                        }
+                    for (int e = 0; e < 4; ++e) {
+                        if constexpr (FIN) z[e] = f2_add(P[c][e], d[2][e]);
+                        P[c][e] = f2_add(Pn[c][e], d[1][e]);
+                        if constexpr (mode == kDgrad) Pn[c][e] = d[0][e];
+                        else Pn[c][e] = f2_add(d[0][e], bias2[kc * 4 + e]);  // the bias enters first
+                    }
+                    if constexpr (FIN) {
+                        // output row y is complete: ((D(y-1)[0] + b) + D(y)[1]) + D(y+1)[2]
+                        uint32_t packed[4];
+                        float a8[8];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
-                            P[c][e] = f2_add(Pn[c][e], d[1][e]);
-                            if constexpr (mode == kDgrad) Pn[c][e] = d[0][e];
-                            else Pn[c][e] = f2_add(d[0][e], bias2[kc * 4 + e]);  // the bias enters first
+                            f32x2 a;
+                            // two chunks a warp leave no registers for the paired forms'
+                            // constants: one lane at a time, the same roundings
+                            if constexpr (mode == kDgrad) {
+                                const f32x2 zp = e % 2 ? zz[c][e / 2].y : zz[c][e / 2].x;
+                                if constexpr (CPW > 1) {
+                                    float p0, p1;
+                                    f2split(zp, p0, p1);
+                                    a = f2_mul(z[e], f2(act_grad_c<ACT>(p0), act_grad_c<ACT>(p1)));
+                                } else {
+                                    a = f2_mul(z[e], act_grad2<ACT>(zp));
+                                }
+                            } else if constexpr (mode == kFwdLast && CPW > 1) {
+                                float p0, p1;
+                                f2split(z[e], p0, p1);
+                                a = f2(act_c<ACT>(p0), act_c<ACT>(p1));
+                            } else {
+                                a = act2<ACT>(z[e]);
+                            }
+                            float a0, a1;
+                            f2split(a, a0, a1);
+                            const __nv_bfloat162 hh = __floats2bfloat162_rn(a0, a1);
+                            packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
+                            a8[2 * e] = __low2float(hh);
+                            a8[2 * e + 1] = __high2float(hh);
                         }
-                    }
-                    if (mode == kFwdLast && k == 2) {
-                        // the quarter's EPW partial projections, summed in warp order
-                        const int par = rows_done & 1;
-                        float* sc = scratch + size_t(par * 4 + q) * (4 * 9 * 32);
+                        if (mode != kDgrad && zio) {
+                            f32x2* z2 = reinterpret_cast<f32x2*>(zio + off + c * kc_stride);
 #pragma unroll
-                        for (int m = 0; m < 5; ++m) {
-                            float t0, t1;
-                            f2split(pt2[m], t0, t1);
-                            sc[(g * 9 + 2 * m) * 32 + lane] = t0;
-                            if (m < 4) sc[(g * 9 + 2 * m + 1) * 32 + lane] = t1;
+                            for (int e = 0; e < 4; ++e) z2[e] = z[e];
                         }
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(&ctl->qbar[par][q]);
-                        if (!(ok = p_wait(&ctl->qbar[par][q], uint32_t((rows_done >> 1) & 1), abort_flag,
-                                          status)))
-                            break;
-                        for (int tp = g; tp < 9; tp += EPW) {
-                            float s_ = sc[tp * 32 + lane];
+                        if constexpr (mode == kFwdLast) {
+                            // channels in order, taps in pairs: each tap's sum is the
+                            // same fma chain as one tap at a time
 #pragma unroll
-                            for (int w = 1; w < EPW; ++w) s_ = __fadd_rn(s_, sc[(w * 9 + tp) * 32 + lane]);
-                            maps[(size_t(f) * 9 + tp) * nn + pix] = s_;
+                            for (int i = 0; i < 8; ++i) {
+                                const f32x2* w2 = reinterpret_cast<const f32x2*>(ctl->wl + (kc * 8 + i) * 10);
+                                const f32x2 ai = f2(a8[i], a8[i]);
+#pragma unroll
+                                for (int m = 0; m < 5; ++m) pt2[m] = f2_fma(w2[m], ai, pt2[m]);
+                            }
                         }
+                        // kFwdLast stores the activations only for training (zio)
+                        if (mode != kFwdLast || zio)
+                            *reinterpret_cast<uint4*>(out + off + c * kc_stride) =
+                                make_uint4(packed[0], packed[1], packed[2], packed[3]);
                     }
-                    if (k == 2) ++rows_done;
                 }
+                if constexpr (FIN && mode == kFwdLast) {
+                    // the quarter's EPW partial projections, summed in warp order
+                    const int par = rows_done & 1;
+                    float* sc = scratch + size_t(par * 4 + q) * (4 * 9 * 32);
+#pragma unroll
+                    for (int m = 0; m < 5; ++m) {
+                        float t0, t1;
+                        f2split(pt2[m], t0, t1);
+                        sc[(g * 9 + 2 * m) * 32 + lane] = t0;
+                        if (m < 4) sc[(g * 9 + 2 * m + 1) * 32 + lane] = t1;
+                    }
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(&ctl->qbar[par][q]);
+                    if (!p_wait(&ctl->qbar[par][q], uint32_t((rows_done >> 1) & 1), abort_flag, status)) return false;
+                    float* map = maps + size_t(cur.f) * 9 * nn + size_t(cur.y) * n + size_t(cur.cb * 128 + q * 32 + lane);
+                    for (int tp = g; tp < 9; tp += EPW) {
+                        float s_ = sc[tp * 32 + lane];
+#pragma unroll
+                        for (int w = 1; w < EPW; ++w) s_ = __fadd_rn(s_, sc[(w * 9 + tp) * 32 + lane]);
+                        map[size_t(tp) * nn] = s_;
+                    }
+                }
+                dp.next();
+                return true;
+            };
+            for (int left = int(u1 - u0); left > 0; --left, cur.next()) {
+                if (rows_done == 0 || cur.y == 0) {  // a new run of rows: its first two input rows complete none
+                    off = ((size_t(cur.f) * KC + g * CPW) * nn + size_t(cur.y) * n + size_t(cur.cb * 128 + q * 32 + lane)) * 8;
+                    if (!take(std::false_type{}) || !take(std::false_type{})) break;
+                }
+                if (!take(std::true_type{})) break;
+                off += size_t(n) * 8;
+                ++rows_done;
             }
         }
     }

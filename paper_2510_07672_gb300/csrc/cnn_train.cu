@@ -86,10 +86,8 @@ template <int C, int ACT>
 __global__ void __launch_bounds__(128) first_fwd_save_kernel(const float* __restrict__ u, __nv_bfloat16* __restrict__ a1,
                                                              float* __restrict__ z0, const float* __restrict__ W,
                                                              const float* __restrict__ bias, int batch, int n) {
-    __shared__ f32x2 ws[C * 9];
-    __shared__ float bs[C];
-    pair_weights<C>(ws, W);
-    for (int i = threadIdx.x; i < C; i += blockDim.x) bs[i] = bias[i];
+    __shared__ __align__(16) f32x2 ws[C * 10];
+    first_weights<C>(ws, W, bias);
     __syncthreads();
     const long long pix = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 2;
     const long long nn = (long long)n * n;
@@ -106,10 +104,7 @@ __global__ void __launch_bounds__(128) first_fwd_save_kernel(const float* __rest
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int o = kc * 8 + i;
-            f32x2 s2 = f2(0.f, 0.f);
-#pragma unroll
-            for (int t = 0; t < 9; ++t) s2 = f2_fma(ws[o * 9 + t], vp[t / 3][t % 3], s2);
-            s2 = f2_add(s2, f2(bs[o], bs[o]));
+            const f32x2 s2 = first_pair(ws, o, vp);
             f2split(s2, z8[0][i], z8[1][i]);
             float a0, a1v;
             f2split(act2<ACT>(s2), a0, a1v);
