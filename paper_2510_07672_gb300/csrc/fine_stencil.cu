@@ -22,9 +22,12 @@
 //
 // Mass-conserving model: beta shifts every cell alike, so u' = p(Lap) r + shift
 // with the shift that puts the mean at the field's entry mean: mean(p(Lap) r) =
-// mean(r) / a.  The sum of r over the field is formed in integers (fixed point,
-// 2^-24 for float32 and two words for float64), which makes it independent of
-// the order and of the split.
+// mean(r) / a.  The sum of r over the field is formed in integers (fixed point:
+// one word for float32, two for float64), which makes it independent of the
+// order and of the split.  In float32 the unit follows the largest cell, so the
+// mean is as exact for small, large, growing and decaying fields as for those of
+// size one; only a field that outgrows its unit, 2^14-fold in 8 steps, becomes
+// not a number.
 //
 // Bound: FP32 (float64: FP64) issue.  Measured, Fourier kernel -> this one:
 //   512 fields of 256^2, mass, 100 steps        11.40 -> 1.98 ms (2.21 with scalar instructions and 8x8x4)
@@ -161,7 +164,8 @@ template <int N, int H, int NW, int P, int M>
 struct RegShape {
     static constexpr int W = N / 32, R = NW * H;
     static constexpr size_t HALO = size_t(2) * 2 * NW * M * N;  // floats
-    static constexpr size_t SMEM = HALO * sizeof(float) + size_t(2) * P * NW * sizeof(long long);
+    static constexpr size_t SMEM = HALO * sizeof(float) + size_t(3) * P * NW * sizeof(long long);
+    static constexpr int ROOM = kGroupRoom - log2i(2 * W);  // of a cell of r, in groups of two rows of a lane
     static_assert(R * P == N && H % 2 == 0 && H >= M && N % 32 == 0, "split");
 };
 
@@ -174,6 +178,7 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* halo = reinterpret_cast<float*>(smem_raw);  // [buffer][0: above, 1: below][warp][M][N]
     long long* tot = reinterpret_cast<long long*>(halo + Sh::HALO);  // [buffer][P NW] sums of the warps
+    long long* aux = tot + 2 * P * NW;                               // [P NW] the warps' entry sums, later their maxima
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int rank = 0;
     if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
@@ -202,45 +207,54 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
     const float* above = halo + warp * M * N;
     const float* below = halo + (NW + warp) * M * N;
 
-    long long target = 0;   // sum of r that keeps the entry mean, in 2^-24
+    // mass model: the sum of r that keeps the entry mean, and it in units of 1 / unit
+    double goal = 0.0;
+    long long target = 0, entry = 0;
+    float unit = 1.f, entry_unit = 1.f;
     double msum = 0.0;      // adjoint: this warp's part of the sum of lambda
-    auto publish_total = [&](long long v, int buf) {
-        for (int q = lane; q < P; q += 32) peer<P>(tot, q)[buf * P * NW + rank * NW + warp] = v;
+    auto publish = [&](long long* to, long long v) {
+        for (int q = lane; q < P; q += 32) peer<P>(to, q)[rank * NW + warp] = v;
     };
-    cl_arrive<P>();
-    if constexpr (MASS && !ADJ) {
-        // entry sum, cell by cell
-        long long acc = 0;
-        bool bad = false;
+    auto largest = [&](const long long* from) {
+        unsigned m = 0;
+        for (int i = lane; i < P * NW; i += 32) m = max(m, unsigned(from[i]));
+        return __reduce_max_sync(0xffffffffu, m);
+    };
+    // largest magnitude of the warp's cells, as bits (not that of a NaN, which
+    // the sums below find)
+    auto measure = [&] {
+        float m = 0.f;
 #pragma unroll
         for (int y = 0; y < H; ++y) {
             float v[W];
             from_lane<W>(u[y], v);
 #pragma unroll
-            for (int c = 0; c < W; ++c) {
-                acc += __float2ll_rn(v[c] * kFix);
-                bad |= !(fabsf(v[c]) < 0x1p19f);
-            }
+            for (int c = 0; c < W; ++c) m = fmaxf(m, fabsf(v[c]));
         }
-        acc = warp_sum_s64(acc);
-        if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
+        return __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    };
+    cl_arrive<P>();
+    if constexpr (MASS && !ADJ) {
+        const unsigned mine = measure();
         cl_wait<P>();
-        publish_total(acc, 1);
+        publish(tot + P * NW, mine);
         cl_arrive<P>();
         cl_wait<P>();
-        long long t = 0;
-        bool b2 = false;
-        for (int i = lane; i < P * NW; i += 32) {
-            t += tot[P * NW + i];
-            b2 |= tot[P * NW + i] == kBadSum;
+        const unsigned m = largest(tot + P * NW);
+        entry_unit = pow2f(fix_scale(m, kCellRoom));
+        unit = pow2f(fix_scale(__float_as_uint(rhs_bound(__uint_as_float(m), cf.mdt, cf.kappa)), Sh::ROOM));
+        // entry sum, cell by cell
+#pragma unroll
+        for (int y = 0; y < H; ++y) {
+            float v[W];
+            from_lane<W>(u[y], v);
+#pragma unroll
+            for (int c = 0; c < W; ++c) entry += __float2ll_rn(v[c] * entry_unit);
         }
-        t = warp_sum_s64(t);
-        b2 = __any_sync(0xffffffffu, b2);
-        target = b2 ? kBadSum : __double2ll_rn(args.a * double(t));
+        entry = warp_sum_s64(entry);
     } else {
         cl_wait<P>();
     }
-    const float inv_fix = float(cf.inv_sum) * (1.f / kFix);
 
     for (int step = 0; step < it.steps; ++step) {
         const int buf = step & 1;
@@ -268,20 +282,22 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
                 bool bad = false;
 #pragma unroll
                 for (int y = 0; y < H; y += 2) {
-                    const float t = pair_sum<W>(u[y], u[y + 1]);
-                    acc += __float2ll_rn(t * kFix);
-                    bad |= !(fabsf(t) < 0x1p24f);  // 2^13 such sums stay below 2^62
+                    const float t = pair_sum<W>(u[y], u[y + 1]) * unit;
+                    acc += __float2ll_rn(t);
+                    bad |= !(fabsf(t) < 0x1p49f);  // 2^13 such sums stay below 2^62
                 }
                 acc = warp_sum_s64(acc);
                 if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
-                publish_total(acc, buf);
+                publish(tot + buf * P * NW, acc);
+                if (step == 0) publish(aux, entry);
+                else if ((step & (kMeasure - 1)) == 0) publish(aux, measure());
             } else {
                 msum = 0.0;
 #pragma unroll
                 for (int y = 0; y < H; y += 2) msum += double(pair_sum<W>(u[y], u[y + 1]));
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
-                publish_total(__double_as_longlong(msum), buf);
+                publish(tot + buf * P * NW, __double_as_longlong(msum));
             }
         }
         if constexpr (MASS) cl_arrive<P>();
@@ -291,8 +307,14 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
         auto collect = [&]() -> float {
             const long long* tb = tot + buf * P * NW;
             if constexpr (!ADJ) {
+                if (step == 0) {
+                    long long e = 0;
+                    for (int i = lane; i < P * NW; i += 32) e += aux[i];
+                    goal = args.a * double(warp_sum_s64(e)) * double(pow2_inv(entry_unit));
+                    target = __double2ll_rn(goal * double(unit));
+                }
                 long long t = 0;
-                bool bad = target == kBadSum;
+                bool bad = false;
 #pragma unroll
                 for (int i0 = 0; i0 < P * NW; i0 += 32) {
                     const long long v = P * NW % 32 == 0 || i0 + lane < P * NW ? tb[i0 + lane] : 0;
@@ -300,8 +322,12 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
                     bad |= v == kBadSum;
                 }
                 t = warp_sum_s64(t);
-                shift = float(target - t) * inv_fix;
+                shift = float(target - t) * float(cf.inv_sum) * pow2_inv(unit);
                 if (__any_sync(0xffffffffu, bad)) shift = __int_as_float(0x7fffffff);
+                if (step > 0 && (step & (kMeasure - 1)) == 0) {
+                    unit = pow2f(fix_scale(largest(aux), Sh::ROOM));
+                    target = __double2ll_rn(goal * double(unit));
+                }
             } else {
                 double t = 0.0;
                 for (int i = lane; i < P * NW; i += 32) t += __longlong_as_double(tb[i]);

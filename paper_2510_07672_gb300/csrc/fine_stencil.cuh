@@ -145,6 +145,11 @@ __device__ __forceinline__ V rhs(V v, V mdt, V kappa) {
     return vfma(v, vfma(mdt, vmul(v, v), kappa), v);
 }
 
+// Bound of |r| over |u| <= m.
+__device__ __forceinline__ float rhs_bound(float m, float mdt, float kappa) {
+    return m * fmaxf(1.f + kappa, fabsf(fmaf(mdt, m * m, 1.f + kappa)));
+}
+
 // r <- p(Lap) r for the warp's H rows; halo(y, x) gives row y of r outside
 // them (-M <= y < 0 or H <= y < H + M).  Rows stream through the M stages; a
 // stage keeps its last row (p) and the three known neighbours of that row's
@@ -216,8 +221,22 @@ __device__ __forceinline__ void apply_poly(LaneV<W> (&r)[H][Lane<W>::E], const C
     }
 }
 
-constexpr float kFix = 16777216.f;  // 2^24: fixed point of the sums of r
+// Sums of r in integers, exact up to the unit: any order and any split give the
+// same bits.  The unit follows the field: a power of two 2^-scale such that the
+// largest magnitude met, taken over the field at entry and every kMeasure steps,
+// is below 2^room units, so a group's rounding is 2^-30 of that magnitude.  What
+// is left of 62 bits (2^14 or more) is room for growth until the next measurement.
+constexpr int kMeasure = 8;
+constexpr int kCellRoom = 40, kGroupRoom = 30;  // one cell of the entry sum; a group of cells of r
+constexpr float kFix = 16777216.f;  // unit of the sums of fine_tiles.cu
 constexpr long long kBadSum = (long long)(1ULL << 63);
+
+constexpr int log2i(int v) { return v > 1 ? 1 + log2i(v / 2) : 0; }
+__device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) << 23); }  // -126 <= k <= 127
+__device__ __forceinline__ float pow2_inv(float p) { return __uint_as_float((254u << 23) - __float_as_uint(p)); }
+// Scale by which every float of at most the magnitude `bits` (its bits without
+// the sign) is below 2^room.
+__device__ __forceinline__ int fix_scale(unsigned bits, int room) { return min(126, room + 126 - int(bits >> 23)); }
 
 // Sum over the warp's lanes of a 62-bit integer, on every lane.
 __device__ __forceinline__ long long warp_sum_s64(long long v) {
