@@ -24,10 +24,10 @@
 // with the shift that puts the mean at the field's entry mean: mean(p(Lap) r) =
 // mean(r) / a.  The sum of r over the field is formed in integers (fixed point:
 // one word for float32, two for float64), which makes it independent of the
-// order and of the split.  In float32 the unit follows the largest cell, so the
-// mean is as exact for small, large, growing and decaying fields as for those of
-// size one; only a field that outgrows its unit, 2^14-fold in 8 steps, becomes
-// not a number.
+// order and of the split.  The unit follows the largest cell, so the mean is as
+// exact for small, large, growing and decaying fields as for those of size one;
+// only a field that outgrows its unit (float32: 2^14-fold in 8 steps, float64:
+// 2^19-fold in one) becomes not a number.
 //
 // Bound: FP32 (float64: FP64) issue.  Measured, Fourier kernel -> this one:
 //   512 fields of 256^2, mass, 100 steps        11.40 -> 1.98 ms (2.21 with scalar instructions and 8x8x4)
@@ -494,20 +494,37 @@ struct ShShape {
     static constexpr int R = N / P, RH = R + 2 * M, RW = R + 2 * (M - 1);
     static constexpr int K = R * N / kShThreads;  // cells per thread
     static constexpr size_t SMEM =
-        sizeof(T) * N * (size_t(2) * RH + size_t(M > 2 ? 2 : 1) * RW) + size_t(2) * 2 * P * 8 * sizeof(long long);
+        sizeof(T) * N * (size_t(2) * RH + size_t(M > 2 ? 2 : 1) * RW) + size_t(2 * 3 + 2) * P * 8 * sizeof(long long);
     static_assert(R >= M && R * N % kShThreads == 0, "split");
 };
 
-// Exact sum pieces of a float64: x = hi 2^-24 + lo 2^-68 to 2^-69, |x| < 2^26
-// (2^16 cells below 2^20 keep both words below 2^61).
-__device__ __forceinline__ void fix64(double x, long long& hi, long long& lo) {
-    constexpr double m1 = 0x1.8p28, m2 = 0x1.8p-16;
-    const double t = x + m1;
-    const double rem = x - (t - m1);
-    const double t2 = rem + m2;
-    hi += __double_as_longlong(t) - __double_as_longlong(m1);
-    lo += __double_as_longlong(t2) - __double_as_longlong(m2);
-}
+// Exact sum pieces of a float64, in units that follow the field: with the
+// largest magnitude below 2^(e + 1), x = hi 2^(e - 24) + lo 2^(e - 68) to
+// 2^(e - 69), for |x| < 2^(e + 20) (2^16 cells keep both words below 2^61).
+struct Fix64 {
+    int e;
+    double m1, m2;  // adding and subtracting one rounds to its word's unit
+    static __device__ __forceinline__ double pow2(int k) { return __longlong_as_double((long long)(k + 1023) << 52); }
+    static __device__ __forceinline__ double pow2_15(int k) {  // 1.5 2^k
+        return __longlong_as_double((long long)(k + 1023) << 52 | 1LL << 51);
+    }
+    // `key`: high word of the largest magnitude (infinities and NaN: any e)
+    __device__ __forceinline__ explicit Fix64(unsigned key)
+        : e(min(max(int(key >> 20) - 1023, -900), 990)), m1(pow2_15(e + 28)), m2(pow2_15(e - 16)) {}
+    __device__ __forceinline__ void add(double x, long long& hi, long long& lo) const {
+        const double t = x + m1;
+        const double rem = x - (t - m1);
+        const double t2 = rem + m2;
+        hi += __double_as_longlong(t) - __double_as_longlong(m1);
+        lo += __double_as_longlong(t2) - __double_as_longlong(m2);
+    }
+    // not a number where a magnitude left the range
+    __device__ __forceinline__ double value(long long hi, long long lo, unsigned key) const {
+        if (int(key >> 20) - 1023 > min(e + 19, 1009)) return __longlong_as_double(0x7ff8000000000000LL);
+        return double(hi) * pow2(e - 24) + double(lo) * pow2(e - 68);
+    }
+};
+__device__ __forceinline__ unsigned abs_key(double x) { return unsigned(__double2hiint(x)) & kAbsMask; }
 
 template <typename T, int N, int P, int M, bool MASS, bool ADJ>
 __device__ __forceinline__ void stencil_smem_body(const FineArgs& args, const Coef<T, M>& cf, int field) {
@@ -518,7 +535,8 @@ __device__ __forceinline__ void stencil_smem_body(const FineArgs& args, const Co
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* rbuf = reinterpret_cast<T*>(smem_raw);       // [2][RH][N], row 0 is row -M
     T* wbuf = rbuf + 2 * RH * N;                     // [1 or 2][RW][N], row 0 is row -(M-1)
-    long long* tot = reinterpret_cast<long long*>(wbuf + (M > 2 ? 2 : 1) * RW * N);  // [buffer][P WARPS][hi, lo]
+    long long* tot = reinterpret_cast<long long*>(wbuf + (M > 2 ? 2 : 1) * RW * N);  // [buffer][P WARPS][hi, lo, largest]
+    long long* aux = tot + 2 * 3 * P * WARPS;                                         // [P WARPS][hi, lo] of the entry sum
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int rank = 0;
     if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
@@ -536,77 +554,54 @@ __device__ __forceinline__ void stencil_smem_body(const FineArgs& args, const Co
         u[i] = in[tid + i * kShThreads];
         if (traj) traj[tid + i * kShThreads] = u[i];
     }
-    auto publish = [&](long long hi, long long lo, bool bad, int buf) {
-        // integer sums: any order gives the same bits
+    // (integer sums: any order gives the same bits)
+    auto warp_sums = [](long long& hi, long long& lo) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             hi += __shfl_xor_sync(0xffffffffu, hi, o);
             lo += __shfl_xor_sync(0xffffffffu, lo, o);
-        }
-        if (__any_sync(0xffffffffu, bad)) lo = kBadSum;
-        for (int q = lane; q < P; q += 32) {
-            long long* p = peer<P>(tot, q) + ((buf * P + rank) * WARPS + warp) * 2;
-            p[0] = hi;
-            p[1] = lo;
         }
     };
-    // the field's sum; not a number when a cell was out of range
-    auto collect = [&](int buf) -> double {
-        long long hi = 0, lo = 0;
-        bool nan = false;
+    auto publish = [&](long long hi, long long lo, unsigned key, int buf) {
+        key = __reduce_max_sync(0xffffffffu, key);
+        for (int q = lane; q < P; q += 32) {
+            long long* p = peer<P>(tot, q) + ((buf * P + rank) * WARPS + warp) * 3;
+            p[0] = hi;
+            p[1] = lo;
+            p[2] = key;
+        }
+    };
+    auto collect = [&](int buf, long long& hi, long long& lo) -> unsigned {
+        unsigned key = 0;
+        hi = lo = 0;
         for (int i = lane; i < P * WARPS; i += 32) {
-            hi += tot[(buf * P * WARPS + i) * 2];
-            lo += tot[(buf * P * WARPS + i) * 2 + 1];
-            nan |= tot[(buf * P * WARPS + i) * 2 + 1] == kBadSum;
+            const long long* p = tot + (buf * P * WARPS + i) * 3;
+            hi += p[0];
+            lo += p[1];
+            key = max(key, unsigned(p[2]));
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            hi += __shfl_xor_sync(0xffffffffu, hi, o);
-            lo += __shfl_xor_sync(0xffffffffu, lo, o);
-        }
-        if (__any_sync(0xffffffffu, nan)) return __longlong_as_double(0x7ff8000000000000LL);
-        return double(hi) * 0x1p-24 + double(lo) * 0x1p-68;
+        warp_sums(hi, lo);
+        return __reduce_max_sync(0xffffffffu, key);
     };
     cl_arrive<P>();
     cl_wait<P>();
-    double mean = 0.0;
-    bool bad = false;
-    // sums of the cells in fixed point, scaled to [-1, 1]-like sizes for the
-    // adjoint, whose fields have no natural scale
-    double scale = 1.0, inv_scale = 1.0;
+    double mean = 0.0;               // mean of r that keeps the entry mean
+    long long ehi = 0, elo = 0;      // entry sum, in units of ufix
+    unsigned key = 0, ukey = 0;      // largest magnitude of r, of the entry field
     if constexpr (MASS) {
-        if constexpr (ADJ) {
-            // power of two at the field's largest entry
-            T mx = T(0);
 #pragma unroll
-            for (int i = 0; i < K; ++i) mx = fmax(mx, fabs(u[i]));
-            long long e = __double_as_longlong(double(mx));
+        for (int i = 0; i < K; ++i) ukey = max(ukey, abs_key(double(u[i])));
+        publish(0, 0, ukey, 1);
+        cl_arrive<P>();
+        cl_wait<P>();
+        ukey = key = collect(1, ehi, elo);
+        if constexpr (!ADJ) {
+            const double m = __hiloint2double(int(ukey), -1);  // |r| <= m max(1 + kappa, |1 + kappa - dt m^2|) over |u| <= m
+            key = abs_key(m * fmax(1.0 + cf.kappa, fabs(fma(double(cf.mdt), m * m, 1.0 + cf.kappa))));
+            const Fix64 ufix(ukey);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e = max(e, (long long)__shfl_xor_sync(0xffffffffu, e, o));
-            for (int q = lane; q < P; q += 32) peer<P>(tot, q)[(P * WARPS + rank * WARPS + warp) * 2] = e;
-            cl_arrive<P>();
-            cl_wait<P>();
-            e = 0;
-            for (int i = lane; i < P * WARPS; i += 32) e = max(e, tot[(P * WARPS + i) * 2]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) e = max(e, (long long)__shfl_xor_sync(0xffffffffu, e, o));
-            // 2^-exponent, exact; a zero or subnormal field keeps 1
-            const int ex = int(e >> 52) - 1023;
-            if (ex > -1000 && ex < 1000) {
-                scale = __longlong_as_double((long long)(1023 - ex) << 52);
-                inv_scale = __longlong_as_double((long long)(1023 + ex) << 52);
-            }
-        } else {
-            long long hi = 0, lo = 0;
-#pragma unroll
-            for (int i = 0; i < K; ++i) {
-                fix64(double(u[i]), hi, lo);
-                bad |= !(fabs(u[i]) < T(0x1p20));
-            }
-            publish(hi, lo, bad, 1);
-            cl_arrive<P>();
-            cl_wait<P>();
-            mean = collect(1) * (args.a * cf.inv_sum);
+            for (int i = 0; i < K; ++i) ufix.add(double(u[i]), ehi, elo);
+            warp_sums(ehi, elo);
         }
     }
 
@@ -614,6 +609,8 @@ __device__ __forceinline__ void stencil_smem_body(const FineArgs& args, const Co
         const int buf = step & 1;
         T* r = rbuf + buf * RH * N;
         long long hi = 0, lo = 0;
+        const Fix64 fix(key);
+        unsigned largest = 0;
 #pragma unroll
         for (int i = 0; i < K; ++i) {
             const int e = tid + i * kShThreads, y = e / N;
@@ -623,16 +620,34 @@ __device__ __forceinline__ void stencil_smem_body(const FineArgs& args, const Co
             if (y < M) rup[buf * RH * N + (M + R) * N + e] = v;
             if (y >= R - M) rdown[buf * RH * N + e - (R - M) * N] = v;
             if constexpr (MASS) {
-                fix64(double(v) * scale, hi, lo);
-                bad |= !(fabs(double(v) * scale) < 0x1p20);
+                fix.add(double(v), hi, lo);
+                largest = max(largest, abs_key(double(v)));
             }
         }
-        if constexpr (MASS) publish(hi, lo, bad, buf);
+        if constexpr (MASS) {
+            warp_sums(hi, lo);
+            publish(hi, lo, largest, buf);
+            if (!ADJ && step == 0 && lane < P) {
+                long long* p = peer<P>(aux, lane) + (rank * WARPS + warp) * 2;
+                p[0] = ehi;
+                p[1] = elo;
+            }
+        }
         cl_arrive<P>();
         cl_wait<P>();
         T shift = T(0);
         if constexpr (MASS) {
-            const double m = collect(buf) * cf.inv_sum * inv_scale;
+            if (!ADJ && step == 0) {
+                ehi = elo = 0;
+                for (int i = lane; i < P * WARPS; i += 32) {
+                    ehi += aux[i * 2];
+                    elo += aux[i * 2 + 1];
+                }
+                warp_sums(ehi, elo);
+                mean = Fix64(ukey).value(ehi, elo, ukey) * (args.a * cf.inv_sum);
+            }
+            key = collect(buf, hi, lo);
+            const double m = fix.value(hi, lo, key) * cf.inv_sum;
             shift = T(ADJ ? m : mean - m);
         }
         // stages: w_k on rows -(M-1-k) .. R + (M-1-k)

@@ -230,6 +230,7 @@ constexpr int kMeasure = 8;
 constexpr int kCellRoom = 40, kGroupRoom = 30;  // one cell of the entry sum; a group of cells of r
 constexpr float kFix = 16777216.f;  // unit of the sums of fine_tiles.cu
 constexpr long long kBadSum = (long long)(1ULL << 63);
+constexpr unsigned kAbsMask = 0x7fffffffu;
 
 constexpr int log2i(int v) { return v > 1 ? 1 + log2i(v / 2) : 0; }
 __device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) << 23); }  // -126 <= k <= 127

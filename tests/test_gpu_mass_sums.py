@@ -6,6 +6,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+import acpr_inputs as I
 import paper_2510_07672_gb300 as G
 
 pytestmark = pytest.mark.gpu
@@ -66,6 +67,17 @@ def test_flat_fields_stay(n, dims, steps):
     assert np.all(err <= np.spacing(np.abs(np.float32(VALUES)))), err
 
 
+@pytest.mark.parametrize("n,lam", [(32, 8e-4), (64, 8e-4), (128, 3e-3), (256, 8e-3)])
+def test_flat_fields_stay_f64(n, lam):
+    """float64: four ulp (the rounded sums of u and of r, three roundings each,
+    and the last step's two)."""
+    fp = params(n, F64, lam)
+    vals = np.array([0.1, -0.9421, 1.2345e-8, 3e-200])
+    u = torch.tensor(vals, device="cuda").reshape(-1, 1, 1).expand(-1, n, n).contiguous()
+    err = (propagate(fp, 3, u) - u).abs().amax(dim=(1, 2)).cpu().numpy()
+    assert np.all(err <= 4 * np.spacing(np.abs(vals))), err
+
+
 @pytest.mark.parametrize("n,dims", GRIDS32)
 def test_small_fields_keep_their_mean(n, dims):
     """Noise of size 1e-6 about 5e-7: the mean moves by less than the rounding
@@ -76,7 +88,7 @@ def test_small_fields_keep_their_mean(n, dims):
     assert (mean(out) - mean(u)).abs().max().item() <= 2.0 ** -25 * u.abs().max().item()
 
 
-@pytest.mark.parametrize("n,dims,prec", [g + (F32,) for g in GRIDS32])
+@pytest.mark.parametrize("n,dims,prec", [g + (F32,) for g in GRIDS32] + [(32, 2, F64), (64, 2, F64), (256, 2, F64)])
 def test_large_fields(n, dims, prec):
     """Fields of size 2^21 at a step that resolves them: against 64 bits, the
     round-off of the comparison at size one."""
@@ -120,7 +132,25 @@ def test_decaying_field_keeps_a_small_mean(n, dims):
     assert (mean(out) - c).abs().item() <= ulp
 
 
-@pytest.mark.parametrize("n,prec", [(64, F32), (128, F32), (256, F32)])
+@pytest.mark.parametrize("n", [32, 64])
+def test_adjoint_of_a_growing_mode_f64(n):
+    """lambda grows by e^19 through states of zero: the Fourier solve's, to the
+    rounding of 2000 steps."""
+    steps = 2000
+    fp = params(n, F64, 8e-4, dt=1e-2)
+    states = torch.zeros((steps, 1, n, n), dtype=torch.float64, device="cuda")
+    lam = torch.tensor(I.random_field(n, seed=4)[None], device="cuda")
+    got = G.ac_fine_adjoint(fp, steps, states, lam)
+    G.ac_fine_set_variant(n, F64, 1)
+    try:
+        ref = G.ac_fine_adjoint(fp, steps, states, lam)
+    finally:
+        G.ac_fine_set_variant(n, F64, 0)
+    assert ref.abs().max().item() > 2.0 ** 21
+    assert (got - ref).abs().max().item() < steps * 2.0 ** -50 * ref.abs().max().item()
+
+
+@pytest.mark.parametrize("n,prec", [(64, F32), (128, F32), (256, F32), (64, F64)])
 def test_batch_size_does_not_change_the_bits(n, prec):
     """Small growing fields, so that the unit of the sums changes on the way:
     every split of the field takes the same units."""
