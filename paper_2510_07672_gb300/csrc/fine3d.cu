@@ -218,6 +218,7 @@ int propagate3d(const ac_params* p, int steps, int fields, const T* u_in, T* u_o
     double* part = reinterpret_cast<double*>(work + part_off);
     const double h = p->length / N;
     if constexpr (sizeof(T) == 4) {
+        static_assert(kSumWords <= kMeanChunks, "the sums of the mass model fit in the mean's partials");
         const SolvePoly poly = solve_poly(1.0 + p->S * p->dt, 4.0 * p->dt * p->eps * p->eps / (h * h), 3, AC_F32, 2, 2);
         // (the streaming kernel reads vectors)
         const bool aligned = (reinterpret_cast<uintptr_t>(u_in) | reinterpret_cast<uintptr_t>(u_out) |

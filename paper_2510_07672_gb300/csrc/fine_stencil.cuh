@@ -228,7 +228,6 @@ __device__ __forceinline__ void apply_poly(LaneV<W> (&r)[H][Lane<W>::E], const C
 // is left of 62 bits (2^14 or more) is room for growth until the next measurement.
 constexpr int kMeasure = 8;
 constexpr int kCellRoom = 40, kGroupRoom = 30;  // one cell of the entry sum; a group of cells of r
-constexpr float kFix = 16777216.f;  // unit of the sums of fine_tiles.cu
 constexpr long long kBadSum = (long long)(1ULL << 63);
 constexpr unsigned kAbsMask = 0x7fffffffu;
 

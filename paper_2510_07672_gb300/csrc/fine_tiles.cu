@@ -14,15 +14,29 @@ namespace acpr {
 namespace {
 
 // Mass-conserving model: the shift of step n needs the sum of r^n over the
-// whole field.  It is accumulated (fixed point, integer atomics: any order
-// gives the same bits) by the launch that makes u^n.  Words per field:
-// entry sum of u, three rotating sums of r, a mark for cells out of range.
+// whole field.  From n = 1 it is accumulated (fixed point, integer atomics: any
+// order gives the same bits) by launch n - 1, which makes u^n, in a unit that
+// follows the largest cell of the last r measured before it: r^0 at entry, then
+// every kMeasure-th launch.  The sums of u^0 and r^0 are float64 partial sums
+// of kSumParts blocks.  Words per field: sum of r that keeps the entry mean
+// (float64), three rotating sums of r, a mark for cells out of range, two
+// rotating largest cells of r (their bits without the sign), the partial sums.
+constexpr int kSumParts = 24;
+static_assert(7 + 2 * kSumParts <= kSumWords, "words of a field");
 struct Sums {
-    long long* w;  // [5][fields]
+    long long* w;  // [kSumWords][fields]
     int fields;
-    __device__ __forceinline__ long long* entry(int f) const { return w + f; }
+    __device__ __forceinline__ double* goal(int f) const { return reinterpret_cast<double*>(w + f); }
     __device__ __forceinline__ long long* slot(int n, int f) const { return w + (long long)(1 + n % 3) * fields + f; }
     __device__ __forceinline__ long long* bad(int f) const { return w + 4LL * fields + f; }
+    // largest cell of r as launch l knows it
+    __device__ __forceinline__ unsigned* top(int l, int f) const {
+        return reinterpret_cast<unsigned*>(w + (long long)(5 + (l / kMeasure & 1)) * fields + f);
+    }
+    // partial sums of u (which = 0) and r^0 (1)
+    __device__ __forceinline__ double* part(int which, int i, int f) const {
+        return reinterpret_cast<double*>(w + (long long)(7 + which * kSumParts + i) * fields + f);
+    }
 };
 
 __device__ __forceinline__ void add_s64(long long* p, long long v) {
@@ -38,36 +52,90 @@ __device__ __forceinline__ void flush_sum(const Sums& s, long long* dst, int f, 
         else add_s64(dst, acc);
     }
 }
-
-// Shift that puts the mean of the new field at the entry mean (one thread of a
-// block computes it: float64 instructions are scarce).
-__device__ __forceinline__ float step_shift(const Sums& s, int n, int f, double a, double inv_sum) {
-    if (*s.bad(f)) return __int_as_float(0x7fffffff);
-    const long long target = __double2ll_rn(a * double(*s.entry(f)));
-    return float(target - *s.slot(n, f)) * (float(inv_sum) * (1.f / kFix));
+// The same of the largest magnitude (not that of a NaN, which the sums find).
+__device__ __forceinline__ void flush_max(unsigned* dst, float m, int lane) {
+    const unsigned bits = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if (lane == 0) atomicMax(dst, bits);
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-// Entry sums of u and of r^0, kSumParts blocks a field; cells a multiple of 4.
-constexpr int kSumParts = 32;
+// What launch l of the mass model works with, by one warp of a block (float64
+// instructions are scarce).  One block of the field (`first`) also keeps the
+// goal and clears the words that the next launches add to.
+struct LaunchSums {
+    float shift;  // puts the mean of u^(l+1) at the entry mean
+    float unit;   // of the sum of r^(l+1)
+};
+__device__ __forceinline__ void launch_sums(LaunchSums* out, const Sums& s, int l, int f, const Coef<float, 2>& cf, double a,
+                                            int room, int lane, bool first) {
+    double gap;  // the sum that r should have, less the one it has
+    if (l == 0) {
+        const double u = warp_sum(lane < kSumParts ? *s.part(0, lane, f) : 0.0);
+        const double r = warp_sum(lane < kSumParts ? *s.part(1, lane, f) : 0.0);
+        gap = a * u - r;
+        if (first && lane == 0) *s.goal(f) = a * u;
+    } else {
+        gap = *s.goal(f) - double(*s.slot(l, f)) * double(pow2_inv(pow2f(fix_scale(*s.top(l - 1, f), room))));
+    }
+    if (lane) return;
+    out->shift = *s.bad(f) ? __int_as_float(0x7fffffff) : float(gap * cf.inv_sum);
+    out->unit = pow2f(fix_scale(*s.top(l, f), room));
+    if (first) {
+        *s.slot(l + 2, f) = 0;
+        if (l % kMeasure == kMeasure / 2) *s.top(l + kMeasure, f) = 0;
+    }
+}
+__device__ __forceinline__ bool measures(int l) { return l % kMeasure == kMeasure - 1; }
+
+// s + e <- s + e + v, the rounding of s + v kept in e (TwoSum, Knuth).
+__device__ __forceinline__ void two_sum(f32x2& s, f32x2& e, f32x2 v) {
+    const f32x2 neg = f2(-1.f, -1.f);
+    const f32x2 t = f2_add(s, v), b = f2_fma(s, neg, t);
+    e = f2_add(e, f2_add(f2_fma(f2_fma(b, neg, t), neg, s), f2_fma(b, neg, v)));
+    s = t;
+}
+
+// Partial sums of u and of r^0, exact to 2^-48 of each thread's, and the
+// largest cell of r^0; kSumParts blocks a field; cells a multiple of 4.
 __global__ void __launch_bounds__(256) entry_sums_kernel(FieldMap src, long long cells, Sums s, float mdt, float kappa) {
-    const int f = blockIdx.x / kSumParts;
+    const int f = blockIdx.x / kSumParts, part = blockIdx.x % kSumParts;
     const float4* u = reinterpret_cast<const float4*>(src.at(f, cells));
-    long long su = 0, sr = 0;
-    bool bad = false;
-    for (long long i = (blockIdx.x % kSumParts) * 256LL + threadIdx.x; i < cells / 4; i += kSumParts * 256LL) {
+    const f32x2 m2 = f2(mdt, mdt), k2 = f2(kappa, kappa);
+    f32x2 su = f2(0.f, 0.f), eu = su, sr = su, er = su;
+    float top = 0.f;
+    for (long long i = part * 256LL + threadIdx.x; i < cells / 4; i += kSumParts * 256LL) {
         const float4 q = u[i];
-        const float v[4] = {q.x, q.y, q.z, q.w};
+        const f32x2 v[2] = {f2(q.x, q.y), f2(q.z, q.w)};
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float r = rhs(v[c], mdt, kappa);
-            su += __float2ll_rn(v[c] * kFix);
-            sr += __float2ll_rn(r * kFix);
-            bad |= !(fabsf(v[c]) < 0x1p16f) | !(fabsf(r) < 0x1p16f);
+        for (int c = 0; c < 2; ++c) {
+            const f32x2 r = rhs(v[c], m2, k2);
+            two_sum(su, eu, v[c]);
+            two_sum(sr, er, r);
+            top = fmaxf(top, fmaxf(fabsf(lo_of(r)), fabsf(hi_of(r))));
         }
     }
-    const int lane = threadIdx.x & 31;
-    flush_sum(s, s.entry(f), f, su, bad, lane);
-    flush_sum(s, s.slot(0, f), f, sr, bad, lane);
+    auto total = [](f32x2 a, f32x2 b) {
+        return warp_sum((double(lo_of(a)) + double(lo_of(b))) + (double(hi_of(a)) + double(hi_of(b))));
+    };
+    const double tu = total(su, eu), tr = total(sr, er);
+    __shared__ double red[2][8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    flush_max(s.top(0, f), top, lane);
+    if (lane == 0) {
+        red[0][warp] = tu;
+        red[1][warp] = tr;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) t += red[threadIdx.x][w];
+        *s.part(threadIdx.x, part, f) = t;
+    }
 }
 
 // ------------------------------------------------------------ 1024 x 1024 --
@@ -82,6 +150,7 @@ __global__ void __launch_bounds__(256) entry_sums_kernel(FieldMap src, long long
 constexpr int kTW = 8, kTH = 9, kTWarps = 16, kRim = 8, kTSteps = 4;
 constexpr int kTCols = 32 * kTW, kTRows = kTWarps * kTH;
 constexpr int kBig = 1024;
+constexpr int kTRoom = kGroupRoom - log2i(kTW);  // of a cell of r, in groups of a lane's row
 constexpr int kTValidC = 208, kTValidR = kTRows - 2 * kRim;
 constexpr int kTilesX = (kBig + kTValidC - 1) / kTValidC, kTilesY = kBig / kTValidR;
 constexpr size_t kTileSmem = size_t(2) * 2 * kTWarps * 2 * kTCols * sizeof(float);
@@ -117,11 +186,8 @@ __global__ void __launch_bounds__(kTWarps * 32, 1) big_tile_kernel(FieldMap src,
     const float* above = halo + warp * M * kTCols;
     const float* below = halo + (kTWarps + warp) * M * kTCols;
     const V mdt = vset<V>(cf.mdt), kappa = vset<V>(cf.kappa);
-    __shared__ float shift_sh;
-    if (MASS && threadIdx.x == 0) {
-        shift_sh = step_shift(sums, n_step, f, a, cf.inv_sum);
-        if (tile == 0) *sums.slot(n_step + 2, f) = 0;
-    }
+    __shared__ LaunchSums now;
+    if (MASS && warp == 0) launch_sums(&now, sums, n_step, f, cf, a, kTRoom, lane, tile == 0);
     for (int s = 0; s < steps; ++s) {
         const int buf = s & 1;
         if (!MASS || n_step == 0) {  // the mass model's launches hand on r
@@ -141,13 +207,14 @@ __global__ void __launch_bounds__(kTWarps * 32, 1) big_tile_kernel(FieldMap src,
             [&](int y, V(&x)[E]) {
                 row_load<kTW>((y < 0 ? above + (y + M) * kTCols : below + (y - kTH) * kTCols) + buf * BUF, x, lane);
             },
-            [&] { return shift_sh; });  // written before the step's barrier
+            [&] { return now.shift; });  // written before the step's barrier
     }
     float* out = dst.at(f, NN) + col0;
     // whole lanes are rim or stored
     const bool keep = lane * kTW >= kRim && lane * kTW < kRim + kTValidC && col0 < kBig;
     long long acc = 0;
     bool bad = false;
+    float top = 0.f;
 #pragma unroll
     for (int y = 0; y < kTH; ++y) {
         const int lr = warp * kTH + y;
@@ -162,14 +229,21 @@ __global__ void __launch_bounds__(kTWarps * 32, 1) big_tile_kernel(FieldMap src,
         p[0] = make_float4(c[0], c[1], c[2], c[3]);
         p[1] = make_float4(c[4], c[5], c[6], c[7]);
         if constexpr (MASS) {
-            float t = 0.f;
+            // a balanced tree: equal cells, a flat phase, add up exactly
+            const V t2 = vadd(vadd(u[y][0], u[y][1]), vadd(u[y][2], u[y][3]));
+            const float t = (lo_of(t2) + hi_of(t2)) * now.unit;
+            acc += __float2ll_rn(t);
+            bad |= !(fabsf(t) < 0x1p45f);  // 2^17 such sums stay below 2^62
+            if (measures(n_step)) {
 #pragma unroll
-            for (int e = 0; e < kTW; ++e) t += c[e];
-            acc += __float2ll_rn(t * kFix);
-            bad |= !(fabsf(t) < 0x1p18f);
+                for (int e = 0; e < kTW; ++e) top = fmaxf(top, fabsf(c[e]));
+            }
         }
     }
-    if (MASS && !last) flush_sum(sums, sums.slot(n_step + 1, f), f, acc, bad, lane);
+    if (MASS && !last) {
+        flush_sum(sums, sums.slot(n_step + 1, f), f, acc, bad, lane);
+        if (measures(n_step)) flush_max(sums.top(n_step + 1, f), top, lane);
+    }
 }
 
 // ------------------------------------------------------------------- cube --
@@ -183,6 +257,7 @@ __global__ void __launch_bounds__(kTWarps * 32, 1) big_tile_kernel(FieldMap src,
 // 16 fields of 128^3  Fourier passes 372, streamed 89 / 75 (2 rows a warp 107 / 65, 4 rows 121 / 102; handing on r
 // instead of u 103 / 93); 48 fields of 64^3 47 / 33.
 constexpr int kCRows = 36, kCValid = kCRows - 4;
+constexpr int kCRoom = kGroupRoom - 5;  // of a cell of r, in groups of up to 32
 template <int N>
 struct CubeShape {  // rows a warp, warps, CTAs per SM
     static constexpr int H = N == 128 ? 3 : 4, WARPS = kCRows / H, MINB = N == 128 ? 1 : 2;
@@ -202,12 +277,9 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
     const int i0 = chunk * planes, j0 = strip * kCValid - 2 + warp * kCH;
     const float* in = u + f * NNN;
     float* out = uo + f * NNN;
-    __shared__ float shift_sh;
+    __shared__ LaunchSums now;
     if constexpr (MASS) {
-        if (threadIdx.x == 0) {
-            shift_sh = step_shift(sums, n_step, f, a, cf.inv_sum);
-            if (strip == 0 && chunk == 0) *sums.slot(n_step + 2, f) = 0;
-        }
+        if (warp == 0) launch_sums(&now, sums, n_step, f, cf, a, kCRoom, lane, strip == 0 && chunk == 0);
         __syncthreads();
     }
     const int up = warp > 0 ? warp - 1 : kCWarps - 1, down = warp < kCWarps - 1 ? warp + 1 : 0;
@@ -229,7 +301,7 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
             to_lane<W>(c, x[y]);
         }
     };
-    const V be0 = vset<V>(cf.be0), b1 = vset<V>(cf.b1), g = vset<V>(cf.g[0]), sh = vset<V>(MASS ? shift_sh : 0.f);
+    const V be0 = vset<V>(cf.be0), b1 = vset<V>(cf.b1), g = vset<V>(cf.g[0]), sh = vset<V>(MASS ? now.shift : 0.f);
     const V mdt = vset<V>(cf.mdt), kappa = vset<V>(cf.kappa);
     // rp, rq: r(i - 1), r(i - 2); s0: the five known neighbours of r(i - 1);
     // wp: w(i - 2); s1: the five known neighbours of w(i - 2)
@@ -242,8 +314,20 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
     load_plane(i0 - 1, odd);
     long long acc = 0;
     bool bad = false;
-    // sums of u' and u'^3 over four planes (float32), then sum r = (1 + kappa) sum u' - dt sum u'^3 in fixed point
-    V part = vset<V>(0.f), cubes = vset<V>(0.f);
+    float top = 0.f;
+    // the next step's r over four planes, rows in balanced trees (equal cells, a
+    // flat phase, add up exactly; one after another they all round alike, which
+    // moved the mean by up to 4e-7 a call)
+    constexpr int G = kCH == 3 ? 2 : 1;
+    V part[2][G];
+    auto add_group = [&](V p) {
+        float t;
+        if constexpr (Lane<W>::PAIR) t = lo_of(p) + hi_of(p);
+        else t = p;
+        t *= now.unit;
+        acc += __float2ll_rn(t);
+        bad |= !(fabsf(t) < 0x1p44f);  // 2^17 such sums stay below 2^61
+    };
     const bool last = n_step == last_step;
     // plane k from `nxt`, which then receives plane k + 2 (two sets in turn:
     // 47 / 33 us against 50 / 37 with a copy, 48 x 64^3)
@@ -259,6 +343,9 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
         if (k < planes) load_plane(i0 + k + 2, nxt);
         if (k >= 2) {
             float* p = out + (long long)(i0 + k - 2) * NN + lane * W;
+            V rows[kCH];
+#pragma unroll
+            for (int y = 0; y < kCH; ++y) rows[y] = vset<V>(0.f);
 #pragma unroll
             for (int y = 0; y < kCH; ++y) {
                 V o[E];
@@ -276,21 +363,27 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
                 else if constexpr (W == 2) *reinterpret_cast<float2*>(q) = make_float2(v[0], v[1]);
                 else *q = v[0];
                 if constexpr (MASS) {
+                    V rn[E];
 #pragma unroll
-                    for (int c = 0; c < E; ++c) {
-                        part = vadd(part, o[c]);
-                        cubes = vfma(vmul(o[c], o[c]), o[c], cubes);
+                    for (int c = 0; c < E; ++c) rn[c] = rhs(o[c], mdt, kappa);
+                    rows[y] = E == 2 ? vadd(rn[0], rn[E - 1]) : rn[0];
+                    if (measures(n_step)) {
+                        float m[W];
+                        from_lane<W>(rn, m);
+#pragma unroll
+                        for (int c = 0; c < W; ++c) top = fmaxf(top, fabsf(m[c]));
                     }
                 }
             }
-            if (MASS && (k & 3) == 1) {
-                part = vfma(mdt, cubes, vfma(kappa, part, part));
-                float t;
-                if constexpr (Lane<W>::PAIR) t = lo_of(part) + hi_of(part);
-                else t = part;
-                acc += __float2ll_rn(t * kFix);
-                bad |= !(fabsf(t) < 0x1p20f);
-                part = cubes = vset<V>(0.f);
+            if constexpr (MASS) {
+                V g[2] = {vadd(rows[0], rows[1]), rows[2]};
+                if constexpr (kCH == 4) g[0] = vadd(g[0], vadd(rows[2], rows[kCH - 1]));
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    if ((k & 2) != 0) part[0][i] = buf ? vadd(part[0][i], g[i]) : g[i];  // (the first planes are k = 2, 3)
+                    else if (buf == 0) part[1][i] = g[i];
+                    else add_group(vadd(part[0][i], vadd(part[1][i], g[i])));
+                }
             }
         }
         row_store<W>(edge[buf][0][0][warp], r[0], lane);
@@ -327,7 +420,10 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
         plane(k, 0, even);
         plane(k + 1, 1, odd);
     }
-    if (MASS && !last) flush_sum(sums, sums.slot(n_step + 1, f), f, acc, bad, lane);
+    if (MASS && !last) {
+        flush_sum(sums, sums.slot(n_step + 1, f), f, acc, bad, lane);
+        if (measures(n_step)) flush_max(sums.top(n_step + 1, f), top, lane);
+    }
 }
 
 int sm_count() {
@@ -347,7 +443,7 @@ int cube_steps(const SolvePoly& poly, double a, double dt, int mass, int steps, 
     constexpr long long NNN = (long long)N * N * N;
     const Coef<float, 2> cf = make_coef<float, 2>(a, dt, double(NNN), poly);
     if (mass) {
-        ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * 5 * fields, st));
+        ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * kSumWords * fields, st));
         FieldMap src{};
         src.base = const_cast<float*>(u_in);
         src.per_group = fields;
@@ -398,7 +494,7 @@ int big_tiles_run(const SolvePoly& poly, double a, double dt, int mass, int fiel
     }
     Sums sums{sum_words, fields};
     if (mass) {
-        ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * 5 * fields, st));
+        ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * kSumWords * fields, st));
         entry_sums_kernel<<<unsigned(fields) * kSumParts, 256, 0, st>>>(src, NN, sums, cf.mdt, cf.kappa);
         ACPR_LAUNCH_CHECK();
     }

@@ -20,8 +20,10 @@ struct FieldMap {
     }
 };
 
+constexpr int kSumWords = 56;
+
 // `steps` >= 1 steps of `fields` 1024 x 1024 fields by a degree-2 polynomial.
-// tmp: as many contiguous fields; sum_words: 5 words per field (mass model).
+// tmp: as many contiguous fields; sum_words: kSumWords words per field (mass model).
 int big_tiles_run(const SolvePoly& poly, double a, double dt, int mass, int fields, int steps, FieldMap src, FieldMap dst,
                   float* tmp, long long* sum_words, cudaStream_t st);
 

@@ -51,7 +51,7 @@ def field_ref(u, fp, steps):
     return v
 
 
-GRIDS32 = [(32, 2), (64, 2), (128, 2), (256, 2), (512, 2)]
+GRIDS32 = [(32, 2), (64, 2), (128, 2), (256, 2), (512, 2), (1024, 2), (32, 3), (64, 3), (128, 3)]
 VALUES = [0.1, 0.9713, -0.9421, 0.9067, 0.9951, 1.1e-3, 1.7e-8, 3e-20]
 
 
