@@ -58,7 +58,9 @@ SolvePoly solve_poly(double a, double lam_scale, int dims, int precision, int mi
     const double tol = precision == AC_F64 ? 0x1p-52 : 0x1p-24;
     int M = std::max(1, min_degree);
     while (M <= max_degree && 4.0 * std::pow(rho, M + 1) > tol) ++M;
-    if (M > max_degree || M > kMaxDegree || !(a > 0.0) || !std::isfinite(rho)) return out;
+    // b_0 = 1 / a is applied as r + (b_0 - 1) r, whose rounding grows to a times
+    // b_0's own: beyond a = 2 the Fourier solve is the more exact one
+    if (M > max_degree || M > kMaxDegree || !(a > 0.0 && a <= 2.0) || !std::isfinite(rho)) return out;
     double c[kMaxDegree + 1];
     double sum = 0.0;
     for (int k = 0; k <= M; ++k) {
