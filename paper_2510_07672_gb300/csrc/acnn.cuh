@@ -44,7 +44,7 @@ __device__ __forceinline__ double acnn_sum_parts(const double* __restrict__ p, i
     return t;
 }
 
-// x + shift rounded once.  float32: shift = hi + lo and the exact error of
+// x + shift rounded once (infinities as IEEE adds them).  float32: shift = hi + lo and the exact error of
 // x + hi (TwoSum, Knuth) in place of float64 instructions, scarce on this GPU.
 template <typename T>
 struct AcnnShift {
@@ -59,7 +59,8 @@ struct AcnnShift<float> {
     __device__ float add(float x) const {
         const float s = __fadd_rn(x, hi), bb = __fsub_rn(s, x);
         const float e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, bb)), __fsub_rn(hi, bb));
-        return __fadd_rn(s, __fadd_rn(e, lo));
+        // the error of an infinite sum is not a number
+        return fabsf(s) < __int_as_float(0x7f800000) ? __fadd_rn(s, __fadd_rn(e, lo)) : s;
     }
 };
 
