@@ -14,7 +14,6 @@
 
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <vector>
 
 struct acnn_net {
@@ -423,13 +422,9 @@ template <typename T, int R>
 int launch_fused_r(const acnn_net* net, int n, int batch, const T* u, T* out, AcnnIO io, double* part,
                    cudaStream_t st) {
     using Sh = FusedShape<T, R>;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(acnn_fused_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        int(Sh::smem));
-    });
-    ACPR_CUDA(attr_err);
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [] { return allow_smem(acnn_fused_kernel<T, R>, Sh::smem); });
+    if (rc) return rc;
     FusedParams<T, R> P;
     std::memcpy(&P, net->host.data(), sizeof(P));
     const int tiles = (n / kTile) * (n / kTile);

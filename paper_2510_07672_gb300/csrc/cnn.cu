@@ -97,9 +97,7 @@ template <int G>
 static int launch_conv_f64(const double* in, double* out, const double* W, const double* bias, int batch, int n, int cin,
                            int cout, int act, int apply_act, const double* resid, const BatchIO& io, cudaStream_t st) {
     const long long pixels = (long long)n * n * batch;
-    const size_t smem = sizeof(double) * G * cin * 9;
-    if (smem > 48 * 1024)
-        ACPR_CUDA(cudaFuncSetAttribute(conv_f64_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    const size_t smem = sizeof(double) * G * cin * 9;  // at most 18 KB (64 channels)
     const dim3 grid(unsigned((pixels + kF64Threads - 1) / kF64Threads), unsigned((cout + G - 1) / G));
     conv_f64_kernel<G><<<grid, kF64Threads, smem, st>>>(in, out, W, bias, batch, n, cin, cout, act, apply_act, resid, io);
     ACPR_LAUNCH_CHECK();
@@ -448,12 +446,9 @@ static int last_layer_f32(const cnn_desc* d, int n, int batch, const __nv_bfloat
     const long long pixels = (long long)n * n * batch;
     const unsigned blocks = unsigned(pixels / ppb);
     const size_t smem = last_smem<C>(n);
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(conv_last_bf16_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(last_smem<C>(256))));
-        configured = true;
-    }
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [] { return allow_smem(conv_last_bf16_kernel<C>, last_smem<C>(256)); });
+    if (rc) return rc;
     conv_last_bf16_kernel<C><<<blocks, kLastThreads, smem, st>>>(a, out, W, Bv, u, batch, n, d->residual, io,
                                                                  d->mass_fix ? zpart : nullptr);
     ACPR_LAUNCH_CHECK();

@@ -753,29 +753,16 @@ int conv_get_variant(int n, int C) {
     return g_conv_pick[cidx(C)][lg2(n)];
 }
 
-static int num_sms() {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-            sms = 1;
-    }
-    return sms;
-}
-
 template <int C, int ACT, int MODE>
 static int launch_rows_mode(const RShape& s, int n, int batch, const __nv_bfloat16* in, __nv_bfloat16* out,
                             const __nv_bfloat16* w, const float* bias, float* zio, int* status, cudaStream_t st,
                             const float* wlast, float* maps) {
     auto kern = conv_rows_tc<C, ACT, MODE>;
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(227 * 1024)));
-        configured = true;
-    }
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [&] { return allow_smem(kern, 227 * 1024); });
+    if (rc) return rc;
     const long long units = (long long)batch * (n / 128) * n;
-    const int grid = int(units < num_sms() ? units : num_sms());
+    const int grid = int(std::min<long long>(units, sm_count()));
     kern<<<grid, RGeom<C>::THREADS, s.smem, st>>>(in, out, w, bias, n, batch, s.RING, s.DS, zio, status,
                                                   g_test_stall, wlast, maps);
     ACPR_LAUNCH_CHECK();
@@ -816,11 +803,9 @@ static int launch_hidden(int n, int batch, const __nv_bfloat16* in, __nv_bfloat1
     const TcShape s = pick_shape(n, C);
     if (s.TY == 0) return AC_ERR_UNSUPPORTED;
     auto kern = act == AC_ACT_TANH ? conv_hidden_tc_kernel<C, AC_ACT_TANH> : conv_hidden_tc_kernel<C, AC_ACT_GELU>;
-    static bool configured[2] = {false, false};
-    if (!configured[act == AC_ACT_TANH]) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(227 * 1024)));
-        configured[act == AC_ACT_TANH] = true;
-    }
+    static DeviceSet configured[2];
+    const int rc = once_per_device(configured[act == AC_ACT_TANH], [&] { return allow_smem(kern, 227 * 1024); });
+    if (rc) return rc;
     const long long blocks = (long long)batch * (n / s.TY);
     kern<<<unsigned(blocks), kTcThreads, s.smem, st>>>(in, out, w, bias, n, s.TY, s.n_mt, s.plane_px, s.ncols, mode,
                                                        zio, status);

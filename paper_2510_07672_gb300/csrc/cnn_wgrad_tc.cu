@@ -302,11 +302,9 @@ int wgrad_tc_partials(int n, int batch, const __nv_bfloat16* a, const __nv_bfloa
         set_error("tensor-core weight gradient: no status word");
         return AC_ERR_ARG;
     }
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kWSmem)));
-        configured = true;
-    }
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [] { return allow_smem(wgrad_tc_kernel, kWSmem); });
+    if (rc) return rc;
     wgrad_tc_kernel<<<chunks, kWThreads, kWSmem, st>>>(a, dz, part, n, batch, chunks, status);
     ACPR_LAUNCH_CHECK();
     return AC_OK;

@@ -8,6 +8,7 @@
 #include <string>
 
 #include "../../include/acpr.h"
+#include "per_device.h"
 
 namespace acpr {
 
@@ -53,6 +54,28 @@ template <typename T> struct Vec2;
 template <> struct Vec2<float> { using type = float2; };
 template <> struct Vec2<double> { using type = double2; };
 template <typename T> using vec2_t = typename Vec2<T>::type;
+
+// Runs set() (AC_OK or an error code) the first time on each device.
+template <class F>
+int once_per_device(DeviceSet& done, F set) {
+    int dev = 0;
+    ACPR_CUDA(cudaGetDevice(&dev));
+    if (done.has(dev)) return AC_OK;
+    const int rc = set();
+    if (rc == AC_OK) done.add(dev);
+    return rc;
+}
+
+// Shared memory (and, for clusters of more than 8 CTAs, their size) a kernel may use.
+template <class K>
+int allow_smem(K kern, size_t bytes, int cluster = 1) {
+    ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+    if (cluster > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    return AC_OK;
+}
+
+// Multiprocessors of the current device (at least 1).
+int sm_count();
 
 inline bool is_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 inline size_t elem_size(int precision) { return precision == AC_F64 ? 8 : 4; }

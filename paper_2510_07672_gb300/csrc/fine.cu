@@ -498,13 +498,9 @@ template <typename T, int N, int P, int A, int B, int MINB, bool ASYNC = false, 
 static int launch_fine(const FineArgs& args, cudaStream_t stream) {
     using Sh = FineShape<T, N, P, A, B, NOX>;
     auto kern = fine_field_kernel<T, N, P, A, B, MINB, ASYNC, NOX>;
-    static bool configured = false;  // per instantiation, once per process
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM)));
-        if (P > 8)
-            ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        configured = true;
-    }
+    static DeviceSet configured;  // per instantiation
+    const int rc = once_per_device(configured, [&] { return allow_smem(kern, Sh::SMEM, P); });
+    if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(args.num_fields * P), 1, 1);
     cfg.blockDim = dim3(Sh::THREADS, 1, 1);

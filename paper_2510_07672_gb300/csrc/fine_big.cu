@@ -412,14 +412,12 @@ int fine_big_run(const ac_params* p, int groups, int per_group, int steps, const
     constexpr size_t kBufs = kIn > kXf ? (kIn > kOut ? kIn : kOut) : (kXf > kOut ? kXf : kOut);
     const size_t smem_rows = sizeof(vec2_t<T>) * (N + size_t(kBigWarps) * A * 33);
     const size_t smem_cols = sizeof(vec2_t<T>) * (N + kBufs) + sizeof(T) * N;
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(big_rows_kernel<T, N, A>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(smem_rows)));
-        ACPR_CUDA(cudaFuncSetAttribute(big_cols_kernel<T, N, A>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(smem_cols)));
-        configured = true;
-    }
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [&] {
+        const int r = allow_smem(big_rows_kernel<T, N, A>, smem_rows);
+        return r ? r : allow_smem(big_cols_kernel<T, N, A>, smem_cols);
+    });
+    if (rc) return rc;
     const unsigned blocks = unsigned(fields * (N / 2 / kBigWarps));
     if (steps == 0) {
         // one forward and one inverse row pass would round; copy instead

@@ -381,12 +381,9 @@ template <typename T, int N, int P, int A, int B>
 int launch_cn(const CnArgs& args, cudaStream_t st) {
     using Sh = CnShape<T, N, P, A, B>;
     auto kern = fine_cn_kernel<T, N, P, A, B>;
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(Sh::SMEM)));
-        if (P > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        configured = true;
-    }
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [&] { return allow_smem(kern, Sh::SMEM, P); });
+    if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned(args.num_fields * P), 1, 1);
     cfg.blockDim = dim3(Sh::THREADS, 1, 1);

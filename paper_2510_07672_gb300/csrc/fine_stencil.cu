@@ -389,13 +389,10 @@ __global__ void __launch_bounds__(NW * 32, 1) stencil_reg_pair_kernel(const __gr
 
 // Launches a kernel in clusters of P CTAs.
 template <typename K, typename... A>
-int launch_clusters(K kern, bool* configured, int P, unsigned fields, int threads, size_t smem, cudaStream_t stream,
+int launch_clusters(K kern, DeviceSet& configured, int P, unsigned fields, int threads, size_t smem, cudaStream_t stream,
                     const A&... a) {
-    if (!*configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        if (P > 8) ACPR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        *configured = true;
-    }
+    const int rc = once_per_device(configured, [&] { return allow_smem(kern, smem, P); });
+    if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(fields * unsigned(P), 1, 1);
     cfg.blockDim = dim3(unsigned(threads), 1, 1);
@@ -416,15 +413,15 @@ int launch_clusters(K kern, bool* configured, int P, unsigned fields, int thread
 template <int N, int H, int NW, int P, int M, int MINB, bool MASS, bool ADJ>
 int launch_reg_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
     using Sh = RegShape<N, H, NW, P, M>;
-    static bool configured = false;
-    return launch_clusters(stencil_reg_kernel<N, H, NW, P, M, MINB, MASS, ADJ>, &configured, P, unsigned(args.num_fields), NW * 32, Sh::SMEM, stream, args,
+    static DeviceSet configured;
+    return launch_clusters(stencil_reg_kernel<N, H, NW, P, M, MINB, MASS, ADJ>, configured, P, unsigned(args.num_fields), NW * 32, Sh::SMEM, stream, args,
                            make_coef<float, M>(args.a, args.dt, double(N) * N, poly));
 }
 
 template <int N, int H, int NW, int P, int M, bool MASS>
 int launch_reg_pair(const FineArgs& adj, const FineArgs& fwd, const SolvePoly& poly, cudaStream_t stream) {
-    static bool configured = false;
-    return launch_clusters(stencil_reg_pair_kernel<N, H, NW, P, M, MASS>, &configured, P,
+    static DeviceSet configured;
+    return launch_clusters(stencil_reg_pair_kernel<N, H, NW, P, M, MASS>, configured, P,
                            unsigned(adj.num_fields + fwd.num_fields), NW * 32, RegShape<N, H, NW, P, M>::SMEM, stream, adj,
                            fwd, make_coef<float, M>(adj.a, adj.dt, double(N) * N, poly));
 }
@@ -711,15 +708,15 @@ __global__ void __launch_bounds__(kShThreads) stencil_smem_pair_kernel(const __g
 template <typename T, int N, int P, int M, bool MASS, bool ADJ>
 int launch_smem_t(const FineArgs& args, const SolvePoly& poly, cudaStream_t stream) {
     using Sh = ShShape<T, N, P, M>;
-    static bool configured = false;
-    return launch_clusters(stencil_smem_kernel<T, N, P, M, MASS, ADJ>, &configured, P, unsigned(args.num_fields), kShThreads, Sh::SMEM, stream, args,
+    static DeviceSet configured;
+    return launch_clusters(stencil_smem_kernel<T, N, P, M, MASS, ADJ>, configured, P, unsigned(args.num_fields), kShThreads, Sh::SMEM, stream, args,
                            make_coef<T, M>(args.a, args.dt, double(N) * N, poly));
 }
 
 template <typename T, int N, int P, int M, bool MASS>
 int launch_smem_pair(const FineArgs& adj, const FineArgs& fwd, const SolvePoly& poly, cudaStream_t stream) {
-    static bool configured = false;
-    return launch_clusters(stencil_smem_pair_kernel<T, N, P, M, MASS>, &configured, P,
+    static DeviceSet configured;
+    return launch_clusters(stencil_smem_pair_kernel<T, N, P, M, MASS>, configured, P,
                            unsigned(adj.num_fields + fwd.num_fields), kShThreads, ShShape<T, N, P, M>::SMEM, stream, adj, fwd,
                            make_coef<T, M>(adj.a, adj.dt, double(N) * N, poly));
 }

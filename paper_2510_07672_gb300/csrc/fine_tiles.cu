@@ -426,17 +426,6 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
     }
 }
 
-int sm_count() {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-            sms = 1;
-    }
-    return sms;
-}
-
 template <int N>
 int cube_steps(const SolvePoly& poly, double a, double dt, int mass, int steps, int fields, const float* u_in,
                float* u_out, float* tmp, Sums sums, cudaStream_t st) {
@@ -486,12 +475,12 @@ int big_tiles_run(const SolvePoly& poly, double a, double dt, int mass, int fiel
                   float* tmp, long long* sum_words, cudaStream_t st) {
     constexpr long long NN = (long long)kBig * kBig;
     const Coef<float, 2> cf = make_coef<float, 2>(a, dt, double(NN), poly);
-    static bool configured = false;
-    if (!configured) {
-        ACPR_CUDA(cudaFuncSetAttribute(big_tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTileSmem)));
-        ACPR_CUDA(cudaFuncSetAttribute(big_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kTileSmem)));
-        configured = true;
-    }
+    static DeviceSet configured;
+    const int rc = once_per_device(configured, [] {
+        const int r = allow_smem(big_tile_kernel<true>, kTileSmem);
+        return r ? r : allow_smem(big_tile_kernel<false>, kTileSmem);
+    });
+    if (rc) return rc;
     Sums sums{sum_words, fields};
     if (mass) {
         ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * kSumWords * fields, st));
