@@ -439,9 +439,11 @@ int cube_steps(const SolvePoly& poly, double a, double dt, int mass, int steps, 
         entry_sums_kernel<<<unsigned(fields) * kSumParts, 256, 0, st>>>(src, NNN, sums, cf.mdt, cf.kappa);
         ACPR_LAUNCH_CHECK();
     }
-    // the last step writes u_out, the ones before alternate with tmp
+    // the last step writes u_out, the ones before alternate with tmp; a first
+    // step that writes u_out may not read cells there
     const float* cur = u_in;
-    if (u_in == u_out && steps % 2) {
+    const uintptr_t from = reinterpret_cast<uintptr_t>(u_in), to = reinterpret_cast<uintptr_t>(u_out);
+    if ((from > to ? from - to : to - from) < sizeof(float) * NNN * fields && steps % 2) {
         ACPR_CUDA(cudaMemcpyAsync(tmp, u_in, sizeof(float) * NNN * fields, cudaMemcpyDeviceToDevice, st));
         cur = tmp;
     }

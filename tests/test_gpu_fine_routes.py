@@ -36,3 +36,21 @@ def test_large_stabilisation_takes_the_fourier_solve(n, prec, variant):
     assert torch.equal(run(fp, 0), run(fp, 1))
     fp = params(n, prec, variant, 1e-3, dt=0.5)
     assert not torch.equal(run(fp, 0), run(fp, 1))
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("steps", [1, 2, 3])
+@pytest.mark.parametrize("lam", [2.5e-3, 2e-2])
+def test_cube_buffers_that_overlap(steps, variant, lam):
+    """u_in and u_out share two of three fields, either one first: the same bits
+    as apart (streamed planes, and the passes that stiff steps take)."""
+    n, size = 32, 32 ** 3
+    fp = params(n, F32, variant, lam)
+    u = random_fields((3, n, n, n), torch.float32)
+    want = G.ac_fine3d_propagate(fp, steps, u)
+    for first, second in ((0, size), (size, 0)):
+        buf = torch.empty(4 * size, device="cuda")
+        src, dst = buf[first:first + 3 * size].view_as(u), buf[second:second + 3 * size].view_as(u)
+        src.copy_(u)
+        G.ac_fine3d_propagate(fp, steps, src, dst)
+        assert torch.equal(dst, want)
