@@ -26,8 +26,8 @@
 // one word for float32, two for float64), which makes it independent of the
 // order and of the split.  The unit follows the largest cell, so the mean is as
 // exact for small, large, growing and decaying fields as for those of size one;
-// only a field that outgrows its unit (float32: 2^14-fold in 8 steps, float64:
-// 2^19-fold in one) becomes not a number.
+// only a field that outgrows its unit (float32: 2^18-fold in two runs of steps,
+// see Coef::run, float64: 2^19-fold in one step; a blow-up) becomes not a number.
 //
 // Bound: FP32 (float64: FP64) issue.  Measured, Fourier kernel -> this one:
 //   512 fields of 256^2, mass, 100 steps        11.40 -> 1.98 ms (2.21 with scalar instructions and 8x8x4)
@@ -166,7 +166,7 @@ template <int N, int H, int NW, int P, int M>
 struct RegShape {
     static constexpr int W = N / 32, R = NW * H;
     static constexpr size_t HALO = size_t(2) * 2 * NW * M * N;  // floats
-    static constexpr size_t SMEM = HALO * sizeof(float) + size_t(3) * P * NW * sizeof(long long);
+    static constexpr size_t SMEM = HALO * sizeof(float) + (size_t(4) * P * NW + NW) * sizeof(long long);
     static constexpr int ROOM = kGroupRoom - log2i(2 * W);  // of a cell of r, in groups of two rows of a lane
     static_assert(R * P == N && H % 2 == 0 && H >= M && N % 32 == 0, "split");
 };
@@ -180,7 +180,8 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* halo = reinterpret_cast<float*>(smem_raw);  // [buffer][0: above, 1: below][warp][M][N]
     long long* tot = reinterpret_cast<long long*>(halo + Sh::HALO);  // [buffer][P NW] sums of the warps
-    long long* aux = tot + 2 * P * NW;                               // [P NW] the warps' entry sums, later their maxima
+    constexpr int AUX = 2 * P * NW;                                  // from there [buffer][P NW] the warps' largest cells
+    double* goal = reinterpret_cast<double*>(tot + 2 * AUX);         // [NW] (the register it would take spills elsewhere)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int rank = 0;
     if constexpr (P > 1) rank = int(cg::this_cluster().block_rank());
@@ -209,13 +210,12 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
     const float* above = halo + warp * M * N;
     const float* below = halo + (NW + warp) * M * N;
 
-    // mass model: the sum of r that keeps the entry mean, and it in units of 1 / unit
-    double goal = 0.0;
-    long long target = 0, entry = 0;
-    float unit = 1.f, entry_unit = 1.f;
+    // mass model: the sum of r that keeps the entry mean (goal), in units of 1 / unit
+    long long target = 0;
+    float unit = 0.f, inv_unit = 0.f;
     double msum = 0.0;      // adjoint: this warp's part of the sum of lambda
-    auto publish = [&](long long* to, long long v) {
-        for (int q = lane; q < P; q += 32) peer<P>(to, q)[rank * NW + warp] = v;
+    auto publish = [&](int at, long long v) {
+        for (int q = lane; q < P; q += 32) peer<P>(tot, q)[at + rank * NW + warp] = v;
     };
     auto largest = [&](const long long* from) {
         unsigned m = 0;
@@ -225,26 +225,38 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
     // largest magnitude of the warp's cells, as bits (not that of a NaN, which
     // the sums below find)
     auto measure = [&] {
-        float m = 0.f;
+        float m[W] = {};
 #pragma unroll
         for (int y = 0; y < H; ++y) {
             float v[W];
             from_lane<W>(u[y], v);
 #pragma unroll
-            for (int c = 0; c < W; ++c) m = fmaxf(m, fabsf(v[c]));
+            for (int c = 0; c < W; ++c) m[c] = fmaxf(m[c], fabsf(v[c]));
         }
-        return __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+#pragma unroll
+        for (int o = W / 2; o > 0; o /= 2)
+#pragma unroll
+            for (int c = 0; c < o; ++c) m[c] = fmaxf(m[c], m[c + o]);
+        return __reduce_max_sync(0xffffffffu, __float_as_uint(m[0]));
+    };
+    // the sums of r while no cell of u is much larger than m
+    auto set_unit = [&](unsigned m) {
+        const float now = pow2f(fix_scale(__float_as_uint(rhs_bound(__uint_as_float(m), cf.mdt, cf.kappa)), Sh::ROOM));
+        if (now == unit) return;
+        unit = now;
+        inv_unit = float(cf.inv_sum) * pow2_inv(unit);
+        target = __double2ll_rn(goal[warp] * double(unit));
     };
     cl_arrive<P>();
+    cl_wait<P>();  // every CTA of the cluster runs
     if constexpr (MASS && !ADJ) {
         const unsigned mine = measure();
-        cl_wait<P>();
-        publish(tot + P * NW, mine);
+        publish(AUX, mine);
         cl_arrive<P>();
         cl_wait<P>();
-        const unsigned m = largest(tot + P * NW);
-        entry_unit = pow2f(fix_scale(m, kCellRoom));
-        unit = pow2f(fix_scale(__float_as_uint(rhs_bound(__uint_as_float(m), cf.mdt, cf.kappa)), Sh::ROOM));
+        const unsigned m = largest(tot + AUX);
+        const float entry_unit = pow2f(fix_scale(m, kCellRoom));
+        long long entry = 0;
         // entry sum, cell by cell
 #pragma unroll
         for (int y = 0; y < H; ++y) {
@@ -253,119 +265,124 @@ __device__ __forceinline__ void stencil_reg_body(const FineArgs& args, const Coe
 #pragma unroll
             for (int c = 0; c < W; ++c) entry += __float2ll_rn(v[c] * entry_unit);
         }
-        entry = warp_sum_s64(entry);
-    } else {
+        publish(P * NW, warp_sum_s64(entry));
+        cl_arrive<P>();
         cl_wait<P>();
+        entry = 0;
+        for (int i = lane; i < P * NW; i += 32) entry += tot[P * NW + i];
+        entry = warp_sum_s64(entry);
+        if (lane == 0) goal[warp] = args.a * double(entry) * double(pow2_inv(entry_unit));
+        __syncwarp();
+        set_unit(m);
     }
 
-    for (int step = 0; step < it.steps; ++step) {
-        const int buf = step & 1;
-        // the rows that others wait for first
-        auto rhs_row = [&](int y) {
-            if constexpr (!ADJ) {
+    // Runs of steps with one unit for the sums of r, from the largest cell at the
+    // start of the run before: handed round with that run's first sums, it needs
+    // no barrier, and nothing of it parts the instructions of a step (asked for
+    // within the steps, even by branches not taken, it made them 5 to 10% longer;
+    // between runs of 16 steps 1 to 5%).
+    const int run = MASS && !ADJ ? cf.run : it.steps;
+    for (int step = 0, odd = 0; step < it.steps; odd ^= 1) {
+        const int tops = AUX + odd * P * NW;
+        if constexpr (MASS && !ADJ) publish(tops, measure());
+        for (const int end = it.steps - step > run ? step + run : it.steps; step < end; ++step) {
+            const int buf = step & 1;
+            // the rows that others wait for first
+            auto rhs_row = [&](int y) {
+                if constexpr (!ADJ) {
 #pragma unroll
-                for (int c = 0; c < E; ++c) u[y][c] = rhs(u[y][c], vset<V>(cf.mdt), vset<V>(cf.kappa));
+                    for (int c = 0; c < E; ++c) u[y][c] = rhs(u[y][c], vset<V>(cf.mdt), vset<V>(cf.kappa));
+                }
+            };
+#pragma unroll
+            for (int y = 0; y < H; ++y)
+                if (y < M || y >= H - M) rhs_row(y);
+#pragma unroll
+            for (int m = 0; m < M; ++m) {
+                row_store<W>(up + buf * BUF + m * N, u[m], lane);
+                row_store<W>(down + buf * BUF + m * N, u[H - M + m], lane);
             }
-        };
+            if constexpr (!MASS) cl_arrive<P>();
 #pragma unroll
-        for (int y = 0; y < H; ++y)
-            if (y < M || y >= H - M) rhs_row(y);
+            for (int y = M; y < H - M; ++y) rhs_row(y);
+            if constexpr (MASS) {
+                if constexpr (!ADJ) {
+                    long long acc = 0;
+                    bool bad = false;
 #pragma unroll
-        for (int m = 0; m < M; ++m) {
-            row_store<W>(up + buf * BUF + m * N, u[m], lane);
-            row_store<W>(down + buf * BUF + m * N, u[H - M + m], lane);
-        }
-        if constexpr (!MASS) cl_arrive<P>();
+                    for (int y = 0; y < H; y += 2) {
+                        const float t = pair_sum<W>(u[y], u[y + 1]) * unit;
+                        acc += __float2ll_rn(t);
+                        bad |= !(fabsf(t) < 0x1p49f);  // 2^13 such sums stay below 2^62
+                    }
+                    acc = warp_sum_s64(acc);
+                    if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
+                    publish(buf * P * NW, acc);
+                } else {
+                    msum = 0.0;
 #pragma unroll
-        for (int y = M; y < H - M; ++y) rhs_row(y);
-        if constexpr (MASS) {
-            if constexpr (!ADJ) {
-                long long acc = 0;
-                bool bad = false;
+                    for (int y = 0; y < H; y += 2) msum += double(pair_sum<W>(u[y], u[y + 1]));
 #pragma unroll
-                for (int y = 0; y < H; y += 2) {
-                    const float t = pair_sum<W>(u[y], u[y + 1]) * unit;
-                    acc += __float2ll_rn(t);
-                    bad |= !(fabsf(t) < 0x1p49f);  // 2^13 such sums stay below 2^62
-                }
-                acc = warp_sum_s64(acc);
-                if (__any_sync(0xffffffffu, bad)) acc = kBadSum;
-                publish(tot + buf * P * NW, acc);
-                if (step == 0) publish(aux, entry);
-                else if ((step & (kMeasure - 1)) == 0) publish(aux, measure());
-            } else {
-                msum = 0.0;
-#pragma unroll
-                for (int y = 0; y < H; y += 2) msum += double(pair_sum<W>(u[y], u[y + 1]));
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
-                publish(tot + buf * P * NW, __double_as_longlong(msum));
-            }
-        }
-        if constexpr (MASS) cl_arrive<P>();
-        cl_wait<P>();
-        // the shift of the mass model, and the adjoint's mean of mu
-        float shift = 0.f;
-        auto collect = [&]() -> float {
-            const long long* tb = tot + buf * P * NW;
-            if constexpr (!ADJ) {
-                if (step == 0) {
-                    long long e = 0;
-                    for (int i = lane; i < P * NW; i += 32) e += aux[i];
-                    goal = args.a * double(warp_sum_s64(e)) * double(pow2_inv(entry_unit));
-                    target = __double2ll_rn(goal * double(unit));
-                }
-                long long t = 0;
-                bool bad = false;
-#pragma unroll
-                for (int i0 = 0; i0 < P * NW; i0 += 32) {
-                    const long long v = P * NW % 32 == 0 || i0 + lane < P * NW ? tb[i0 + lane] : 0;
-                    t += v;
-                    bad |= v == kBadSum;
-                }
-                t = warp_sum_s64(t);
-                shift = float(target - t) * float(cf.inv_sum) * pow2_inv(unit);
-                if (__any_sync(0xffffffffu, bad)) shift = __int_as_float(0x7fffffff);
-                if (step > 0 && (step & (kMeasure - 1)) == 0) {
-                    unit = pow2f(fix_scale(largest(aux), Sh::ROOM));
-                    target = __double2ll_rn(goal * double(unit));
-                }
-            } else {
-                double t = 0.0;
-                for (int i = lane; i < P * NW; i += 32) t += __longlong_as_double(tb[i]);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-                shift = float(t * cf.inv_sum);
-            }
-            return shift;
-        };
-        apply_poly<W, H, M, MASS && !ADJ>(
-            u, cf, lane,
-            [&](int y, V(&x)[E]) {
-                row_load<W>((y < 0 ? above + (y + M) * N : below + (y - H) * N) + buf * BUF, x, lane);
-            },
-            collect);
-        if constexpr (MASS && ADJ) collect();
-        if constexpr (ADJ) {
-            const float* un = static_cast<const float*>(args.states) +
-                              ((long long)(it.steps - 1 - step) * args.num_fields + field) * NN + (long long)row0 * N;
-#pragma unroll
-            for (int y = 0; y < H; ++y) {
-                V v[E];
-                grow_load<W>(un + y * N, v, lane);
-                const V one = vset<V>(1.f), m3 = vset<V>(-3.f), a = vset<V>(cf.a), dt = vset<V>(cf.dt), ms = vset<V>(-shift);
-#pragma unroll
-                for (int c = 0; c < E; ++c) {
-                    const V f = vmul(dt, vfma(m3, vmul(v[c], v[c]), one));
-                    u[y][c] = vfma(a, u[y][c], vmul(f, vadd(u[y][c], ms)));
+                    for (int o = 16; o > 0; o >>= 1) msum += __shfl_xor_sync(0xffffffffu, msum, o);
+                    publish(buf * P * NW, __double_as_longlong(msum));
                 }
             }
-        }
-        if (traj) {
-            float* ts = traj + (step + 1) * traj_step;
+            if constexpr (MASS) cl_arrive<P>();
+            cl_wait<P>();
+            // the shift of the mass model, and the adjoint's mean of mu
+            float shift = 0.f;
+            auto collect = [&]() -> float {
+                const long long* tb = tot + buf * P * NW;
+                if constexpr (!ADJ) {
+                    long long t = 0;
+                    bool bad = false;
 #pragma unroll
-            for (int y = 0; y < H; ++y) grow_store<W>(ts + y * N, u[y], lane);
+                    for (int i0 = 0; i0 < P * NW; i0 += 32) {
+                        const long long v = P * NW % 32 == 0 || i0 + lane < P * NW ? tb[i0 + lane] : 0;
+                        t += v;
+                        bad |= v == kBadSum;
+                    }
+                    t = warp_sum_s64(t);
+                    shift = float(target - t) * inv_unit;
+                    if (__any_sync(0xffffffffu, bad)) shift = __int_as_float(0x7fffffff);
+                } else {
+                    double t = 0.0;
+                    for (int i = lane; i < P * NW; i += 32) t += __longlong_as_double(tb[i]);
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                    shift = float(t * cf.inv_sum);
+                }
+                return shift;
+            };
+            apply_poly<W, H, M, MASS && !ADJ>(
+                u, cf, lane,
+                [&](int y, V(&x)[E]) {
+                    row_load<W>((y < 0 ? above + (y + M) * N : below + (y - H) * N) + buf * BUF, x, lane);
+                },
+                collect);
+            if constexpr (MASS && ADJ) collect();
+            if constexpr (ADJ) {
+                const float* un = static_cast<const float*>(args.states) +
+                                  ((long long)(it.steps - 1 - step) * args.num_fields + field) * NN + (long long)row0 * N;
+#pragma unroll
+                for (int y = 0; y < H; ++y) {
+                    V v[E];
+                    grow_load<W>(un + y * N, v, lane);
+                    const V one = vset<V>(1.f), m3 = vset<V>(-3.f), a = vset<V>(cf.a), dt = vset<V>(cf.dt), ms = vset<V>(-shift);
+#pragma unroll
+                    for (int c = 0; c < E; ++c) {
+                        const V f = vmul(dt, vfma(m3, vmul(v[c], v[c]), one));
+                        u[y][c] = vfma(a, u[y][c], vmul(f, vadd(u[y][c], ms)));
+                    }
+                }
+            }
+            if (traj) {
+                float* ts = traj + (step + 1) * traj_step;
+#pragma unroll
+                for (int y = 0; y < H; ++y) grow_store<W>(ts + y * N, u[y], lane);
+            }
         }
+        if constexpr (MASS && !ADJ) set_unit(largest(tot + tops));
     }
 #pragma unroll
     for (int y = 0; y < H; ++y) grow_store<W>(out + y * N, u[y], lane);

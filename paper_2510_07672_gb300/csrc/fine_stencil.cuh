@@ -17,6 +17,7 @@ struct Coef {
     T be0, b1;      // u' = r + be0 r + b1 T w_1
     T g[M];         // g[k], k = 0 .. M - 2: stage k, w = r + g[k] T (input)
     T a, dt;        // adjoint: lambda' = a mu + dt f'(u) (mu - mean)
+    int run;        // steps between two measurements of the largest cell (mass model)
     double inv_sum;  // 1 / (a cells): sum of r -> mean of p(Lap) r (no division on the device: float64 is scarce)
 };
 
@@ -34,6 +35,9 @@ Coef<T, M> make_coef(double a, double dt, double cells, const SolvePoly& p) {
     }
     c.a = T(a);
     c.dt = T(dt);
+    // A cell of size below one grows at most by (a + dt) / a a step, and a unit
+    // serves two runs: 2^18 of the 2^19 that it leaves.
+    c.run = int(std::fmin(64.0, std::fmax(4.0, 9.0 / std::log2((a + dt) / a))));
     c.inv_sum = 1.0 / (a * cells);
     return c;
 }
@@ -223,10 +227,9 @@ __device__ __forceinline__ void apply_poly(LaneV<W> (&r)[H][Lane<W>::E], const C
 
 // Sums of r in integers, exact up to the unit: any order and any split give the
 // same bits.  The unit follows the field: a power of two 2^-scale such that the
-// largest magnitude met, taken over the field at entry and every kMeasure steps,
-// is below 2^room units, so a group's rounding is 2^-30 of that magnitude.  What
-// is left of 62 bits (2^14 or more) is room for growth until the next measurement.
-constexpr int kMeasure = 8;
+// largest magnitude met, taken over the field at entry and every few steps, is
+// below 2^room units, so a group's rounding is 2^-30 of that magnitude.  What is
+// left of 62 bits is room for growth until the next measurement.
 constexpr int kCellRoom = 40, kGroupRoom = 30;  // one cell of the entry sum; a group of cells of r
 constexpr long long kBadSum = (long long)(1ULL << 63);
 constexpr unsigned kAbsMask = 0x7fffffffu;

@@ -22,6 +22,7 @@ namespace {
 // (float64), three rotating sums of r, a mark for cells out of range, two
 // rotating largest cells of r (their bits without the sign), the partial sums.
 constexpr int kSumParts = 24;
+constexpr int kMeasure = 8;  // (a unit leaves 2^14: 3.3-fold growth a step)
 static_assert(7 + 2 * kSumParts <= kSumWords, "words of a field");
 struct Sums {
     long long* w;  // [kSumWords][fields]
