@@ -21,8 +21,8 @@ namespace {
 // of kSumParts blocks.  Words per field: sum of r that keeps the entry mean
 // (float64), three rotating sums of r, a mark for cells out of range, two
 // rotating largest cells of r (their bits without the sign), the partial sums.
-constexpr int kSumParts = 24;
-constexpr int kMeasure = 8;  // (a unit leaves 2^14: 3.3-fold growth a step)
+constexpr int kSumParts = 24, kSumThreads = 512;
+constexpr int kMeasure = 8;  // (a unit leaves 2^14 and serves 9 steps: 2.9-fold growth a step)
 static_assert(7 + 2 * kSumParts <= kSumWords, "words of a field");
 struct Sums {
     long long* w;  // [kSumWords][fields]
@@ -101,14 +101,16 @@ __device__ __forceinline__ void two_sum(f32x2& s, f32x2& e, f32x2 v) {
 }
 
 // Partial sums of u and of r^0, exact to 2^-48 of each thread's, and the
-// largest cell of r^0; kSumParts blocks a field; cells a multiple of 4.
-__global__ void __launch_bounds__(256) entry_sums_kernel(FieldMap src, long long cells, Sums s, float mdt, float kappa) {
-    const int f = blockIdx.x / kSumParts, part = blockIdx.x % kSumParts;
+// largest cell of r^0; parts blocks a field (the words of the others stay zero);
+// cells a multiple of 4.
+__global__ void __launch_bounds__(kSumThreads) entry_sums_kernel(FieldMap src, long long cells, Sums s, int parts, float mdt,
+                                                                  float kappa) {
+    const int f = blockIdx.x / parts, part = blockIdx.x % parts;
     const float4* u = reinterpret_cast<const float4*>(src.at(f, cells));
     const f32x2 m2 = f2(mdt, mdt), k2 = f2(kappa, kappa);
     f32x2 su = f2(0.f, 0.f), eu = su, sr = su, er = su;
     float top = 0.f;
-    for (long long i = part * 256LL + threadIdx.x; i < cells / 4; i += kSumParts * 256LL) {
+    for (long long i = part * (long long)kSumThreads + threadIdx.x; i < cells / 4; i += parts * kSumThreads) {
         const float4 q = u[i];
         const f32x2 v[2] = {f2(q.x, q.y), f2(q.z, q.w)};
 #pragma unroll
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(256) entry_sums_kernel(FieldMap src, long long
         return warp_sum((double(lo_of(a)) + double(lo_of(b))) + (double(hi_of(a)) + double(hi_of(b))));
     };
     const double tu = total(su, eu), tr = total(sr, er);
-    __shared__ double red[2][8];
+    __shared__ double red[2][kSumThreads / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     flush_max(s.top(0, f), top, lane);
     if (lane == 0) {
@@ -134,9 +136,18 @@ __global__ void __launch_bounds__(256) entry_sums_kernel(FieldMap src, long long
     if (threadIdx.x < 2) {
         double t = 0.0;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) t += red[threadIdx.x][w];
+        for (int w = 0; w < kSumThreads / 32; ++w) t += red[threadIdx.x][w];
         *s.part(threadIdx.x, part, f) = t;
     }
+}
+
+int entry_sums(const FieldMap& src, long long cells, const Sums& sums, const Coef<float, 2>& cf, cudaStream_t st) {
+    ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * kSumWords * sums.fields, st));
+    // four vectors a thread or more: 32^3 takes 4 blocks
+    const int parts = int(std::min<long long>(kSumParts, std::max<long long>(1, cells / (16 * kSumThreads))));
+    entry_sums_kernel<<<unsigned(sums.fields) * parts, kSumThreads, 0, st>>>(src, cells, sums, parts, cf.mdt, cf.kappa);
+    ACPR_LAUNCH_CHECK();
+    return AC_OK;
 }
 
 // ------------------------------------------------------------ 1024 x 1024 --
@@ -147,7 +158,7 @@ __global__ void __launch_bounds__(256) entry_sums_kernel(FieldMap src, long long
 // Fourier passes moved 16 bytes a cell and step.  The mass model needs the
 // field's sum each step and runs one step per launch.
 // Bound: FP32 issue.  us a step, 32 fields: two Fourier passes 213, tiles 34.5 (scalar
-// arithmetic on 7 columns a lane 48); mass-conserving 82 (one step a launch).
+// arithmetic on 7 columns a lane 48); mass-conserving 79 (one step a launch).
 constexpr int kTW = 8, kTH = 9, kTWarps = 16, kRim = 8, kTSteps = 4;
 constexpr int kTCols = 32 * kTW, kTRows = kTWarps * kTH;
 constexpr int kBig = 1024;
@@ -255,8 +266,8 @@ __global__ void __launch_bounds__(kTWarps * 32, 1) big_tile_kernel(FieldMap src,
 // the warps above and below.  A step reads and writes the fields once (the
 // five Fourier passes: 40 bytes a cell).  Bound: the latency of a plane
 // (loads, barrier, exchange), 4 TB/s of HBM traffic beside it.  us a step, mass / classic:
-// 16 fields of 128^3  Fourier passes 372, streamed 89 / 75 (2 rows a warp 107 / 65, 4 rows 121 / 102; handing on r
-// instead of u 103 / 93); 48 fields of 64^3 47 / 33.
+// 16 fields of 128^3  Fourier passes 372, streamed 86 / 75 (2 rows a warp 107 / 65, 4 rows 121 / 102; handing on r
+// instead of u 103 / 93); 48 fields of 64^3 42 / 33.
 constexpr int kCRows = 36, kCValid = kCRows - 4;
 constexpr int kCRoom = kGroupRoom - 5;  // of a cell of r, in groups of up to 32
 template <int N>
@@ -316,11 +327,10 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
     long long acc = 0;
     bool bad = false;
     float top = 0.f;
-    // the next step's r over four planes, rows in balanced trees (equal cells, a
+    // the next step's r over four planes (two of four rows), rows in balanced trees (equal cells, a
     // flat phase, add up exactly; one after another they all round alike, which
     // moved the mean by up to 4e-7 a call)
-    constexpr int G = kCH == 3 ? 2 : 1;
-    V part[2][G];
+    V part[2][2];
     auto add_group = [&](V p) {
         float t;
         if constexpr (Lane<W>::PAIR) t = lo_of(p) + hi_of(p);
@@ -368,23 +378,31 @@ __global__ void __launch_bounds__(CubeShape<N>::WARPS * 32, CubeShape<N>::MINB) 
 #pragma unroll
                     for (int c = 0; c < E; ++c) rn[c] = rhs(o[c], mdt, kappa);
                     rows[y] = E == 2 ? vadd(rn[0], rn[E - 1]) : rn[0];
-                    if (measures(n_step)) {
-                        float m[W];
-                        from_lane<W>(rn, m);
-#pragma unroll
-                        for (int c = 0; c < W; ++c) top = fmaxf(top, fabsf(m[c]));
-                    }
                 }
             }
             if constexpr (MASS) {
-                V g[2] = {vadd(rows[0], rows[1]), rows[2]};
-                if constexpr (kCH == 4) g[0] = vadd(g[0], vadd(rows[2], rows[kCH - 1]));
+                if constexpr (kCH == 3) {
+                    const V g[2] = {vadd(rows[0], rows[1]), rows[2]};
 #pragma unroll
-                for (int i = 0; i < G; ++i) {
-                    if ((k & 2) != 0) part[0][i] = buf ? vadd(part[0][i], g[i]) : g[i];  // (the first planes are k = 2, 3)
-                    else if (buf == 0) part[1][i] = g[i];
-                    else add_group(vadd(part[0][i], vadd(part[1][i], g[i])));
+                    for (int i = 0; i < 2; ++i) {
+                        if ((k & 2) != 0) part[0][i] = buf ? vadd(part[0][i], g[i]) : g[i];  // (the first planes are k = 2, 3)
+                        else if (buf == 0) part[1][i] = g[i];
+                        else add_group(vadd(part[0][i], vadd(part[1][i], g[i])));
+                    }
+                } else {
+                    const V g = vadd(vadd(rows[0], rows[1]), vadd(rows[2], rows[kCH - 1]));
+                    if (buf == 0) part[0][0] = g;
+                    else add_group(vadd(part[0][0], g));
                 }
+            }
+        }
+        if (MASS && measures(n_step)) {  // (of this step's r: the planes' ends part the instructions anyway)
+#pragma unroll
+            for (int y = 0; y < kCH; ++y) {
+                float m[W];
+                from_lane<W>(r[y], m);
+#pragma unroll
+                for (int c = 0; c < W; ++c) top = fmaxf(top, fabsf(m[c]));
             }
         }
         row_store<W>(edge[buf][0][0][warp], r[0], lane);
@@ -433,12 +451,11 @@ int cube_steps(const SolvePoly& poly, double a, double dt, int mass, int steps, 
     constexpr long long NNN = (long long)N * N * N;
     const Coef<float, 2> cf = make_coef<float, 2>(a, dt, double(NNN), poly);
     if (mass) {
-        ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * kSumWords * fields, st));
         FieldMap src{};
         src.base = const_cast<float*>(u_in);
         src.per_group = fields;
-        entry_sums_kernel<<<unsigned(fields) * kSumParts, 256, 0, st>>>(src, NNN, sums, cf.mdt, cf.kappa);
-        ACPR_LAUNCH_CHECK();
+        const int rc = entry_sums(src, NNN, sums, cf, st);
+        if (rc) return rc;
     }
     // the last step writes u_out, the ones before alternate with tmp; a first
     // step that writes u_out may not read cells there
@@ -479,16 +496,14 @@ int big_tiles_run(const SolvePoly& poly, double a, double dt, int mass, int fiel
     constexpr long long NN = (long long)kBig * kBig;
     const Coef<float, 2> cf = make_coef<float, 2>(a, dt, double(NN), poly);
     static DeviceSet configured;
-    const int rc = once_per_device(configured, [] {
+    int rc = once_per_device(configured, [] {
         const int r = allow_smem(big_tile_kernel<true>, kTileSmem);
         return r ? r : allow_smem(big_tile_kernel<false>, kTileSmem);
     });
     if (rc) return rc;
     Sums sums{sum_words, fields};
     if (mass) {
-        ACPR_CUDA(cudaMemsetAsync(sums.w, 0, sizeof(long long) * kSumWords * fields, st));
-        entry_sums_kernel<<<unsigned(fields) * kSumParts, 256, 0, st>>>(src, NN, sums, cf.mdt, cf.kappa);
-        ACPR_LAUNCH_CHECK();
+        if ((rc = entry_sums(src, NN, sums, cf, st))) return rc;
     }
     FieldMap buf{};
     buf.base = tmp;

@@ -3,6 +3,7 @@
     python -m paper_2510_07672_gb300.profile_cases fine     # ac_fine_propagate_slices, 512 x 256^2, 20 steps (stencil_reg_kernel)
     python -m paper_2510_07672_gb300.profile_cases fine_fft # the same by the Fourier solve (fine_field_kernel)
     python -m paper_2510_07672_gb300.profile_cases conv     # cnn_coarse_step, 16 x 256^2, 1-32x6-1 gelu bf16, mass shift
+    python -m paper_2510_07672_gb300.profile_cases conv64   # cnn_coarse_step, 1 x 1024^2, 1-64x8-1 gelu bf16
     python -m paper_2510_07672_gb300.profile_cases big      # ac_fine_propagate_slices, 16 x 1024^2, 4 steps (big_tile_kernel)
     python -m paper_2510_07672_gb300.profile_cases big_fft  # 2 steps too stiff for the tiles (big_rows_kernel, big_cols_kernel)
     python -m paper_2510_07672_gb300.profile_cases acnn     # acnn_forward (fused), 512 x 256^2, C = 4, 2 blocks
@@ -46,6 +47,12 @@ def main(case: str) -> None:
         net = G.CoarseNet(W.layers, W.channels, wt.astype(np.float32), bs.astype(np.float32), act=W.act,
                           precision=G.AC_F32, mass_fix=W.mass_fix)
         u = torch.tensor(W.ics(), dtype=torch.float32, device="cuda")
+        for _ in range(2):
+            G.cnn_coarse_step(net, u)
+    elif case == "conv64":
+        wt, bs = I.cnn_weights(8, 64, seed=0, sigma=0.05)
+        net = G.CoarseNet(8, 64, wt.astype(np.float32), bs.astype(np.float32), act=G.AC_ACT_GELU, precision=G.AC_F32)
+        u = torch.tensor(I.random_field(1024, seed=0)[None], dtype=torch.float32, device="cuda")
         for _ in range(2):
             G.cnn_coarse_step(net, u)
     elif case in ("big", "big_fft"):
