@@ -41,11 +41,9 @@ UNIT = "cell-steps/s"
 WL = I.MASS_F32_256
 
 
-def fine_flops_per_cell_step(n: int) -> float:
-    """Algorithmic flops of one fine step per grid cell: a forward and an
-    inverse real 2D FFT at 2.5 * M * log2(M) flops each (M = n^2), plus 10
-    pointwise flops (right-hand side and symbol divide)."""
-    return 5.0 * np.log2(n * n) + 10.0
+# Flops per cell and step of the degree-2 polynomial solve: 3 instructions (5
+# flops) for the right-hand side, 4 (5) and 5 (7) for its two stages.
+POLY2_FLOPS = 17.0
 
 
 def peak_fp32_tflops(sm_mhz: float) -> float:
@@ -433,15 +431,15 @@ def run_fine3d(args):
     cells = F * n ** 3 * steps
     peaks, src = measured_peaks()
     hbm = peaks.get("hbm_gbs", 6800.0)
-    pass_bytes = 40.0 * cells  # five passes: 80 bytes per complex cell pair and step
+    pass_bytes = 8.0 * cells  # one float32 read and write per cell and step
     print(json.dumps({
-        "metric": "3D fine propagation (periodic cube, 7-point Laplacian, FFT solve)",
+        "metric": "3D fine propagation (periodic cube, 7-point Laplacian)",
         "workload": "fine3d-mass-f32-128cube-16f-20steps", "ms_per_call": ms, "cell_steps_per_s": cells / (ms * 1e-3),
         "us_per_step": ms * 1e3 / steps, "gpu_launches_per_call": launches / args.steps,
         "roofline": {"bound": "hbm", "achieved": pass_bytes / (ms * 1e-3) / 1e9, "peak": hbm, "unit": "GB/s",
                      "frac": pass_bytes / (ms * 1e-3) / 1e9 / hbm,
-                     "traffic_model": "40 B per cell-step (5 passes, complex pairs); the one-read-one-write "
-                                      "minimum is 8 B", "peak_source": src},
+                     "traffic_model": "8 B per cell-step (one pass: one float32 read and write per cell)",
+                     "peak_source": src},
         "mass_drift": float((out.double().mean(dim=(1, 2, 3)) - u.double().mean(dim=(1, 2, 3))).abs().max().item()),
         "steps": args.steps, "warmup": args.warmup}), flush=True)
 
@@ -668,7 +666,7 @@ def run_large(args):
     U = pr.trajectory()[0]
     err_vs_seq = float(((U[-1].double() - seq_final[0].double()).norm() / seq_final[0].double().norm()).item())
     peaks, src = measured_peaks()
-    hbm = peaks.get("hbm_gbs", 6800.0)
+    fp32 = peak_fp32_tflops(peaks.get("sm_max_mhz", 2070.0))
     bf16 = peaks.get("bf16_tflops", 1900.0)
     cells_batch = s * c * n * n
     conv_fl = conv_flops_per_cell(W.layers, W.channels) * n * n
@@ -687,22 +685,21 @@ def run_large(args):
         "phase_ms": {"fine": st["fine_ms"], "coarse": st["coarse_ms"], "increment": st["increment_ms"]},
         "sequential_us_per_step": seq_ms * 1e3 / (s * c),
         "batched_fine": {"fields": s, "steps": c, "ms": batch_ms, "cell_steps_per_s": cells_batch / (batch_ms * 1e-3),
-                         "roofline": {"bound": "hbm", "achieved": 16.0 * cells_batch / (batch_ms * 1e-3) / 1e9,
-                                      "peak": hbm, "unit": "GB/s",
-                                      "frac": 16.0 * cells_batch / (batch_ms * 1e-3) / 1e9 / hbm,
-                                      "traffic_model": "16 B per cell-step (rows pass and columns pass, each "
-                                                       "one float32 read and write per cell)", "peak_source": src}},
+                         "roofline": {"bound": "alu", "kernel": "big_tile_kernel",
+                                      "achieved": POLY2_FLOPS * cells_batch / (batch_ms * 1e-3) / 1e12,
+                                      "peak": fp32, "unit": "TFLOP/s",
+                                      "frac": POLY2_FLOPS * cells_batch / (batch_ms * 1e-3) / 1e12 / fp32,
+                                      "flops_per_cell_step": POLY2_FLOPS, "peak_source": src}},
         "coarse_g": {"ms_per_application": g_ms, "tflops": conv_fl / (g_ms * 1e-3) / 1e12,
                      "frac_of_bf16_peak": conv_fl / (g_ms * 1e-3) / 1e12 / bf16},
         "cpu_baseline": cpu,
         "steps": 1, "warmup": 1}), flush=True)
 
 
-# DRAM bytes (read + write) the fine kernel moved per field-slice in one ncu
-# capture of the 256^2 launch shape (512 fields x 20 steps: 134.3 MB read,
-# 87.7 MB written); a slice is read once and written once whatever its step
+# DRAM bytes (read + write) stencil_reg_kernel moved per field-slice in one ncu
+# capture at 256^2 (512 fields x 20 steps: 134.3 MB read, 79.2 MB written); a slice is read once and written once whatever its step
 # count, so a launch's traffic scales with the field-slices it processes.
-FINE_DRAM_BYTES_PER_FIELD_SLICE_256 = (134.330112e6 + 87.662080e6) / 512
+FINE_DRAM_BYTES_PER_FIELD_SLICE_256 = (134.255616e6 + 79.208448e6) / 512
 
 
 def max_over_ranks(x: float, world: int, device) -> float:
@@ -938,9 +935,8 @@ def main():
     if rank == 0:
         peaks, src = measured_peaks()
         sm_mhz = peaks.get("sm_max_mhz", 2070.0)
-        # the polynomial solve of degree 2: 3 instructions (5 flops) for the right-hand
-        # side, 4 (5) and 5 (7) for its two stages
-        fpc = 17.0
+        assert 4.0 * WL.dt * (WL.eps * WL.n) ** 2 < 4.9e-3, "not a step of polynomial degree 2"
+        fpc = POLY2_FLOPS
         fine_tflops = st["fine_cell_steps"] * fpc / (st["fine_ms"] * 1e-3) / 1e12 if st["fine_ms"] else 0.0
         peak = peak_fp32_tflops(sm_mhz)
         conv_tflops = (st["coarse_cells"] * conv_flops_per_cell(WL.layers, WL.channels) /
@@ -966,16 +962,9 @@ def main():
             "conv_tflops": conv_tflops,
             "roofline": {"bound": "alu", "kernel": "stencil_reg_kernel", "achieved": fine_tflops,
                          "peak": peak, "unit": "TFLOP/s", "frac": fine_tflops / peak,
-                         # the counters were taken on the asynchronous-exchange launch shape (2 CTAs
-                         # per SM); the default shape has changed since (no exchange buffer, 3 CTAs per
-                         # SM) and was not captured again
-                         "traffic": None,
-                         "traffic_earlier_shape": fine_traffic_per_launch(st, WL, steps),
-                         "traffic_unit": "bytes per launch (ncu DRAM bytes per field-slice x field-slices per launch)",
-                         "traffic_note": "null: the DRAM counters (433.6 KB per field-slice, 512 KB algorithmic) "
-                                         "are of the asynchronous-exchange launch shape, not of the current "
-                                         "default (no exchange buffer, 3 CTAs per SM); traffic_earlier_shape "
-                                         "scales them to this run's launches",
+                         "traffic": fine_traffic_per_launch(st, WL, steps),
+                         "traffic_unit": "bytes per launch (ncu DRAM bytes per field-slice, 417 KB of the 512 KB "
+                                         "read and written, x field-slices per launch)",
                          "peak_source": f"FP32 lanes x 2 x sm_max_mhz {sm_mhz:.0f} from {src} peaks",
                          "flops_per_cell_step": fpc},
             "cpu_baseline": cpu,

@@ -100,15 +100,24 @@ const char* ac_last_error(void);
 
 /* 1 if the fine-step kernels are built for this (n, precision), else 0:
  * n = 8 .. 512 (float32) and 8 .. 256 (float64) on one thread-block cluster
- * per field; n = 1024 float32 through two passes per step over L2/HBM (fine
- * step and slice propagation only, not the adjoint or trajectory modes). */
+ * per field; n = 1024 float32 on tiles or passes over L2/HBM (fine step and
+ * slice propagation only, not the adjoint or trajectory modes).
+ *
+ * The solve of a step.  With lambda = 4 dt eps^2 / h^2 the inverse of
+ * (1 + S dt) I - dt eps^2 Lap_h is applied as a polynomial in the neighbour sum,
+ * exact to a rounding, where the step allows one: n >= 32, 1 + S dt <= 2, and at
+ * 1 + S dt = 1 lambda up to about 5.7e-2 (float32, n <= 256), 2.2e-2 (512),
+ * 4.9e-3 (1024), 3.3e-3 (the cube), 9.6e-3 (float64, n <= 256).  Other steps are
+ * solved by FFT, at several times the cost; both are the same step to round-off. */
 int ac_fine_supported(int n, int precision);
 
-/* Launch shapes of the fine kernel built for (n, precision) -- cluster size,
- * threads per CTA, occupancy target -- and the one in use.  Every shape
- * computes the same steps; they differ in how the field is split over CTAs
- * and so in which rows share a complex line, which moves results by
- * round-off.  Each shape is a deterministic function of its input; do not
+/* Launch shapes of the fine kernel built for (n, precision) -- the polynomial
+ * solve ("stencil", where n >= 32; a step it is not built for takes the next
+ * shape), and the FFT's cluster sizes, threads per CTA and occupancy targets --
+ * and the one in use (0 unless set).  Indices belong to a build of the library;
+ * names identify a shape.  Every shape computes the same steps; they differ in
+ * the solve, in how the field is split over CTAs and so in which rows share a
+ * complex line, which moves results by round-off.  Each shape is a deterministic function of its input; do not
  * change the shape in the middle of a Parareal solve.  ac_fine_autotune runs each shape on the caller's problem
  * (u_in -> u_out, num_fields fields, `steps` steps; twice after a warm-up),
  * writes the mean time per call in ms to ms_out[i] (may be NULL; room for
@@ -146,10 +155,16 @@ int ac_cn_propagate_slices(const ac_params* params, int num_fields, int steps, c
 /* The fine propagator F(t_n, t_{n+1}, U_n) of Eq. (fine_operator): for every
  * one of `num_fields` independent fields, `steps_per_slice` fine steps
  * (Algorithm 2: the parallel fine solves of all slices).  The field stays on
- * chip for all steps (n <= 512; at n = 1024 each step is two passes through
- * L2/HBM); HBM is touched once on entry and once on exit.  In the
- * mass-conserving variant the spectrum's mean mode is held at the field's
- * float64 mean taken on entry, so mass is conserved to rounding.
+ * chip for all steps (n <= 512; at n = 1024 the field goes through L2/HBM every
+ * four steps, every step in the mass-conserving variant and twice a step when
+ * solved by FFT); HBM is touched once on entry and once on exit.  In the
+ * mass-conserving variant the mean is held at the field's mean taken on entry,
+ * so mass is conserved to rounding: the FFT holds the spectrum's mean mode at the
+ * float64 mean, the polynomial solve shifts every step by exact fixed-point sums
+ * whose unit follows the largest cell.  A field that outgrows its unit (2^18-fold
+ * within up to 128 steps for float32, fewer for larger dt; 2^14-fold within 9
+ * steps at n = 1024; 2^19-fold in one step for float64), which only a blow-up
+ * does, comes out as NaN, as does one that holds an infinity or a NaN.
  * u_starts, u_ends: device [num_fields][n][n]; they may not overlap. */
 int ac_fine_propagate_slices(const ac_params* params, int num_fields, int steps_per_slice,
                              const void* u_starts, void* u_ends, acpr_stream stream);
@@ -164,7 +179,7 @@ int ac_fine_propagate_work(const ac_params* params, int count, const void* work,
                            void* u_out, acpr_stream stream);
 
 /* ac_fine_propagate_slices with a caller-owned workspace: at n = 1024 the
- * two-pass path keeps each field's half spectra between passes in
+ * intermediate fields and sums, or the half spectra of the FFT's passes, are in
  * `workspace` (device, 256-byte aligned, at least
  * ac_fine_workspace_bytes(n, num_fields, precision) bytes) and the call
  * allocates nothing.  Without a workspace (ac_fine_propagate_slices) the
@@ -203,7 +218,9 @@ int ac_energy(const ac_params* params, int num_fields, const void* u, double* en
 /* dE_h/du = h^2 (-eps^2 Lap_h u - f(u)) for each field (device, params precision). */
 int ac_energy_grad(const ac_params* params, int num_fields, const void* u, void* grad, acpr_stream stream);
 
-/* Bytes of the workspace ac_energy_gradient_ic needs. */
+/* Bytes of the workspace of ac_energy_gradient_ic: the checkpoints and the states
+ * of two segments, one of which is recomputed while the adjoint runs through the
+ * other.  checkpoint_every + 1 fields less also do, without that overlap. */
 size_t ac_energy_gradient_workspace(const ac_params* params, int steps, int checkpoint_every);
 
 /* Gradient of E_h(u^steps) with respect to the initial field u0 (one field,
@@ -361,10 +378,13 @@ int mse_loss_grad(const float* pred, const float* target, long long count, doubl
  * The fine step on the periodic cube (d = 3; the 3D experiments of Sec. 4):
  * the stabilised semi-implicit step of ac_params with the periodic 7-point
  * Laplacian (symbol -(4/h^2)(sin^2(pi a/N) + sin^2(pi b/N) + sin^2(pi c/N))),
- * solved by a 3D FFT in five passes over L2/HBM per step.  Fields are
- * [num_fields][n][n][n] row-major (last index fastest), params->n = n per
- * side.  The mass-conserving variant holds the zero mode at the field's
- * mean taken when the call starts (the scheme conserves it exactly).
+ * solved by the polynomial in the 7-point neighbour sum in one pass over the
+ * field per step (float32, 16-byte aligned pointers, lambda up to 3.3e-3: see
+ * ac_fine_supported), else by a 3D FFT in five passes over L2/HBM per step.
+ * Fields are [num_fields][n][n][n] row-major (last index fastest), params->n = n
+ * per side.  The mass-conserving variant holds the field's mean taken when the
+ * call starts (the scheme conserves it exactly), as ac_fine_propagate_slices
+ * does at n = 1024.
  * ------------------------------------------------------------------------ */
 
 /* 1 if the 3D step is built for (n, precision): n = 32, 64 or 128. */
@@ -375,7 +395,7 @@ int ac_fine3d_supported(int n, int precision);
 size_t ac_fine3d_work_bytes(int n, int num_fields, int precision);
 
 /* `steps` fine steps of every field: u_out = F^steps(u_in).  u_in may equal
- * u_out.  work: ac_fine3d_work_bytes() bytes of device memory.  Asynchronous
+ * or overlap u_out.  work: ac_fine3d_work_bytes() bytes of device memory.  Asynchronous
  * on `stream`. */
 int ac_fine3d_propagate(const ac_params* params, int steps, int num_fields, const void* u_in, void* u_out,
                         void* work, size_t work_bytes, acpr_stream stream);

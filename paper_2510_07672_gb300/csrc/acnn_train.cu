@@ -321,8 +321,9 @@ __global__ void __launch_bounds__(128) wgrad_finish_kernel(const double* __restr
 // adjacent pixels: it loads their 6 x 3 window once (18 vector loads for 4
 // pixels, not 36) and each tap's weights serve all four; channels go in pairs
 // through the paired instructions.  Same order of every sum as the kernels
-// above.  Bound: FP32 issue.  16 fields of 256^2: convolution 28 -> 10 us,
-// input gradient 45 -> 13 us, weight gradient 38 -> 13 us.
+// above.  Bound: the latency of the window's loads (issue 28 to 40%).  16 fields
+// of 256^2, operands in L2, C -> C: convolution 28 -> 12 us, input gradient
+// 45 -> 13 us, weight gradient 38 -> 34 us (1 -> C and C -> 1: 13 us).
 constexpr int kRowsPx = 4;
 
 struct StripPos {  // this thread's field, column and first row
@@ -515,9 +516,11 @@ __global__ void __launch_bounds__(kThreads) strip_dgrad_kernel(const float* __re
 }
 
 // Weight-gradient partials: a thread walks 16 rows of its column with the 3 x 3
-// window sliding (3 new vector loads a row), all COUT CIN 9 + COUT sums in
+// window sliding (3 new vector loads a row), its COUT CIN 9 + COUT sums in
 // registers; a warp's sums are folded by exchanging halves (each of the five
-// exchanges halves the values a lane holds), the warps' in order.
+// exchanges halves the values a lane holds; the values are indexed by a half
+// that is a loop variable and so pass through local memory, 640 bytes a thread
+// for C -> C, 256 for the ends), the warps' in order.
 constexpr int kWsRows = 16, kWsThreads = 128;
 
 template <int CIN, int COUT>

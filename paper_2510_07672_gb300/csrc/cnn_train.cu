@@ -14,14 +14,17 @@
 // every accumulation is float32; weight gradients are reduced over pixel
 // chunks in a fixed order (deterministic).  Hidden-layer dgrads run on the
 // tensor cores through the forward kernel with channel-transposed, tap-flipped
-// weights; the first and last layers and the weight gradients on CUDA cores.
+// weights, the hidden weight gradients for C = 64 and n a multiple of 128 through
+// cnn_wgrad_tc.cu; the first and last layers and the other weight gradients run
+// on CUDA cores.
 //
 // Workspace (cnn_train_bytes), in this order:
 //   A_l, l = 1..L-1   bf16 [B][C/8][n][n][8]     inputs of layers 1..L-1
 //   Z_l, l = 0..L-2   f32  [B][C/8][n][n][8]     pre-activations of layers 0..L-2
 //   dZ ping-pong      2 x bf16 [B][C/8][n][n][8]
 //   Wt                bf16 (L-2) x 9*C*C          transposed, flipped hidden weights
-//   partials          f32  kChunks x 9 x (C*C + C)  weight / bias gradient partials
+//   partials          f32  chunks x 9 x (C*C + C)  weight / bias gradient partials
+//                          (kTcChunks for C = 64, kChunks otherwise)
 //   g centred         f32  [B][n][n]               (mass shift only)
 //   z partials        f64  block sums of the last layer (mass shift only)
 #include <cuda_bf16.h>
@@ -31,7 +34,7 @@
 namespace acpr {
 
 constexpr int kChunks = 64;      // pixel chunks of the weight-gradient reduction
-constexpr int kTcChunks = 152;   // of the tensor-core kernel: one CTA per SM
+constexpr int kTcChunks = 152;   // for C = 64: one CTA of the tensor-core kernel per SM
 constexpr int kWgThreads = 256;
 
 __device__ __forceinline__ int wrapi(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
@@ -210,11 +213,10 @@ __global__ void first_dgrad_kernel(const float* __restrict__ g, const __nv_bfloa
     du[pix] = g[pix] + acc;
 }
 
-// Weight and bias gradient partials of one layer, one (tap, chunk) per block:
+// Weight and bias gradient partials of a hidden layer, one (tap, chunk) per block:
 //   part[chunk][tap][o][c] = sum_{pixels q of the chunk} dz[o][q] * a[c][q + off(tap)]
 //   part[chunk][tap][C*C + o] = sum dz[o][q]  (tap 0 blocks only)
-// a: bf16 chunked activations, or (CIN == 1) the float32 field rounded to bf16.
-// dz: bf16 chunked, or (COUT == 1) the float32 output gradient rounded to bf16.
+// a, dz: bf16 chunked activations and pre-activation gradients.
 // Block rows of 64 pixels are staged in shared memory; thread (o, c-group)
 // accumulates a strip of input channels.
 // Each thread owns a TO x TC block of (output, input) channel pairs and, per
@@ -248,8 +250,7 @@ wgrad_kernel(const void* __restrict__ a_src, const void* __restrict__ dz_src, fl
     constexpr int TO = WgTile<PER>::TO, TC = WgTile<PER>::TC;
     constexpr int NCB = CIN / TC;                // input-channel blocks
     constexpr int NTH = (COUT / TO) * NCB;       // threads that own pairs
-    constexpr int PA = CIN >= 4 ? CIN + 4 : CIN + 1;    // row pitches (16-byte rows for vector loads)
-    constexpr int PD = COUT >= 4 ? COUT + 4 : COUT + 1;
+    constexpr int PA = CIN + 4, PD = COUT + 4;   // row pitches (16-byte rows for vector loads)
     __shared__ __align__(16) float s_a[TP][PA];
     __shared__ __align__(16) float s_dz[TP][PD];
     const int tap = blockIdx.x % 9;
@@ -279,12 +280,8 @@ wgrad_kernel(const void* __restrict__ a_src, const void* __restrict__ dz_src, fl
                 const int b = int(p >> (2 * lg));
                 const int y = wrapi((int(p >> lg) & (n - 1)) + dy, n), x = wrapi((int(p) & (n - 1)) + dx, n);
                 const long long q = (long long)y * n + x;
-                if constexpr (CIN == 1) {
-                    v = bf16r(static_cast<const float*>(a_src)[(long long)b * nn + q]);
-                } else {
-                    v = __bfloat162float(static_cast<const __nv_bfloat16*>(a_src)[
-                        (((long long)b * (CIN / 8) + c / 8) * nn + q) * 8 + c % 8]);
-                }
+                v = __bfloat162float(static_cast<const __nv_bfloat16*>(a_src)[
+                    (((long long)b * (CIN / 8) + c / 8) * nn + q) * 8 + c % 8]);
             }
             s_a[pi][c] = v;
         }
@@ -295,12 +292,8 @@ wgrad_kernel(const void* __restrict__ a_src, const void* __restrict__ dz_src, fl
             if (p < p1) {
                 const int b = int(p >> (2 * lg));
                 const long long q = p & (nn - 1);
-                if constexpr (COUT == 1) {
-                    v = bf16r(static_cast<const float*>(dz_src)[(long long)b * nn + q]);
-                } else {
-                    v = __bfloat162float(static_cast<const __nv_bfloat16*>(dz_src)[
-                        (((long long)b * (COUT / 8) + o / 8) * nn + q) * 8 + o % 8]);
-                }
+                v = __bfloat162float(static_cast<const __nv_bfloat16*>(dz_src)[
+                    (((long long)b * (COUT / 8) + o / 8) * nn + q) * 8 + o % 8]);
             }
             s_dz[pi][o] = v;
         }

@@ -1,5 +1,7 @@
 // fine.cu -- the fine propagator F: stabilised semi-implicit Allen-Cahn steps
-// on a periodic n x n grid, many independent fields at once.
+// on a periodic n x n grid, many independent fields at once, and the choice of
+// the launch shape.  The kernel here solves by FFT; steps whose solve is a
+// polynomial of a built degree run in fine_stencil.cu.
 //
 // One step (Sec. 3.1 fine operator, the stabilised linear scheme):
 //   r      = (1 + S dt) u + dt f(u),                f(u) = u - u^3
@@ -547,13 +549,14 @@ static const FineVariant* fine_variants(int n, int* count) {
         static const FineVariant v128[] = {ACPR_POLY, ACPR_FV(T, 128, 2, 16, 8, 2), ACPR_FV(T, 128, 4, 16, 8, 3),
                                            ACPR_FV(T, 128, 1, 16, 8, 1), ACPR_FVA(T, 128, 4, 16, 8, 3),
                                            ACPR_FVA(T, 128, 2, 16, 8, 2)};
-        // entry 0 (clusters of 8, asynchronous exchange, no separate exchange
-        // buffer, 3 CTAs per SM) measured fastest on large batches (512 fields,
-        // 20 steps: 2.46 ms; with the exchange buffer 2.56 ms; cluster
-        // barriers 2.97 ms).  16-CTA clusters are 10% faster on 16 fields, but a
-        // shape change alters the rounding, and F must stay one function within
-        // a solve and between a Parareal solve and its sequential reference
-        // (exactness at k = s): the default does not depend on the batch size.
+        // The first Fourier shape (clusters of 8, asynchronous exchange, no
+        // separate exchange buffer, 3 CTAs per SM) measured fastest on large
+        // batches (512 fields, 20 steps: 2.46 ms; with the exchange buffer
+        // 2.56 ms; cluster barriers 2.97 ms; the polynomial solve 0.40 ms).  16-CTA
+        // clusters are 10% faster on 16 fields, but a shape change alters the
+        // rounding, and F must stay one function within a solve and between a
+        // Parareal solve and its sequential reference (exactness at k = s): the
+        // default does not depend on the batch size.
         static const FineVariant v256[] = {ACPR_POLY, ACPR_FVN(T, 256, 8, 16, 16, 3), ACPR_FVA(T, 256, 8, 16, 16, 2),
                                            ACPR_FVA(T, 256, 16, 16, 16, 3), ACPR_FVA(T, 256, 4, 16, 16, 1),
                                            ACPR_FV(T, 256, 8, 16, 16, 2), ACPR_FV(T, 256, 4, 16, 16, 1),

@@ -1,5 +1,5 @@
 // fine.cuh -- launch arguments shared by the fine-step kernels of fine.cu
-// (Fourier solve) and fine_stencil.cu (polynomial solve).
+// (Fourier solve) and fine_stencil.cu (polynomial solve), and the polynomial.
 #pragma once
 
 #include "common.cuh"

@@ -29,8 +29,9 @@
 // only a field that outgrows its unit (float32: 2^18-fold in two runs of steps,
 // see Coef::run, float64: 2^19-fold in one step; a blow-up) becomes not a number.
 //
-// Bound: FP32 (float64: FP64) issue.  Measured, Fourier kernel -> this one:
-//   512 fields of 256^2, mass, 100 steps        11.40 -> 1.98 ms (2.21 with scalar instructions and 8x8x4)
+// Bound: FP32 (float64: FP64) issue and the step's barrier (512 fields of 256^2:
+// FP32 pipe 62% busy, half of the issue slots).  Measured, Fourier kernel -> this one:
+//   512 fields of 256^2, mass, 100 steps        11.40 -> 1.95 ms (2.21 with scalar instructions and 8x8x4)
 //   21 fields of 512^2, 50 to 90 steps           3.01 -> 0.25 ms (0.37)
 //   float64 256^2, 300 steps, their recomputation and adjoint  138 -> 22.5 ms (32.3 one after the other)
 //   one step of one 128^2 field (call included)  16.4 -> 9.6 us
@@ -453,7 +454,8 @@ int launch_reg(const FineArgs& args, const SolvePoly& poly, cudaStream_t st) {
 }
 
 // The split (rows a warp, warps a CTA, CTAs a field, CTAs per SM) by size and
-// batch.  40 steps, us, mass-conserving / classic, measured for each line:
+// batch.  40 steps, us, mass-conserving / classic, measured for each line (the
+// mass-conserving ones within 10% of the present sums'):
 //   256: 4x4x16  1 field 60/36, 8 70/45; 8x4x8 (1 CTA per SM's registers)  8 fields 62/42, 24 87/67;
 //        8x4x8 (4 CTAs)  38 fields 106/83, 512 825/650; 8x8x4 512 fields 923/645, 8x16x2 999/703
 //   512: 8x4x16  1 field 105/70, 21 216/164, 64 599/504; 4x8x16  112/72, 317/206, 1033/677
