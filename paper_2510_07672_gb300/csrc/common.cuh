@@ -8,7 +8,7 @@
 #include <string>
 
 #include "../../include/acpr.h"
-#include "per_device.h"
+#include "per_device.cuh"
 
 namespace acpr {
 

@@ -55,7 +55,9 @@ SolvePoly solve_poly(double a, double lam_scale, int dims, int precision, int mi
     // rounding in float32, two in float64.  Against a long double
     // solve, 300 steps at 128^2 (lambda = 1.25e-3): degree 4 6e-14, degree 5
     // 2.6e-14, a float64 Fourier solve 5e-14; at 64^2 (1e-3), 400 steps:
-    // degree 4 2.8e-14, Fourier 6e-14.
+    // degree 4 2.8e-14, Fourier 6e-14.  Against a float64 Fourier solve, whose
+    // own rounding another Fourier solve shares in part: a Parareal solve at
+    // 64^2 (1e-3, degree 4) 1.0e-13, the Fourier kernel 8.2e-14.
     const double tol = precision == AC_F64 ? 0x1p-52 : 0x1p-24;
     int M = std::max(1, min_degree);
     while (M <= max_degree && 4.0 * std::pow(rho, M + 1) > tol) ++M;

@@ -1,4 +1,4 @@
-// per_device.h -- host state that belongs to a CUDA device.
+// per_device.cuh -- host state that belongs to a CUDA device.
 #pragma once
 
 #include <atomic>

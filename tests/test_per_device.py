@@ -12,7 +12,7 @@ MAIN = r"""
 #include <cstdio>
 #include <thread>
 #include <vector>
-#include "per_device.h"
+#include "per_device.cuh"
 int main() {
     acpr::DeviceSet s;
     if (s.has(0) || s.has(1)) return 1;
